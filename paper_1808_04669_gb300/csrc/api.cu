@@ -14,6 +14,7 @@
 #include "../../include/dgdf.h"
 #include "device.cuh"
 #include "kcommon.cuh"
+#include "ml_device.hpp"
 #include "multilevel.hpp"
 #include "setup.hpp"
 
@@ -643,61 +644,36 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
     std::string merr;
     if ((rc = dgdf::build_multilevel(M->hm, mlh, merr))) return cleanup(fail(rc, merr));
     // the V-cycle's precision: FP32 in the mixed form (a preconditioner needs no more; the PCG
-    // vectors and S stay FP64), FP64 in the FP64 form
+    // vectors and S stay FP64), FP64 in the FP64 form. The dense level may take in more rows in
+    // FP32: 2048^2 words are 16 MB, two microseconds from L2, while in FP64 1024^2 multiply-adds
+    // already take 1.7 us of the FP64 pipes.
     const bool ml32 = p.precision == DG_PRECISION_MIXED;
-    auto f32 = [](const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); };
-    auto fill = [&](auto& lv, auto conv, auto* cpinv_out, auto** xc, auto** bc) -> int {
-      for (size_t l = 0; l < mlh.lv.size(); ++l) {
-        const dgdf::MLHostLevel& H = mlh.lv[l];
-        auto& L = lv[l];
-        using T = std::remove_pointer_t<decltype(L.x)>;
-        L.stencil = H.stencil ? 1 : 0;
-        L.bs = H.bs;
-        L.n = H.n;
-        L.inject = H.inject ? 1 : 0;
-        L.n_next = H.n_next;
-        L.bs_next = H.bs_next;
-        L.c0 = T(H.cheb[0]);
-        L.c1 = T(H.cheb[1]);
-        L.c2 = T(H.cheb[2]);
-        int rc2 = 0;
-        if ((rc2 = upload(M, &L.binv, conv(H.binv)))) return rc2;
-        if (!H.stencil && ((rc2 = upload(M, &L.a_rp, H.A.rp)) || (rc2 = upload(M, &L.a_ci, H.A.ci)) ||
-                           (rc2 = upload(M, &L.a_v, conv(H.A.v)))))
-          return rc2;
-        if (!H.inject && ((rc2 = upload(M, &L.p_rp, H.P.rp)) || (rc2 = upload(M, &L.p_ci, H.P.ci)) ||
-                          (rc2 = upload(M, &L.p_v, conv(H.P.v))) || (rc2 = upload(M, &L.r_rp, H.R.rp)) ||
-                          (rc2 = upload(M, &L.r_ci, H.R.ci)) || (rc2 = upload(M, &L.r_v, conv(H.R.v)))))
-          return rc2;
-        const size_t nv = size_t(H.n) * H.bs;
-        if constexpr (std::is_same<T, double>::value) {
-          if (l == 0) {   // level 0 works on the PCG vectors: b = r, x = z
-            L.b = d.r;
-            L.x = d.z;
-          }
-        }
-        if (!L.b && ((rc2 = dalloc(M, &L.b, nv)) || (rc2 = dalloc(M, &L.x, nv)))) return rc2;
-        if ((rc2 = dalloc(M, &L.r, nv)) || (rc2 = dalloc(M, &L.d, nv))) return rc2;
-      }
-      int rc2 = 0;
-      if ((rc2 = upload(M, cpinv_out, conv(mlh.cpinv))) || (rc2 = dalloc(M, xc, size_t(mlh.nc))) ||
-          (rc2 = dalloc(M, bc, size_t(mlh.nc))))
-        return rc2;
-      return 0;
+    dgdf::fuse_levels(mlh, ml32 ? 4 : 8, ml32 ? 2048 : 1024, dgdf::ml_grid_threads());
+    auto up = [&](auto** out, const auto& v) { return upload(M, out, v); };
+    auto al = [&](auto** out, size_t n) {
+      int rc2 = dalloc(M, out, n);
+      if (!rc2 && cudaMemsetAsync(*out, 0, n * sizeof(**out), M->stream) != cudaSuccess)
+        rc2 = fail(DG_ERR_CUDA, "multilevel: clearing a vector failed");
+      return rc2;
     };
+    const bool tables = dgdf::ml_class_tables_fit(hm.nl, 5, ml32, hm.n_stencil);
+    auto table = [&](int word) {
+      return dgdf::ml_operator_table(tables, hm.nl, 5, hm.n_stencil, d.n_facet, hm.facet_stencil.data(),
+                                     hm.stencil_blocks.data(), word);
+    };
+    d.ml_ncls = tables ? hm.n_stencil : 0;
+    if ((rc = upload(M, &d.ml_tab, table(8)))) return cleanup(rc);
     if (ml32) {
-      std::vector<dgdf::MLLevelT<float>> lv(mlh.lv.size());
-      if ((rc = fill(lv, f32, &d.ml_cpinv_f, &d.ml_xc_f, &d.ml_bc_f))) return cleanup(rc);
-      const dgdf::MLLevelT<float>* lvd = nullptr;
-      if ((rc = upload(M, &lvd, lv))) return cleanup(rc);
-      d.ml_lv_f = lvd;
-    } else {
-      std::vector<dgdf::MLLevelDev> lv(mlh.lv.size());
-      if ((rc = fill(lv, [](const std::vector<double>& v) { return v; }, &d.ml_cpinv, &d.ml_xc, &d.ml_bc)))
+      std::vector<dgdf::MLLevelT<float>> lv;
+      if ((rc = upload(M, &d.ml_tab_f, to_float(table(4)))) ||
+          (rc = dgdf::ml_fill<float>(mlh, lv, up, al, d.r, d.z, &d.ml_cpinv_f, &d.ml_xc_f, &d.ml_bc_f, &d.ml_ld)) ||
+          (rc = upload(M, &d.ml_lv_f, lv)))
         return cleanup(rc);
-      const dgdf::MLLevelDev* lvd = nullptr;
-      if ((rc = upload(M, &lvd, lv))) return cleanup(rc);
-      d.ml_lv = lvd;
+    } else {
+      std::vector<dgdf::MLLevelDev> lv;
+      if ((rc = dgdf::ml_fill<double>(mlh, lv, up, al, d.r, d.z, &d.ml_cpinv, &d.ml_xc, &d.ml_bc, &d.ml_ld)) ||
+          (rc = upload(M, &d.ml_lv, lv)))
+        return cleanup(rc);
     }
     d.ml_nlev = int(mlh.lv.size());
     d.ml_nc = mlh.nc;

@@ -9,6 +9,7 @@
 #include "../../include/dgdf.h"
 #include "../../include/dgdf3.h"
 #include "device3.cuh"
+#include "ml_device.hpp"
 #include "multilevel.hpp"
 #include "setup3.hpp"
 
@@ -247,48 +248,28 @@ int dg3_mesh_create(int64_t n_tet, const int64_t* tet_vertex_ids, const double* 
     // the V-cycle runs in FP32 (a preconditioner needs no more; the PCG vectors and S stay FP64):
     // level operators, transfers, Chebyshev coefficients and the coarsest pseudo-inverse rounded
     // once; level 0 has vectors of its own, filled from r and written back to z
-    auto f32 = [](const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); };
-    std::vector<dgdf::MLLevelT<float>> lv(mlh.lv.size());
-    const float* blk32 = nullptr;
-    if ((rc = upload3(M, &blk32, f32(hm.stencil_blocks)))) return cleanup(rc);
-    for (size_t l = 0; l < mlh.lv.size(); ++l) {
-      const dgdf::MLHostLevel& H = mlh.lv[l];
-      dgdf::MLLevelT<float>& L = lv[l];
-      L.stencil = H.stencil ? 1 : 0;
-      L.bs = H.bs;
-      L.n = H.n;
-      L.inject = H.inject ? 1 : 0;
-      L.n_next = H.n_next;
-      L.bs_next = H.bs_next;
-      L.modes = 1;
-      L.c0 = float(H.cheb[0]);
-      L.c1 = float(H.cheb[1]);
-      L.c2 = float(H.cheb[2]);
-      if ((rc = upload3(M, &L.binv, f32(H.binv)))) return cleanup(rc);
-      if (H.stencil) {   // level 0: block Jacobi on the seven-block face stencil
-        L.st_cls = d.face_stencil;
-        L.st_nbr = d.face_nbr;
-        L.st_nnb = 6;
-        L.st_blk = blk32;
-      } else if ((rc = upload3(M, &L.a_rp, H.A.rp)) || (rc = upload3(M, &L.a_ci, H.A.ci)) ||
-                 (rc = upload3(M, &L.a_v, f32(H.A.v)))) {
-        return cleanup(rc);
-      }
-      if (!H.inject && ((rc = upload3(M, &L.p_rp, H.P.rp)) || (rc = upload3(M, &L.p_ci, H.P.ci)) ||
-                        (rc = upload3(M, &L.p_v, f32(H.P.v))) || (rc = upload3(M, &L.r_rp, H.R.rp)) ||
-                        (rc = upload3(M, &L.r_ci, H.R.ci)) || (rc = upload3(M, &L.r_v, f32(H.R.v)))))
-        return cleanup(rc);
-      const size_t nv = size_t(H.n) * H.bs;
-      if ((rc = dalloc3(M, &L.b, nv)) || (rc = dalloc3(M, &L.x, nv)) || (rc = dalloc3(M, &L.r, nv)) ||
-          (rc = dalloc3(M, &L.d, nv)))
-        return cleanup(rc);
-    }
+    dgdf::fuse_levels(mlh, 4, 2048, dgdf::ml_grid_threads());
+    auto up = [&](auto** out, const auto& w) { return upload3(M, out, w); };
+    auto al = [&](auto** out, size_t n) {
+      int rc2 = dalloc3(M, out, n);
+      if (!rc2 && cudaMemsetAsync(*out, 0, n * sizeof(**out), M->stream) != cudaSuccess)
+        rc2 = api_fail(DG_ERR_CUDA, "multilevel: clearing a vector failed");
+      return rc2;
+    };
     dgdf::DevMesh& v = M->mv;
-    const dgdf::MLLevelT<float>* lvd = nullptr;
-    if ((rc = upload3(M, &lvd, lv)) || (rc = upload3(M, &v.ml_cpinv_f, f32(mlh.cpinv))) ||
-        (rc = dalloc3(M, &v.ml_xc_f, size_t(mlh.nc))) || (rc = dalloc3(M, &v.ml_bc_f, size_t(mlh.nc))))
+    const bool tables = dgdf::ml_class_tables_fit(hm.nl, 7, true, d.n_stencil);
+    auto table = [&](int word) {
+      return dgdf::ml_operator_table(tables, hm.nl, 7, d.n_stencil, d.n_face, hm.face_stencil.data(),
+                                     hm.stencil_blocks.data(), word);
+    };
+    const std::vector<double> tab4 = table(4);
+    std::vector<dgdf::MLLevelT<float>> lv;
+    v.ml_ncls = tables ? d.n_stencil : 0;
+    if ((rc = upload3(M, &v.ml_tab, table(8))) ||
+        (rc = upload3(M, &v.ml_tab_f, std::vector<float>(tab4.begin(), tab4.end()))) ||
+        (rc = dgdf::ml_fill<float>(mlh, lv, up, al, d.r, d.z, &v.ml_cpinv_f, &v.ml_xc_f, &v.ml_bc_f, &v.ml_ld)) ||
+        (rc = upload3(M, &v.ml_lv_f, lv)))
       return cleanup(rc);
-    v.ml_lv_f = lvd;
     v.ml_nlev = int(lv.size());
     v.ml_nc = mlh.nc;
     v.k = d.k;
@@ -299,7 +280,8 @@ int dg3_mesh_create(int64_t n_tet, const int64_t* tet_vertex_ids, const double* 
     v.bar = d.bar;
     v.stats = d.stats;
     M->use_ml = true;
-    M->ml_blocks = dgdf::solver3_ml_blocks(d, true);
+    M->ml_blocks = dgdf::solver3_ml_blocks(d, M->mv);
+    if (M->ml_blocks < 1) return cleanup(api_fail(DG_ERR_CUDA, "multilevel solver does not fit"));
   }
   *out = M;
   return DG_OK;

@@ -50,12 +50,10 @@ struct GridBar {
 template <typename R>
 struct MLLevelT {
   int stencil;        // 1: the facet stencil of S on the first bs modes; 0: the CSR matrix a_*
-  int bs, n;          // values per row, rows
+  int bs, n;          // values per row (FP32 rows of three are padded to four), rows
   int inject;         // 1: transfer to the next level keeps the leading bs_next modes (same facet rows)
   int n_next, bs_next;
-  int modes;          // CSR level 0 of an assembled hierarchy: values per face (row i is mode i % modes);
-                      // 0 or 1 otherwise
-  const R* binv;      // stencil: [n_stencil][bs][bs]; CSR: [n] 1 / a_ii
+  const R* binv;      // CSR levels: [n] 1 / a_ii (stencil levels: in the operator tables)
   const int32_t *a_rp, *a_ci;
   const R* a_v;
   const int32_t *p_rp, *p_ci;   // prolongation [n x n_next] (CSR transfer)
@@ -64,11 +62,12 @@ struct MLLevelT {
   const R* r_v;
   R c0, c1, c2;       // Chebyshev(2) coefficients
   R *x, *b, *r, *d;   // work vectors [n * bs]
-  // a stencil level with a stencil of its own (NULL st_nbr: the facet stencil of the mesh):
-  // row i couples to itself and to st_nbr[i][0..st_nnb) through st_blk[st_cls[i]][1 + st_nnb][bs][bs]
-  const int32_t *st_cls, *st_nbr;
-  int st_nnb;
-  const R* st_blk;
+  // fused level (fuse_levels): b_next = D b and x = U [b; x_next] in sliced rows, dg / ug lanes a
+  // row. x_next follows b in memory ([n] then [n_next]); CSR arrays, r and d are not used
+  int fused;
+  int dg, ug;
+  const int32_t *d_ptr, *d_ci, *u_ptr, *u_ci;
+  const R *d_v, *u_v;
 };
 using MLLevelDev = MLLevelT<double>;
 
@@ -144,7 +143,13 @@ struct DevMesh {
   const MLLevelDev* ml_lv;            // [ml_nlev] in device memory
   const MLLevelT<float>* ml_lv_f;
   int ml_nlev, ml_nc;                 // smoothing levels, rows of the coarsest level
-  const double* ml_cpinv;             // [ml_nc][ml_nc] pseudo-inverse of the coarsest operator
+  int ml_ld;                          // row length of the pseudo-inverse (ml_nc padded to 4)
+  // operator tables of the solver kernel (ml_operator_table), in FP64 for the PCG and in the
+  // V-cycle's precision: per stencil class (ml_ncls > 0) or per facet (ml_ncls = 0)
+  int ml_ncls;
+  const double* ml_tab;
+  const float* ml_tab_f;              // mixed form
+  const double* ml_cpinv;             // [ml_nc][ml_ld] pseudo-inverse of the coarsest operator
   double *ml_xc, *ml_bc;              // coarsest vectors
   const float* ml_cpinv_f;
   float *ml_xc_f, *ml_bc_f;
@@ -239,6 +244,9 @@ cudaError_t launch_solve(const DevMesh& m, const SolveArgs& a, int nblocks, cuda
 // FP64 PCG with the multilevel preconditioner (k_multilevel.cu)
 cudaError_t launch_solve_ml(const DevMesh& m, const SolveArgs& a, int nblocks, cudaStream_t s);
 int solver_ml_blocks(const DevMesh& m);
+int ml_grid_threads();   // threads of the solver's full grid on the current device
+// whether the operators of ncls stencil classes (nl modes, nb blocks) fit in shared memory
+bool ml_class_tables_fit(int nl, int nb, bool fp32, int ncls);
 cudaError_t launch_ml_apply(const DevMesh& m, const double* r, double* z, int nblocks, cudaStream_t s);
 int solver_max_blocks(const DevMesh& m, int mixed);
 size_t lattice_smem_bytes(int k, int N, int fp32, int grp);

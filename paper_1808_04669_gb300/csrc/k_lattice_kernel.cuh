@@ -819,7 +819,7 @@ __device__ __forceinline__ void block_acc(Acc (&v)[N]) {
 }
 
 template <int N, typename Acc>
-__device__ bool lat_reduce(const DevMesh& m, int slot0, const Acc (&v)[N], GridBar* bar, double (&out)[N]) {
+__device__ bool lat_reduce(const DevMesh& m, int slot0, const Acc (&v)[N], Barrier& bar, double (&out)[N]) {
   Acc b[N];
 #pragma unroll
   for (int i = 0; i < N; ++i) b[i] = v[i];
@@ -900,7 +900,7 @@ __global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveAr
   __syncthreads();
   const int nF = m.n_facet;
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
-  GridBar* bar = m.bar;
+  Barrier bar(m.bar);
   // g from both sides of every facet and the warm start lam0. With a history (the same stage
   // of earlier steps), lam0 = c1 hist1 + c2 hist2 and r = g - S lam0 in the same pass (every
   // facet forms its neighbours' lam0 from the history, which this launch only reads until

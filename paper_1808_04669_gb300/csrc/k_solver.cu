@@ -30,7 +30,7 @@ namespace {
 // (two direction buffers), q. Returns iterations; sets *conv.
 template <int NL, typename R>
 __device__ int pcg(const DevMesh& m, R* x, R* rv, R* zv, R* pa, R* pb, R* qv, const R* blk_all, const R* binv_all,
-                   double stop_abs, int maxit, bool x_zero, GridBar* bar, bool* conv, double* rr_out) {
+                   double stop_abs, int maxit, bool x_zero, Barrier& bar, bool* conv, double* rr_out) {
   const int nF = m.n_facet;
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
   // z = B r, rho = r.z, rr = r.r ; x = 0 if requested. The residual norm used for
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve(DevMesh m, SolveArgs a
   constexpr int NL = K + 1;
   const int nF = m.n_facet;
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
-  GridBar* bar = m.bar;
+  Barrier bar(m.bar);
   // g_F = sum over both sides of the side's contribution mapped to canonical orientation
   double gg[2] = {0.0, 0.0};
   for (int f = gtid; f < nF; f += gsz) {
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve_noalloc(DevMesh m, con
   constexpr int NL = K + 1;
   const int nF = m.n_facet;
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
-  GridBar* bar = m.bar;
+  Barrier bar(m.bar);
   double gg[2] = {0.0, 0.0};
   for (int f = gtid; f < nF; f += gsz)
 #pragma unroll

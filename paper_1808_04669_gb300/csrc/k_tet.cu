@@ -321,14 +321,14 @@ __global__ void k_pressure3_finish(DevMesh3 m, double* pe, double* pf, const dou
 
 // Grid sum of N per-thread partials (fixed order; the result in every thread).
 template <int N>
-__device__ bool reduce3(const DevMesh3& m, int slot0, double (&v)[N]) {
+__device__ bool reduce3(const DevMesh3& m, Barrier& bar, int slot0, double (&v)[N]) {
   double s[N];
 #pragma unroll
   for (int i = 0; i < N; ++i) s[i] = block_sum(v[i]);
   if (threadIdx.x == 0)
 #pragma unroll
     for (int i = 0; i < N; ++i) m.red[size_t(slot0 + i) * kMaxSolverBlocks + blockIdx.x] = s[i];
-  if (!grid_sync(m.bar, m.stats)) return false;
+  if (!grid_sync(bar, m.stats)) return false;
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     double a = 0.0;
@@ -380,6 +380,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
   const int nF = m.n_face;
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
   const double inv_nf = 1.0 / double(nF);
+  Barrier bar(m.bar);
   double gg[2] = {0.0, 0.0};
   for (int f = gtid; f < nF; f += gsz) {
     const int t0 = m.face_tet[size_t(f) * 2], t1 = m.face_tet[size_t(f) * 2 + 1];
@@ -394,7 +395,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
     }
     warm_start_row<NL>(m.lam, a, size_t(f) * NL);
   }
-  if (!reduce3<2>(m, 4, gg)) return;
+  if (!reduce3<2>(m, bar, 4, gg)) return;
   const double c0 = gg[1] * inv_nf;
   const double gnorm = sqrt(fmax(gg[0] - gg[1] * gg[1] * inv_nf, 0.0));
   const double stop = a.rtol * gnorm;
@@ -424,7 +425,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
       }
       red[2] += r[0];
     }
-    if (!reduce3<3>(m, 1, red)) return;
+    if (!reduce3<3>(m, bar, 1, red)) return;
     double rho = red[0];
     rr = fmax(red[1] - red[2] * red[2] * inv_nf, 0.0);
     double beta = 0.0;
@@ -469,7 +470,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
           pq[0] += p0[j] * y[j];
         }
       }
-      if (!reduce3<1>(m, 0, pq)) return;
+      if (!reduce3<1>(m, bar, 0, pq)) return;
       if (!(pq[0] > 0.0)) {
         if (!isfinite(pq[0]) && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&m.stats->flags, kFlagNonFinite);
         break;
@@ -494,7 +495,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
         }
         red2[2] += r[0];
       }
-      if (!reduce3<3>(m, 1, red2)) return;
+      if (!reduce3<3>(m, bar, 1, red2)) return;
       beta = red2[0] / rho;
       rho = red2[0];
       rr = fmax(red2[1] - red2[2] * red2[2] * inv_nf, 0.0);

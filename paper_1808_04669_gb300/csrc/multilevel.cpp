@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <thread>
 
 #include "../../include/dgdf.h"
 
@@ -19,23 +20,35 @@ double dot(const Vec& a, const Vec& b) {
   return s;
 }
 
+// fn(begin, end, worker) over [0, n) on up to `most` of the host's cores, `grain` rows each at least
+template <typename F>
+void parallel_rows(int n, F fn, int most = 16, int grain = 512) {
+  const int nt = std::max(1, std::min({int(std::thread::hardware_concurrency()), most, n / grain}));
+  std::vector<std::thread> th;
+  for (int w = 1; w < nt; ++w)
+    th.emplace_back([&, w] { fn(int(int64_t(n) * w / nt), int(int64_t(n) * (w + 1) / nt), w); });
+  fn(0, n / nt, 0);
+  for (std::thread& t : th) t.join();
+}
+
 // ---- operators of one level on the host
 
 // y = A x on a stencil level: row F, modes i < bs: sum over the five stencil slots of the
 // leading bs x bs sub-block of S's (k+1) x (k+1) block times the neighbour's first bs values.
 void stencil_apply(const HostMesh& hm, int bs, const double* x, double* y) {
   const int nl = hm.nl;
-  const int64_t nf = hm.topo.n_facet;
-  for (int64_t f = 0; f < nf; ++f) {
-    const double* blk = &hm.stencil_blocks[size_t(hm.facet_stencil[f]) * 5 * nl * nl];
-    int64_t nb[5] = {f, hm.facet_nbr[f * 4], hm.facet_nbr[f * 4 + 1], hm.facet_nbr[f * 4 + 2], hm.facet_nbr[f * 4 + 3]};
-    for (int i = 0; i < bs; ++i) {
-      double v = 0.0;
-      for (int b = 0; b < 5; ++b)
-        for (int j = 0; j < bs; ++j) v += blk[(size_t(b) * nl + i) * nl + j] * x[nb[b] * bs + j];
-      y[f * bs + i] = v;
+  parallel_rows(int(hm.topo.n_facet), [&](int f0, int f1, int) {
+    for (int64_t f = f0; f < f1; ++f) {
+      const double* blk = &hm.stencil_blocks[size_t(hm.facet_stencil[f]) * 5 * nl * nl];
+      int64_t nb[5] = {f, hm.facet_nbr[f * 4], hm.facet_nbr[f * 4 + 1], hm.facet_nbr[f * 4 + 2], hm.facet_nbr[f * 4 + 3]};
+      for (int i = 0; i < bs; ++i) {
+        double v = 0.0;
+        for (int b = 0; b < 5; ++b)
+          for (int j = 0; j < bs; ++j) v += blk[(size_t(b) * nl + i) * nl + j] * x[nb[b] * bs + j];
+        y[f * bs + i] = v;
+      }
     }
-  }
+  }, 8, 8192);
 }
 
 void csr_apply(const CsrHost& A, const double* x, double* y) {
@@ -389,13 +402,37 @@ void vcycle(const HostMesh& hm, const MLHost& ml, size_t l, const double* b, dou
   smooth(hm, L, b, x1.data(), x);
 }
 
+// In-place inverse of a symmetric positive definite matrix by symmetric sweeps (Gauss-Jordan steps
+// on the lower triangle, n^3 / 2 multiply-adds); false if a pivot is not positive.
+bool invert_spd(Vec& A, int n) {
+  Vec v(n);
+  for (int k = 0; k < n; ++k) {
+    const double d = A[size_t(k) * n + k];
+    if (!(d > 0.0)) return false;
+    for (int j = 0; j < k; ++j) v[j] = A[size_t(k) * n + j];
+    for (int i = k + 1; i < n; ++i) v[i] = A[size_t(i) * n + k];
+    v[k] = 0.0;
+    for (int i = 0; i < n; ++i) {
+      const double s = v[i] / d;
+      double* row = &A[size_t(i) * n];
+      for (int j = 0; j <= i; ++j) row[j] -= s * v[j];
+    }
+    for (int j = 0; j < k; ++j) A[size_t(k) * n + j] = v[j] / d;
+    for (int i = k + 1; i < n; ++i) A[size_t(i) * n + k] = v[i] / d;
+    A[size_t(k) * n + k] = -1.0 / d;
+  }
+  for (int i = 0; i < n; ++i)
+    for (int j = 0; j <= i; ++j) A[size_t(i) * n + j] = A[size_t(j) * n + i] = -A[size_t(i) * n + j];
+  return true;
+}
+
 // Pseudo-inverse of the coarsest operator A (symmetric positive semi-definite, nc rows), dense,
 // symmetrised. Up to 256 rows: from its eigen-decomposition, the eigenvalues below 1e-10 of the
 // largest dropped. Larger (the Jacobi eigensolver's cost grows as nc^3 per sweep): when the
 // near-null vector v is in the kernel (|A v| <= 1e-9 |A|_F |v|, a closed mesh), through the
 // definite matrix B = A + s u u^T (u = v / |v|, s the mean diagonal entry), whose inverse is
 // A^+ + u u^T / s, so that A^+ = B^-1 - u u^T / s; otherwise (A definite) A^-1. Both by
-// Gauss-Jordan elimination with partial pivoting. Returns false if the matrix is singular.
+// symmetric sweeps (invert_spd). Returns false if the matrix is not definite.
 bool coarse_pinv(const CsrHost& A, const Vec& v, Vec& out) {
   const int nc = A.n_rows;
   Vec D(size_t(nc) * nc, 0.0);
@@ -434,7 +471,7 @@ bool coarse_pinv(const CsrHost& A, const Vec& v, Vec& out) {
   if (kernel)
     for (int r = 0; r < nc; ++r)
       for (int c = 0; c < nc; ++c) D[size_t(r) * nc + c] += s * v[r] * v[c] / vv;
-  if (!host_invert(D, nc)) return false;
+  if (!invert_spd(D, nc)) return false;
   for (int r = 0; r < nc; ++r)
     for (int c = 0; c < nc; ++c) {
       double x = 0.5 * (D[size_t(r) * nc + c] + D[size_t(c) * nc + r]);
@@ -444,7 +481,240 @@ bool coarse_pinv(const CsrHost& A, const Vec& v, Vec& out) {
   return true;
 }
 
+// Sparse accumulator over a row of n columns
+struct RowAcc {
+  Vec v;
+  std::vector<int32_t> mark, cols;
+  int row = -1;
+  explicit RowAcc(int n) : v(n, 0.0), mark(n, -1) {}
+  void start(int r) {
+    row = r;
+    cols.clear();
+  }
+  void add(int c, double x) {
+    if (mark[c] != row) {
+      mark[c] = row;
+      v[c] = 0.0;
+      cols.push_back(c);
+    }
+    v[c] += x;
+  }
+};
+
+// rows (columns and values of each) -> sliced layout with G lanes a row
+SellHost make_sell(const CsrHost& M, int grid_threads) {
+  SellHost S;
+  S.n_rows = M.n_rows;
+  while (S.G < 32 && int64_t(2) * S.G * M.n_rows <= grid_threads) S.G *= 2;
+  const int per = 32 / S.G, ns = (M.n_rows + per - 1) / per;
+  S.ptr.assign(ns + 1, 0);
+  for (int s = 0; s < ns; ++s) {
+    int w = 0;
+    for (int i = s * per; i < std::min(M.n_rows, (s + 1) * per); ++i)
+      w = std::max(w, (M.rp[i + 1] - M.rp[i] + S.G - 1) / S.G);
+    S.ptr[s + 1] = S.ptr[s] + w;
+  }
+  S.ci.assign(size_t(S.ptr[ns]) * 32, 0);
+  S.v.assign(size_t(S.ptr[ns]) * 32, 0.0);
+  parallel_rows(ns, [&](int s0, int s1, int) {
+    for (int s = s0; s < s1; ++s)
+      for (int i = s * per; i < std::min(M.n_rows, (s + 1) * per); ++i)
+        for (int p = M.rp[i]; p < M.rp[i + 1]; ++p) {
+          const int q = p - M.rp[i];
+          const size_t o = (size_t(S.ptr[s]) + q / S.G) * 32 + (i - s * per) * S.G + q % S.G;
+          S.ci[o] = M.ci[p];
+          S.v[o] = M.v[p];
+        }
+  });
+  return S;
+}
+
+// Of a level with operator A, diagonal inverse B and prolongation P: M2 = 2 N - N A N and
+// DT = (I - N A) P (N: fuse_levels). Row by row: t = N_i, s = t A, M2_i = 2 t - s N, DT_i = P_i - s P.
+void fused_rows(const MLHostLevel& L, const CsrHost& A, CsrHost& M2, CsrHost& DT) {
+  const int n = A.n_rows;
+  const double c0 = L.cheb[0], c1 = L.cheb[1], c2 = L.cheb[2], a = (1.0 + c1) * c0 + c2, c = c2 * c0;
+  Vec B(n, 0.0);
+  for (int i = 0; i < n; ++i)
+    for (int p = A.rp[i]; p < A.rp[i + 1]; ++p)
+      if (A.ci[p] == i) B[i] += A.v[p];
+  for (double& d : B) d = 1.0 / d;
+  CsrHost N = A;
+  for (int i = 0; i < n; ++i) {
+    bool first = true;
+    for (int p = A.rp[i]; p < A.rp[i + 1]; ++p) {
+      N.v[p] = -c * B[i] * A.v[p] * B[A.ci[p]];
+      if (A.ci[p] == i && first) {
+        N.v[p] += a * B[i];
+        first = false;
+      }
+    }
+  }
+  struct Part {
+    int i0 = 0;
+    std::vector<int32_t> len[2], ci[2];
+    Vec v[2];
+  };
+  std::vector<Part> parts(17);
+  parallel_rows(n, [&](int i0, int i1, int w) {
+    Part& Q = parts[w];
+    Q.i0 = i0;
+    RowAcc s(n), m(n), d(L.P.n_cols);
+    for (int i = i0; i < i1; ++i) {
+      s.start(i);
+      m.start(i);
+      d.start(i);
+      for (int p = N.rp[i]; p < N.rp[i + 1]; ++p) {
+        const int k = N.ci[p];
+        m.add(k, 2.0 * N.v[p]);
+        for (int q = A.rp[k]; q < A.rp[k + 1]; ++q) s.add(A.ci[q], N.v[p] * A.v[q]);
+      }
+      for (int p = L.P.rp[i]; p < L.P.rp[i + 1]; ++p) d.add(L.P.ci[p], L.P.v[p]);
+      for (int k : s.cols) {
+        const double x = s.v[k];
+        for (int q = N.rp[k]; q < N.rp[k + 1]; ++q) m.add(N.ci[q], -x * N.v[q]);
+        for (int q = L.P.rp[k]; q < L.P.rp[k + 1]; ++q) d.add(L.P.ci[q], -x * L.P.v[q]);
+      }
+      RowAcc* acc[2] = {&m, &d};
+      for (int h = 0; h < 2; ++h) {
+        Q.len[h].push_back(int32_t(acc[h]->cols.size()));
+        for (int k : acc[h]->cols) {
+          Q.ci[h].push_back(k);
+          Q.v[h].push_back(acc[h]->v[k]);
+        }
+      }
+    }
+  });
+  CsrHost* out[2] = {&M2, &DT};
+  for (int h = 0; h < 2; ++h) {
+    CsrHost& C = *out[h];
+    C = CsrHost();
+    C.n_rows = n;
+    C.n_cols = h == 0 ? n : L.P.n_cols;
+    C.rp.assign(1, 0);
+    std::vector<const Part*> order;
+    for (const Part& Q : parts)
+      if (!Q.len[h].empty()) order.push_back(&Q);
+    std::sort(order.begin(), order.end(), [](const Part* x, const Part* y) { return x->i0 < y->i0; });
+    for (const Part* Q : order) {
+      for (int32_t l : Q->len[h]) C.rp.push_back(C.rp.back() + l);
+      C.ci.insert(C.ci.end(), Q->ci[h].begin(), Q->ci[h].end());
+      C.v.insert(C.v.end(), Q->v[h].begin(), Q->v[h].end());
+    }
+  }
+}
+
 }  // namespace
+
+void fuse_levels(MLHost& ml, int word, int dense_max, int grid_threads) {
+  std::vector<CsrHost> M2(ml.lv.size()), DT(ml.lv.size());
+  for (int l = int(ml.lv.size()) - 1; l >= 0; --l) {
+    MLHostLevel& L = ml.lv[l];
+    if (L.bs != 1 || L.inject || L.A.n_rows != L.n || L.P.n_rows != L.n) break;
+    // a level far above the limits is not formed: A's third power reaches some five times its
+    // entries on facets of triangles, more elsewhere
+    if (5.0 * double(L.A.ci.size()) * (4 + word) > kMLFuseBytes) break;
+    fused_rows(L, L.A, M2[l], DT[l]);
+    const double entries = double(M2[l].ci.size()) + 2.0 * double(DT[l].ci.size());
+    if (L.n > dense_max && (entries > kMLFuseFill * double(L.A.ci.size()) || entries * (4 + word) > kMLFuseBytes)) break;
+    L.fused = true;
+  }
+  while (!ml.lv.empty() && ml.lv.back().fused && ml.lv.back().n <= dense_max && ml.lv.size() > 1) {
+    const int l = int(ml.lv.size()) - 1, n = ml.lv[l].n, nc = ml.nc;
+    const CsrHost &T = DT[l], D = transpose(T);
+    Vec W(size_t(nc) * n, 0.0), M(size_t(n) * n, 0.0);   // W = pinv D, M = M2 + D^T W
+    parallel_rows(nc, [&](int i0, int i1, int) {
+      for (int i = i0; i < i1; ++i)
+        for (int k = 0; k < nc; ++k) {
+          const double x = ml.cpinv[size_t(i) * nc + k];
+          for (int p = D.rp[k]; p < D.rp[k + 1]; ++p) W[size_t(i) * n + D.ci[p]] += x * D.v[p];
+        }
+    });
+    parallel_rows(n, [&](int i0, int i1, int) {
+      for (int i = i0; i < i1; ++i) {
+        double* row = &M[size_t(i) * n];
+        for (int p = T.rp[i]; p < T.rp[i + 1]; ++p) {
+          const double x = T.v[p], *w = &W[size_t(T.ci[p]) * n];
+          for (int j = 0; j < n; ++j) row[j] += x * w[j];
+        }
+        for (int p = M2[l].rp[i]; p < M2[l].rp[i + 1]; ++p) row[M2[l].ci[p]] += M2[l].v[p];
+      }
+    });
+    ml.cpinv.swap(M);
+    ml.nc = n;
+    ml.lv.pop_back();
+  }
+  for (size_t l = 0; l < ml.lv.size(); ++l) {
+    MLHostLevel& L = ml.lv[l];
+    if (!L.fused) continue;
+    L.D = make_sell(transpose(DT[l]), grid_threads);
+    CsrHost U;   // [M2 | D^T]
+    U.n_rows = L.n;
+    U.n_cols = L.n + L.n_next;
+    U.rp.assign(1, 0);
+    for (int i = 0; i < L.n; ++i) {
+      U.ci.insert(U.ci.end(), M2[l].ci.begin() + M2[l].rp[i], M2[l].ci.begin() + M2[l].rp[i + 1]);
+      U.v.insert(U.v.end(), M2[l].v.begin() + M2[l].rp[i], M2[l].v.begin() + M2[l].rp[i + 1]);
+      for (int p = DT[l].rp[i]; p < DT[l].rp[i + 1]; ++p) {
+        U.ci.push_back(L.n + DT[l].ci[p]);
+        U.v.push_back(DT[l].v[p]);
+      }
+      U.rp.push_back(int32_t(U.ci.size()));
+    }
+    L.U = make_sell(U, grid_threads);
+  }
+}
+
+std::vector<double> ml_operator_table(bool class_tables, int nl, int nb, int n_cls, int n, const int32_t* cls,
+                                      const double* blocks, int word) {
+  const int rs = ml_row_stride(nl), lp = ml_lanes(nl) * ml_modes(nl), bb = nl * nl;
+  // inverses of the leading m x m sub-blocks of the own block
+  auto inverse = [&](int s, int m) {
+    std::vector<double> B(size_t(m) * m);
+    for (int a = 0; a < m; ++a)
+      for (int c = 0; c < m; ++c) B[size_t(a) * m + c] = blocks[size_t(s) * nb * bb + a * nl + c];
+    invert_small(B, m);
+    return B;
+  };
+  std::vector<double> out;
+  if (class_tables) {
+    const int st = ml_class_stride(nl, nb, word);
+    out.assign(size_t(n_cls) * st, 0.0);
+    for (int s = 0; s < n_cls; ++s) {
+      double* o = &out[size_t(s) * st];
+      for (int b = 0; b < nb; ++b)
+        for (int i = 0; i < nl; ++i)
+          for (int j = 0; j < nl; ++j) o[(b * nl + i) * rs + j] = blocks[(size_t(s) * nb + b) * bb + i * nl + j];
+      o += nb * nl * rs;
+      const std::vector<double> Bn = inverse(s, nl), B2 = inverse(s, 2);
+      for (int i = 0; i < nl; ++i)
+        for (int j = 0; j < nl; ++j) o[i * rs + j] = Bn[i * nl + j];
+      o += nl * rs;
+      std::copy(B2.begin(), B2.end(), o);
+      o[4] = 1.0 / blocks[size_t(s) * nb * bb];
+    }
+    return out;
+  }
+  const size_t N = size_t(n);
+  out.assign(N * (size_t(nb + 1) * nl * lp + 5), 0.0);
+  double *bn = &out[N * nb * nl * lp], *b2 = bn + N * nl * lp, *b1 = b2 + 4 * N;
+  parallel_rows(n, [&](int f0, int f1, int) {
+    for (int f = f0; f < f1; ++f) {
+      const int s = cls[f];
+      for (int b = 0; b < nb; ++b)
+        for (int i = 0; i < nl; ++i)
+          for (int j = 0; j < nl; ++j)
+            out[((size_t(b) * nl + j) * N + f) * lp + i] = blocks[(size_t(s) * nb + b) * bb + i * nl + j];
+      const std::vector<double> Bn = inverse(s, nl), B2 = inverse(s, 2);
+      for (int i = 0; i < nl; ++i)
+        for (int j = 0; j < nl; ++j) bn[(size_t(j) * N + f) * lp + i] = Bn[i * nl + j];
+      for (int i = 0; i < 2; ++i)
+        for (int j = 0; j < 2; ++j) b2[(size_t(j) * N + f) * 2 + i] = B2[i * 2 + j];
+      b1[f] = 1.0 / blocks[size_t(s) * nb * bb];
+    }
+  });
+  return out;
+}
 
 int build_multilevel(const HostMesh& hm, MLHost& ml, std::string& err) {
   ml = MLHost();
@@ -491,6 +761,7 @@ int build_multilevel(const HostMesh& hm, MLHost& ml, std::string& err) {
       if (last.stencil && last.bs == 1 && last.P.n_rows == 0) {
         last.P = P;
         last.R = R;
+        last.A = A;
         last.inject = false;
         last.n_next = P.n_cols;
       } else {

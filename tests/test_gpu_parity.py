@@ -590,3 +590,23 @@ def test_iteration_cap_reports_not_converged(g):
     with pytest.raises(DGError) as e:
         mesh.project_divfree()
     assert e.value.code == -5
+
+
+@pytest.mark.parametrize("N,k,walls,perturb", [(3, 1, True, 0.0), (17, 2, True, 0.0), (22, 3, False, 0.1),
+                                               (45, 1, False, 0.1), (97, 2, True, 0.0), (300, 1, True, 0.0)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_multilevel_solver_forms_match_the_host_v_cycle(g, N, k, walls, perturb, precision):
+    # the forms a V-cycle takes on the device against the host's: fewer facets than one block's
+    # lanes, the coarsest level taking in the level above (17^2, 45^2), operators per stencil class
+    # (walls) and per facet (perturbed), fused levels, and at 300^2 a facet-constant level too large
+    # to fuse above fused ones. FP64: sums of some hundred terms through five levels, 1e-12; FP32:
+    # the same at 2^-24, amplified by the cycle as in the tests above, 1e-5
+    vid, X = synth.split_square_mesh(N, L=1.0, periodic=not walls)
+    if perturb:
+        rng = np.random.default_rng(N)
+        X = X + (perturb / N * rng.uniform(-1, 1, size=(N * N, 2)))[vid]
+    mesh = g.DGMesh(vid, X, k, 1e-4, precision=precision, precond=g.PRECOND_MULTILEVEL)
+    r = np.random.default_rng(2).standard_normal((mesh.n_facet, k + 1))
+    r[:, 0] -= r[:, 0].mean()
+    host = g.host_multilevel(vid, X, k, r=r.reshape(1, -1))["z"][0]
+    assert rel(mesh.test_multilevel_apply(r.ravel()), host) < (1e-5 if precision else 1e-12)
