@@ -317,6 +317,7 @@ int solve(dg_mesh* M, double warm_scale, int stage = -1, double dt = 0.0, bool h
       a.c2 = -1.0;
     }
   }
+  if (stage >= 0 && M->use_lattice) a.hist_new = M->hist[stage][0];
   a.rtol = M->p.cg_rtol;
   a.maxit = M->p.cg_maxit;
   a.mixed = M->p.precision == DG_PRECISION_MIXED;
@@ -338,12 +339,14 @@ int solve(dg_mesh* M, double warm_scale, int stage = -1, double dt = 0.0, bool h
 }
 
 // After the solve of RK stage s with step size dt: the new multipliers become the newest
-// history entry (the solver already moved the older ones down one slot).
+// history entry (the solver already moved the older ones down one slot; the lattice solver
+// has stored the new one, too).
 int push_history(dg_mesh* M, int s, double dt) {
   if (M->hist_len == 0) return DG_OK;
-  const void* lam = M->dm.lam_is_df ? static_cast<const void*>(M->dm.lam_df) : static_cast<const void*>(M->dm.lam);
-  M->prof_prev = nullptr;   // a copy between two launches: no chained profiling event across it
-  CK(cudaMemcpyAsync(M->hist[s][0], lam, M->hist_bytes, cudaMemcpyDeviceToDevice, M->stream));
+  if (!M->use_lattice) {
+    M->prof_prev = nullptr;   // a copy between two launches: no chained profiling event across it
+    CK(cudaMemcpyAsync(M->hist[s][0], M->dm.lam, M->hist_bytes, cudaMemcpyDeviceToDevice, M->stream));
+  }
   for (int h = M->hist_len - 1; h > 0; --h) M->hist_dt[s][h] = M->hist_dt[s][h - 1];
   M->hist_dt[s][0] = dt;
   M->hist_n[s] = std::min(M->hist_n[s] + 1, M->hist_len);
@@ -806,6 +809,19 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
       }
     }
     d.lat_facet_of = fo;
+    {
+      std::vector<int2> src(size_t(d.n_facet));
+      for (int f = 0; f < d.n_facet; ++f) {
+        int v[2];
+        for (int q = 0; q < 2; ++q) {
+          const int64_t t = hm.topo.facet_tri[size_t(f) * 2 + q];
+          const int e = hm.topo.facet_loc[size_t(f) * 2 + q];
+          v[q] = int((t * 3 + e) * hm.nl * 2 + (hm.topo.tri_orient[size_t(t) * 3 + e] < 0 ? 1 : 0));
+        }
+        src[f] = make_int2(v[0], v[1]);
+      }
+      if ((rc = upload(M, &d.lat_src, src))) return cleanup(rc);
+    }
     d.facet_ext = fe;
     d.lat_tw = tw;
     d.lat_N = N;

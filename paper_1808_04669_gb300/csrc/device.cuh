@@ -123,6 +123,8 @@ struct DevMesh {
   int lat_bufsz;                    // complex elements of the shared-memory transform buffer
   int lat_grp;                      // rows per transform group (scratch of lat_grp rows)
   const int32_t* lat_facet_of;        // [3][N][N]
+  const int2* lat_src;                // [n_facet] where the two sides' condensation outputs lie in gl:
+                                      // 2 x the offset of mode 0, + 1 if the side runs the facet backwards
   const void* lat_sinv;               // [N/2+1][C(C+1)/2 (FP32) or C*C (FP64)][N] complex
   const double* lat_tw;               // [N][2]
   void* lat_x;                        // [C][N/2+1][N] complex work array
@@ -172,6 +174,7 @@ constexpr int kRedSlots = 8;
 constexpr int kMLHist = 512;
 constexpr int kDnClasses = 4;
 constexpr int kMaxSolverBlocks = 2048;
+constexpr int kLatStencils = 3;     // stencil classes that the lattice solver keeps in shared memory
 
 // Stage kernel modes.
 enum StageMode : int {
@@ -208,6 +211,7 @@ struct SolveArgs {
   void* hist2;
   void* hist3;
   double c1, c2, c3;
+  void* hist_new;      // lattice solver: where to store the new lam too (NULL: nowhere); may be hist1
 };
 
 // Launchers (k dispatched at run time). Return the launch error.

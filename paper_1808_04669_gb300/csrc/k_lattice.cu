@@ -54,14 +54,21 @@ bool lattice_split(int N) {
   return N % 2 == 0 && N >= 64 && N / 2 + 1 <= sms;
 }
 
+// complex elements before the half-length twiddles: the twiddles and the transform buffers, in
+// which the reductions keep kLatSums rows of 8-byte partials
 size_t lattice_tw2_offset(int k, int N, int fp32, int grp) {
-  return size_t(N) + lattice_buffer_elems(k, N, fp32) + size_t(grp) * lattice_scratch_row(N);
+  const size_t buf = lattice_buffer_elems(k, N, fp32) + size_t(grp) * lattice_scratch_row(N);
+  const size_t sums = size_t(kLatSums) * kLatThreads * 8 / (fp32 ? 8 : 16);
+  return size_t(N) + (buf > sums ? buf : sums);
 }
 
 size_t lattice_smem_bytes(int k, int N, int fp32, int grp) {
   const size_t cx = fp32 ? 8 : 16;
   return (lattice_tw2_offset(k, N, fp32, grp) + (lattice_split(N) ? size_t(N / 2) : 0)) * cx;
 }
+
+// static shared memory of the kernel: three stencil classes of BDM_3 and the solve's scalars
+constexpr size_t kLatStatic = 2400;
 
 // Rows per transform group: all of them if two blocks per SM still fit, else the most
 // that fit at two blocks per SM, else at one block per SM; 0 if not even one row fits.
@@ -71,7 +78,7 @@ int lattice_group_rows(int k, int N, int fp32) {
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   const int rows = int(lattice_buffer_elems(k, N, fp32) / size_t(N));
-  const size_t two = size_t(per_sm) / 2 - 2048, one = size_t(optin) - 2048;
+  const size_t two = size_t(per_sm) / 2 - 1024 - kLatStatic, one = size_t(optin) - kLatStatic;
   for (size_t budget : {two, one})
     for (int g = rows; g >= 1; --g)
       if (lattice_smem_bytes(k, N, fp32, g) <= budget) return g;

@@ -4,11 +4,17 @@
 // On such a mesh the facet operator S is block circulant over the N x N cell
 // grid: a 2-D discrete Fourier transform turns it into one Hermitian block
 // S^(kappa) of size C = 3(k+1) per wavenumber, and S^+ r = IDFT(S^(kappa)^+ DFT(r))
-// (pseudo-inverse at kappa = 0, the constant multiplier). This kernel runs PCG
-// preconditioned by that Fourier-space inverse:
-//   FP64 form : FP64 vectors, FP64 SpMV, FP64 transforms (one or two iterations);
-//   mixed form: double-float vectors and SpMV on the FP32 units, FP32 transforms
-//               (a few iterations: the preconditioned operator is I + O(FP32 rounding)).
+// (pseudo-inverse at kappa = 0, the constant multiplier). The Fourier-space inverse B is S^+ up
+// to rounding, so the solve is iterative refinement:
+//   z = B r,  lam += z,  r -= S z   until |r| <= rtol |g|.
+//   FP64 form : FP64 vectors, FP64 products, FP64 transforms (one iteration);
+//   mixed form: double-float vectors and products on the FP32 units, FP32 transforms (two or
+//               three iterations: each gains the FP32 rounding times cond(S), 1e4 at N = 256).
+// Where an iteration gains less than a factor of ten, the solve goes on as PCG preconditioned by B
+// (lat_pcg), which needs two more vectors, their traffic, two more reductions an iteration and a
+// last row pass for nothing. The solve is bound by latency (16 warps an SM between grid barriers):
+// 9 grid-wide phases at 2 iterations. N = 256, BDM_3, mixed form: 244 us as PCG with a thread a
+// facet, 170 us now; FP64 form at N = 128: 222 -> 157 us; N = 8, BDM_2, FP64: 98 -> 55 us.
 // The residual is real, so only the wavenumbers ki in [0, N/2] are transformed:
 //   rows   : two facet rows j, j+1 packed as one complex row, FFT along i, split
 //            into the two half spectra (Hermitian symmetry)
@@ -222,25 +228,70 @@ struct FourStepMax<double2> {
   static constexpr int logn = 8;
 };
 
-// Direct DFT of `rows` rows of length n (any n): out[r][k] = sum_t in[r][t] w^(t k mod n),
-// w[m] = exp(-2 pi i m / n) (conjugated for the inverse). Natural order in and out.
+// DFT of `rows` rows of any length N = R1 R2 held in a (natural order, in place) through the scratch
+// s, as fft_four_step with direct sums in both passes: N (R1 + R2) multiply-adds a row instead of
+// the N^2 of one sum (R1 = 1, a prime N). A thread forms kDftOut outputs at once, so that an input
+// read from shared memory serves as many sums. tw[t] = exp(-2 pi i t / N), conjugated for the
+// inverse. (N = 150, BDM_3, mixed form, 3.5 iterations: with this and the refinement a solve fell
+// from 563 to 199 us; at the prime 127 only the shared inputs help.)
+constexpr int kDftOut = 4;
 template <typename C2>
-__device__ void dft(const C2* in, C2* out, int rows, int n, const C2* tw, bool inverse) {
-  for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
-    const int row = e / n, k = e - row * n;
-    const C2* x = in + row * n;
-    C2 acc = {0, 0};
-    int idx = 0;
-    for (int t = 0; t < n; ++t) {
-      C2 w = tw[idx];
-      if (inverse) w.y = -w.y;
-      acc = cadd(acc, cmul(x[t], w));
-      idx += k;
-      if (idx >= n) idx -= n;
+__device__ void dft_two_factor(C2* a, C2* s, int rows, int N, int R1, const C2* tw, bool inverse) {
+  const int R2 = N / R1;
+  // out[j0 + u] = sum_t in[t is] w^(t step (j0 + u)), u < kDftOut (outputs past `n` are dropped)
+  auto sums = [&](const C2* in, int is, int n, int step, int j0, C2 (&acc)[kDftOut]) {
+    int idx[kDftOut], inc[kDftOut];
+#pragma unroll
+    for (int u = 0; u < kDftOut; ++u) {
+      acc[u] = C2{0, 0};
+      idx[u] = 0;
+      inc[u] = j0 + u < n ? (j0 + u) * step : 0;   // < N
     }
-    out[e] = acc;
+    for (int t = 0; t < n; ++t) {
+      const C2 x = in[t * is];
+#pragma unroll
+      for (int u = 0; u < kDftOut; ++u) {
+        C2 w = tw[idx[u]];
+        if (inverse) w.y = -w.y;
+        cmad(acc[u], w, x);
+        idx[u] += inc[u];
+        if (idx[u] >= N) idx[u] -= N;
+      }
+    }
+  };
+  // pass 1: over n2 for each n1, then the twiddle w^(n1 k2): s[k2 R1 + n1]
+  const int g2 = (R2 + kDftOut - 1) / kDftOut;
+  for (int e = threadIdx.x; e < rows * R1 * g2; e += blockDim.x) {
+    const int n1 = e % R1, rest = e / R1, k0 = (rest % g2) * kDftOut, row = rest / g2;
+    C2 acc[kDftOut];
+    sums(a + size_t(row) * N + n1, R1, R2, R1, k0, acc);
+#pragma unroll
+    for (int u = 0; u < kDftOut; ++u)
+      if (k0 + u < R2) {
+        C2 w = tw[n1 * (k0 + u)];
+        if (inverse) w.y = -w.y;
+        s[size_t(row) * N + (k0 + u) * R1 + n1] = cmul(acc[u], w);
+      }
   }
   __syncthreads();
+  // pass 2: over n1 for each k2: X[k2 + R2 k1]
+  const int g1 = (R1 + kDftOut - 1) / kDftOut;
+  for (int e = threadIdx.x; e < rows * R2 * g1; e += blockDim.x) {
+    const int k2 = e % R2, rest = e / R2, k0 = (rest % g1) * kDftOut, row = rest / g1;
+    C2 acc[kDftOut];
+    sums(s + size_t(row) * N + k2 * R1, 1, R1, R2, k0, acc);
+#pragma unroll
+    for (int u = 0; u < kDftOut; ++u)
+      if (k0 + u < R1) a[size_t(row) * N + k2 + R2 * (k0 + u)] = acc[u];
+  }
+  __syncthreads();
+}
+
+// the divisor of N nearest to its square root from below
+__device__ __forceinline__ int dft_factor(int N) {
+  int r = int(sqrtf(float(N)) + 0.5f);
+  while (N % r) --r;
+  return r;
 }
 
 template <int K, bool MIXED>
@@ -257,7 +308,8 @@ struct LatCtx {
   static constexpr int NP = MIXED ? C + 1 + C * (C + 1) / 2 : C * C;
   int N, logn, NK, ntj;   // NK = N/2 + 1 wavenumbers ki; ntj row tiles per facet type
   int grp;                // rows transformed at a time (the scratch holds grp rows)
-  bool pow2;              // FFT (N a power of two) or direct DFT
+  bool pow2;              // FFT (N a power of two) or two-factor DFT
+  int r1;                 // its first factor
   C2* tw;                 // [N] exp(-2 pi i t / N)
   C2* bufa;               // transform data, max(C, 2(k+1)) rows of N
   C2* scr;                // scratch, grp rows of lattice_scratch_row(N)
@@ -276,8 +328,8 @@ struct LatCtx {
 
 // Forward or inverse transform, in place, of `rows` natural-order rows held in a: groups
 // of L.grp rows go through the scratch buffer. Powers of two up to FourStepMax: the
-// two-pass FFT; larger powers of two: Stockham passes; other N: the direct DFT (both
-// out of place; a result left in the scratch is copied back).
+// two-pass FFT; larger powers of two: Stockham passes (a result left in the scratch is
+// copied back); other N: the two-factor DFT.
 template <int K, bool MIXED>
 __device__ void xform(const LatCtx<K, MIXED>& L, typename LatT<MIXED>::C2* a, int rows, bool inverse) {
   using C2 = typename LatT<MIXED>::C2;
@@ -305,16 +357,14 @@ __device__ void xform(const LatCtx<K, MIXED>& L, typename LatT<MIXED>::C2* a, in
       }
       continue;
     }
-    const C2* res;
     if (L.pow2) {
-      res = fft_stockham(d, L.scr, gr, L.logn, L.tw, inverse);
+      const C2* res = fft_stockham(d, L.scr, gr, L.logn, L.tw, inverse);
+      if (res != d) {
+        for (int e = threadIdx.x; e < gr * N; e += blockDim.x) d[e] = res[e];
+        __syncthreads();
+      }
     } else {
-      dft(d, L.scr, gr, N, L.tw, inverse);
-      res = L.scr;
-    }
-    if (res != d) {
-      for (int e = threadIdx.x; e < gr * N; e += blockDim.x) d[e] = res[e];
-      __syncthreads();
+      dft_two_factor(d, L.scr, gr, N, L.r1, L.tw, inverse);
     }
   }
 }
@@ -408,18 +458,11 @@ __device__ __forceinline__ void stf(double* p, const double (&v)[NL]) {
 // facet type with all k+1 modes is one contiguous range of the facet-major vectors:
 // DOF index ((type N + j) N + i) VS + m.
 
-// Row pass, forward: per tile read r and update it: with `update`, r -= alpha q + c_prev 1 and
-// lam += alpha_lam p (1 is the constant multiplier, mode 0 on every facet); without (the first
-// pass of a solve, r holding g - S lam0), r = scale (r - c_prev 1), and the multiplier history
-// moves down one slot (hdst <- hsrc, when hsrc is set). Accumulate r.r and the sum of the
-// mode-0 entries of r, pack rows j0+2p (real part) and j0+2p+1 (imaginary part) per mode, FFT
-// along i, split into the two rows' half spectra and store them in X.
-template <int K, bool MIXED>
-__device__ void rows_forward(const LatCtx<K, MIXED>& L, bool update, typename LatT<MIXED>::A alpha,
-                             typename LatT<MIXED>::A alpha_lam, typename LatT<MIXED>::A c_prev,
-                             const typename LatT<MIXED>::V* p, typename LatT<MIXED>::Acc& rr,
-                             typename LatT<MIXED>::Acc& r0sum, typename LatT<MIXED>::A scale,
-                             const typename LatT<MIXED>::V* hsrc, typename LatT<MIXED>::V* hdst) {
+// Row pass, forward: per tile read r; src(o, rv) sees (and may change) the values of the facet that
+// start at o; pack rows j0+2p (real part) and j0+2p+1 (imaginary part) per mode, FFT along i, split
+// into the two rows' half spectra and store them in X.
+template <int K, bool MIXED, typename Src>
+__device__ __forceinline__ void rows_forward(const LatCtx<K, MIXED>& L, Src src) {
   using T = LatT<MIXED>;
   using C2 = typename T::C2;
   using R = typename T::R;
@@ -437,34 +480,9 @@ __device__ void rows_forward(const LatCtx<K, MIXED>& L, bool update, typename La
       const size_t o = base + size_t(e) * VS;
       A rv[NL];
       ldf<NL, VS>(L.r + o, rv);
-      if (update) {
-        A qv[NL], lv[NL], pv[NL];
-        ldf<NL, VS>(L.q + o, qv);
-        ldf<NL, VS>(L.lam + o, lv);
-        ldf<NL, VS>(p + o, pv);
-#pragma unroll
-        for (int mm = 0; mm < NL; ++mm) {
-          rv[mm] = rv[mm] - alpha * qv[mm];
-          lv[mm] = lv[mm] + alpha_lam * pv[mm];
-        }
-        rv[0] = rv[0] - c_prev;   // the constant-multiplier component measured last pass
-        stf<NL, VS>(L.r + o, rv);
-        stf<NL, VS>(L.lam + o, lv);
-      } else {
-        rv[0] = rv[0] - c_prev;
-#pragma unroll
-        for (int mm = 0; mm < NL; ++mm) rv[mm] = scale * rv[mm];
-        stf<NL, VS>(L.r + o, rv);
-        if (hsrc) {
-          A hv[NL];
-          ldf<NL, VS>(hsrc + o, hv);
-          stf<NL, VS>(hdst + o, hv);
-        }
-      }
-      acc_add(r0sum, rv[0]);
+      src(o, rv);
 #pragma unroll
       for (int mm = 0; mm < NL; ++mm) {
-        mad(rr, rv[mm], rv[mm]);
         C2* slot = &L.bufa[((r_ >> 1) * NL + mm) * N + i];
         if (r_ & 1) slot->y = fft_in(rv[mm]);
         else slot->x = fft_in(rv[mm]);
@@ -562,6 +580,7 @@ __device__ void columns(const LatCtx<K, MIXED>& L) {
     Lh.N = h;
     Lh.logn = L.logn - 1;
     Lh.pow2 = (h & (h - 1)) == 0;
+    Lh.r1 = dft_factor(h);
     Lh.tw = L.tw2;
     for (int item = blockIdx.x; item < 2 * NK; item += gridDim.x) {
       const int ki = item >> 1, par = item & 1;
@@ -614,11 +633,10 @@ __device__ void columns(const LatCtx<K, MIXED>& L) {
 }
 
 // Row pass, inverse: rebuild W = Y_even + i Y_odd over all k (Y[N-k] = conj Y[k]),
-// inverse FFT along i, z = the real / imaginary parts scaled by 1/N^2 in facet order.
-// Accumulates r.z_new into rz and, if with_old, r.z_old into rzo.
-template <int K, bool MIXED>
-__device__ void rows_inverse(const LatCtx<K, MIXED>& L, bool with_old, typename LatT<MIXED>::Acc& rz,
-                             typename LatT<MIXED>::Acc& rzo) {
+// inverse FFT along i, z = the real / imaginary parts scaled by 1/N^2 in facet order, stored and
+// given to fin(o, zv).
+template <int K, bool MIXED, typename Fin>
+__device__ __forceinline__ void rows_inverse(const LatCtx<K, MIXED>& L, Fin fin) {
   using T = LatT<MIXED>;
   using C2 = typename T::C2;
   using R = typename T::R;
@@ -664,17 +682,13 @@ __device__ void rows_inverse(const LatCtx<K, MIXED>& L, bool with_old, typename 
     for (int e = threadIdx.x; e < rows * N; e += blockDim.x) {
       const int r_ = e / N, i = e - r_ * N;
       const size_t o = base + size_t(e) * VS;
-      typename T::A rv[NL];
-      Z zv[NL], zo[NL];
-      ldf<NL, VS>(L.r + o, rv);
-      if (with_old) ldf<NL, VS>(L.z + o, zo);
+      Z zv[NL];
 #pragma unroll
       for (int mm = 0; mm < NL; ++mm) {
         const C2 v = res[((r_ >> 1) * NL + mm) * N + i];
         zv[mm] = Z((r_ & 1) ? v.y : v.x) * Z(scale);
-        if (with_old) mad(rzo, rv[mm], zo[mm]);
-        mad(rz, rv[mm], zv[mm]);
       }
+      fin(o, zv);
       stf<NL, VS>(L.z + o, zv);
     }
     __syncthreads();
@@ -799,108 +813,345 @@ __device__ __forceinline__ dacc red_load(const double* p, dacc) {
   return dacc{v.x, v.y};
 }
 
-// Block sum of v in every thread (all threads of the block call it).
-template <int N, typename Acc>
-__device__ __forceinline__ void block_acc(Acc (&v)[N]) {
-  __shared__ Acc part[kLatThreads / 32][N];
+// Grid sums of N per-thread partials, in the accumulator's own arithmetic and in a fixed order;
+// thread 0 of every block then takes them to fn(sums), whose results other threads read from shared
+// memory after the call. FP64 instructions occupy a quarter of an SM for 64 cycles a warp, so the
+// partials go through shared memory (one warp a sum, eight values a lane) instead of a butterfly
+// over every warp, and no scalar is formed by more than one warp. scr: N rows of kLatThreads.
+constexpr int kLatSums = 4;
+template <int N, typename Acc, typename F>
+__device__ __forceinline__ bool lat_reduce(const DevMesh& m, Barrier& bar, int slot0, const Acc (&v)[N],
+                                           Acc (*scr)[kLatThreads], F&& fn) {
+  static_assert(N <= kLatSums, "scratch rows");
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    const Acc ws = warp_acc(v[i]);
-    if (l == 0) part[w][i] = ws;
-  }
+  for (int i = 0; i < N; ++i) scr[i][threadIdx.x] = v[i];
   __syncthreads();
+  if (w < N) {
+    Acc b = scr[w][l];
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    Acc b = (l < kLatThreads / 32) ? part[l][i] : acc_zero(Acc{});
-    v[i] = warp_acc(b);
+    for (int k = 1; k < kLatThreads / 32; ++k) b = acc_combine(b, scr[w][l + 32 * k]);
+    b = warp_acc(b);
+    if (l == 0) red_store(&m.red[size_t(slot0 + w) * kMaxSolverBlocks + blockIdx.x], b);
   }
-  __syncthreads();
-}
-
-template <int N, typename Acc>
-__device__ bool lat_reduce(const DevMesh& m, int slot0, const Acc (&v)[N], Barrier& bar, double (&out)[N]) {
-  Acc b[N];
-#pragma unroll
-  for (int i = 0; i < N; ++i) b[i] = v[i];
-  block_acc<N>(b);
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int i = 0; i < N; ++i) red_store(&m.red[size_t(slot0 + i) * kMaxSolverBlocks + blockIdx.x], b[i]);
   if (!grid_sync(bar, m.stats)) return false;
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    Acc gsum = acc_zero(Acc{});
-    for (int k = threadIdx.x; k < gridDim.x; k += blockDim.x)
-      gsum = acc_combine(gsum, red_load(&m.red[size_t(slot0 + i) * kMaxSolverBlocks + k], Acc{}));
-    b[i] = gsum;
+  if (w < N) {
+    Acc g = acc_zero(Acc{});
+    for (int k = l; k < int(gridDim.x); k += 32)
+      g = acc_combine(g, red_load(&m.red[size_t(slot0 + w) * kMaxSolverBlocks + k], Acc{}));
+    g = warp_acc(g);
+    if (l == 0) scr[w][0] = g;
   }
-  block_acc<N>(b);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t[N];
 #pragma unroll
-  for (int i = 0; i < N; ++i) out[i] = acc_val(b[i]);
+    for (int i = 0; i < N; ++i) t[i] = acc_val(scr[i][0]);
+    fn(t);
+  }
+  __syncthreads();
   return true;
 }
 
-// Scalars of one PCG step, computed by thread 0 of each block (identically in every
-// block) and broadcast through shared memory.
+// Scalars of the solve: written by thread 0 of each block (identically in every block), read by
+// all after a block barrier.
 template <typename A>
 struct LatScal {
-  A alpha, alpha_lam, beta;
+  A alpha, alpha_lam, beta, mean, sigma;
+  double sum[2];
   int done, conv;
   double relres;
 };
 
+// ---- facet passes, a lane per value: LP lanes a facet (the last idle for three modes), lane i its
+// mode i. Against a thread a facet this needs a quarter of the registers, so that a thread keeps
+// the loads of several values in flight, and every access of a warp is a contiguous run.
+template <int NL>
+struct LatLanes {
+  static constexpr int LP = NL == 2 ? 2 : 4;
+};
+// fn(f, i, live): lanes past the last facet or mode run along with live = false.
+template <int NL, typename F>
+__device__ __forceinline__ void lat_facets(int nF, F&& fn) {
+  constexpr int LP = LatLanes<NL>::LP;
+  const int i0 = threadIdx.x & (LP - 1), i = i0 < NL ? i0 : NL - 1;
+  const int step = int(gridDim.x * blockDim.x) / LP;
+  const int f0 = int(blockIdx.x * blockDim.x + threadIdx.x) / LP;
+  const int w0 = int(blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / LP;
+#pragma unroll 2
+  for (int d = 0; w0 + d < nF; d += step) {
+    const int f = f0 + d;
+    fn(f < nF ? f : nF - 1, i, f < nF && i0 < NL);
+  }
+}
+
+__device__ __forceinline__ double shfl_lane(double v, int l, int w) { return __shfl_sync(0xffffffffu, v, l, w); }
+__device__ __forceinline__ dfl shfl_lane(dfl v, int l, int w) {
+  return dfl(__shfl_sync(0xffffffffu, v.hi, l, w), __shfl_sync(0xffffffffu, v.lo, l, w));
+}
+
+// an entry of the stencil classes' blocks, [class][5][NL][NL] in the vector type
+template <int NL>
+__device__ __forceinline__ double lat_entry(const double* S, int o, double) { return S[o]; }
+template <int NL>
+__device__ __forceinline__ dfl lat_entry(const float2* S, int o, dfl) { return to_dfl(S[o]); }
+
+// Mode i of g at facet f from the packed offsets of its two sides' condensation outputs
+// (m.lat_src: 2 x offset of the side's mode 0, + 1 where the side runs the facet backwards: odd
+// Legendre modes change sign).
+__device__ __forceinline__ double lat_g(const DevMesh& m, int f, int i, double) {
+  const int2 s = __ldg(&m.lat_src[f]);
+  const double a = __ldcg(&m.gl[(s.x >> 1) + i]), b = __ldcg(&m.gl[(s.y >> 1) + i]);
+  return ((s.x & i & 1) ? -a : a) + ((s.y & i & 1) ? -b : b);
+}
+__device__ __forceinline__ dfl lat_g(const DevMesh& m, int f, int i, dfl) {
+  const int2 s = __ldg(&m.lat_src[f]);
+  const dfl a = to_dfl(__ldcg(&m.gl_df[(s.x >> 1) + i])), b = to_dfl(__ldcg(&m.gl_df[(s.y >> 1) + i]));
+  return ((s.x & i & 1) ? -a : a) + ((s.y & i & 1) ? -b : b);
+}
+
+// The squares that give |r| and |g| are summed as FP32 pairs in the mixed form, of values scaled
+// by a power of two: 2^32 keeps values of 1e-28 to 1e9 within the FP32 exponents. Outside
+// [kLatSumMin, kLatSumMax] the sums say nothing, and lat_pcg (which scales by |g|) takes the solve.
+constexpr float kLatScale = 4294967296.f;
+constexpr double kLatSumMin = 1e-8, kLatSumMax = 1e36;
+__device__ __forceinline__ void add_square(double& a, double v) { a = fma(v, v, a); }
+__device__ __forceinline__ void add_square(dacc& a, dfl v) {
+  const float x = v.hi * kLatScale;
+  acc_add(a, dfl(x * x, 0.f));
+}
+
+// Iterative refinement. Returns 0 when the solve ended (st.conv, st.relres and it are set), -1 when
+// a barrier's wait ran out, 1 when lat_pcg has to take the solve from its start, 2 when it has to
+// go on from lam (the history has moved then).
 template <int K, bool MIXED>
-__global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveArgs a) {
+__device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, const LatCtx<K, MIXED>& L,
+                                          const typename LatT<MIXED>::V* S, Barrier& bar,
+                                          LatScal<typename LatT<MIXED>::A>& sc,
+                                          typename LatT<MIXED>::Acc (*scr)[kLatThreads], int& it) {
   using T = LatT<MIXED>;
-  using C2 = typename T::C2;
-  using R = typename T::R;
+  using V = typename T::V;
+  using A = typename T::A;
+  using Acc = typename T::Acc;
+  using Z = typename T::Z;
+  constexpr int NL = K + 1, VS = LatCtx<K, MIXED>::VS, LP = LatLanes<NL>::LP;
+  const int nF = m.n_facet;
+  const A warm = A(a.warm_scale), hc1 = A(a.c1), hc2 = A(a.c2);
+  V* hist1 = static_cast<V*>(a.hist1);
+  V* hist2 = static_cast<V*>(a.hist2);
+  V* hnew = static_cast<V*>(a.hist_new);
+  const bool use2 = a.c2 != 0.0, lam0 = hist1 || a.warm_scale != 0.0;
+  // (S x)_i from the lanes' x of the five facets
+  auto product = [&](const A (&x)[5], int cls, int i) {
+    Acc acc = acc_zero(Acc{});
+    const V* row = S + (cls * 5 * NL + i) * NL;
+#pragma unroll
+    for (int b = 0; b < 5; ++b)
+#pragma unroll
+      for (int j = 0; j < NL; ++j) mad(acc, lat_entry<NL>(row, b * NL * NL + j, A{}), shfl_lane(x[b], j, LP));
+    return fin(acc);
+  };
+  // g from both sides of every facet, the warm start lam0 = c1 hist1 + c2 hist2 (or warm_scale lam,
+  // or zero) and r = g - S lam0 in one pass: a facet forms its neighbours' lam0 from the history
+  // with the same operations as they do, so that lam0 is the same bits wherever it is formed
+  Acc s4[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) s4[i] = acc_zero(Acc{});
+  lat_facets<NL>(nF, [&](int f, int i, bool live) {
+    const size_t o = size_t(f) * VS + i;
+    const A g = lat_g(m, f, i, A{});
+    A r = g;
+    if (lam0) {
+      const int4 nb = __ldg(reinterpret_cast<const int4*>(m.facet_nbr) + f);
+      const int n5[5] = {f, nb.x, nb.y, nb.z, nb.w};
+      const int cls = __ldg(&m.facet_stencil[f]);
+      const V* src = hist1 ? hist1 : L.lam;
+      A x[5], x2[5];
+#pragma unroll
+      for (int b = 0; b < 5; ++b) x[b] = ldv(src + size_t(n5[b]) * VS + i);
+      if (hist1 && use2) {
+#pragma unroll
+        for (int b = 0; b < 5; ++b) x2[b] = ldv(hist2 + size_t(n5[b]) * VS + i);
+#pragma unroll
+        for (int b = 0; b < 5; ++b) x[b] = hc1 * x[b] + hc2 * x2[b];
+      } else {
+        const A c = hist1 ? hc1 : warm;
+#pragma unroll
+        for (int b = 0; b < 5; ++b) x[b] = c * x[b];
+      }
+      r = g - product(x, cls, i);
+      if (hist1 && live) stv(L.lam + o, x[0]);
+    }
+    if (!live) return;
+    stv(L.r + o, r);
+    add_square(s4[0], g);
+    add_square(s4[1], r);
+    if (i == 0) {
+      acc_add(s4[2], g);
+      acc_add(s4[3], r);
+    }
+  });
+  // thread 0's own: the squared norms (scaled), without the constant-multiplier component
+  double stop2 = 0.0, floor2 = 0.0, gg = 0.0, rr = 0.0;
+  const double f2 = MIXED ? double(kLatScale) * double(kLatScale) : 1.0;
+  if (!lat_reduce<4>(m, bar, 4, s4, scr, [&](const double (&t)[4]) {
+        const double inv = 1.0 / double(nF);
+        gg = t[0] - t[2] * t[2] * f2 * inv;
+        rr = fmax(t[1] - t[3] * t[3] * f2 * inv, 0.0);
+        stop2 = a.rtol * a.rtol * gg;
+        floor2 = a.floor_rtol * a.floor_rtol * gg;
+        sc.mean = A(t[3] * inv);
+        sc.conv = 0;
+        sc.done = 0;
+        if (!(stop2 >= (MIXED ? kLatSumMin * 1e-22 : 1e-280) && gg <= (MIXED ? kLatSumMax : 1e280) && rr <= 1e280)) {
+          sc.done = 3;   // out of range, zero or not finite
+        } else if (rr <= stop2) {
+          sc.done = sc.conv = 1;
+          sc.relres = sqrt(rr / gg);
+        }
+      }))
+    return -1;
+  if (sc.done == 3) return 1;
+  const bool at_once = sc.done != 0;
+  while (!sc.done) {
+    const bool first = it == 0;
+    // z = B r. The constant multiplier is in the kernel of S and of B: refinement cannot reduce r's
+    // component along it, which only rounding feeds; it is left out of the norms and subtracted
+    // from r in the next update.
+    rows_forward<K, MIXED>(L, [](size_t, A (&)[NL]) {});
+    if (!grid_sync(bar, m.stats)) return -1;
+    columns<K, MIXED>(L);
+    if (!grid_sync(bar, m.stats)) return -1;
+    // lam += z; the first pass moves the history down one slot, every pass stores the new entry
+    const A mean = sc.mean;
+    rows_inverse<K, MIXED>(L, [&](size_t o, const Z (&zv)[NL]) {
+      A lv[NL];
+      if (first && !lam0) {
+#pragma unroll
+        for (int j = 0; j < NL; ++j) lv[j] = as_a(zv[j]);
+      } else {
+        ldf<NL, VS>(L.lam + o, lv);
+#pragma unroll
+        for (int j = 0; j < NL; ++j) lv[j] = (first && !hist1 ? warm * lv[j] : lv[j]) + as_a(zv[j]);
+      }
+      stf<NL, VS>(L.lam + o, lv);
+      if (first && hist1) {
+        A hv[NL];
+        ldf<NL, VS>(hist1 + o, hv);
+        stf<NL, VS>(hist2 + o, hv);
+      }
+      if (hnew) stf<NL, VS>(hnew + o, lv);
+    });
+    if (!grid_sync(bar, m.stats)) return -1;
+    // r -= S z and its constant component
+    Acc s2[2] = {acc_zero(Acc{}), acc_zero(Acc{})};
+    lat_facets<NL>(nF, [&](int f, int i, bool live) {
+      const size_t o = size_t(f) * VS + i;
+      const int4 nb = __ldg(reinterpret_cast<const int4*>(m.facet_nbr) + f);
+      const int n5[5] = {f, nb.x, nb.y, nb.z, nb.w};
+      const int cls = __ldg(&m.facet_stencil[f]);
+      A r = ldv(L.r + o);
+      Z z[5][NL];
+#pragma unroll
+      for (int b = 0; b < 5; ++b) ldf<NL, VS>(L.z + size_t(n5[b]) * VS, z[b]);
+      Acc acc = acc_zero(Acc{});
+      const V* row = S + (cls * 5 * NL + i) * NL;
+#pragma unroll
+      for (int b = 0; b < 5; ++b)
+#pragma unroll
+        for (int j = 0; j < NL; ++j) mad(acc, lat_entry<NL>(row, b * NL * NL + j, A{}), z[b][j]);
+      r = r - fin(acc);
+      if (i == 0) r = r - mean;
+      if (!live) return;
+      stv(L.r + o, r);
+      add_square(s2[0], r);
+      if (i == 0) acc_add(s2[1], r);
+    });
+    ++it;
+    const int n = it;
+    if (!lat_reduce<2>(m, bar, n & 1 ? 0 : 2, s2, scr, [&](const double (&t)[2]) {
+          const double inv = 1.0 / double(nF), prev = rr;
+          rr = fmax(t[0] - t[1] * t[1] * f2 * inv, 0.0);
+          sc.mean = A(t[1] * inv);
+          sc.relres = sqrt(rr / gg);
+          if (!isfinite(rr)) {
+            if (blockIdx.x == 0) atomicOr(&m.stats->flags, kFlagNonFinite);
+            sc.done = 1;
+          } else if (rr <= stop2 || (rr <= floor2 && rr > 0.25 * prev)) {
+            // converged, or at the rounding floor (an iteration no longer halves the residual)
+            sc.done = sc.conv = 1;
+          } else if (n >= a.maxit) {
+            sc.done = 1;
+          } else if (!(rr <= 0.01 * prev)) {
+            sc.done = 3;
+          }
+        }))
+      return -1;
+  }
+  if (sc.done == 3) return 2;
+  if (at_once) {   // no pass has moved the history or stored lam
+    const int gsz = gridDim.x * blockDim.x;
+    for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nF; f += gsz) {
+      const size_t o = size_t(f) * VS;
+      A lv[NL], hv[NL];
+      if (hist1) {
+        ldf<NL, VS>(hist1 + o, hv);
+        stf<NL, VS>(hist2 + o, hv);
+      }
+      if (!hist1) {
+#pragma unroll
+        for (int j = 0; j < NL; ++j) lv[j] = A(0);
+        if (lam0) {
+          ldf<NL, VS>(L.lam + o, lv);
+#pragma unroll
+          for (int j = 0; j < NL; ++j) lv[j] = warm * lv[j];
+        }
+        stf<NL, VS>(L.lam + o, lv);
+      } else {
+        ldf<NL, VS>(L.lam + o, lv);
+      }
+      if (hnew) stf<NL, VS>(hnew + o, lv);
+    }
+  }
+  return 0;
+}
+
+// lat_reduce with the sums in every thread
+template <int N, typename Acc, typename A>
+__device__ __forceinline__ bool lat_sums(const DevMesh& m, Barrier& bar, int slot0, const Acc (&v)[N],
+                                         Acc (*scr)[kLatThreads], LatScal<A>& sc, double (&out)[N]) {
+  if (!lat_reduce<N>(m, bar, slot0, v, scr, [&](const double (&t)[N]) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) sc.sum[i] = t[i];
+      }))
+    return false;
+#pragma unroll
+  for (int i = 0; i < N; ++i) out[i] = sc.sum[i];
+  return true;
+}
+
+__device__ __forceinline__ bool grid_reduce_pair(const DevMesh& m, Barrier& bar, int slot0, double a, double b,
+                                                 double (&out)[2]) {
+  out[0] = a;
+  out[1] = b;
+  return grid_reduce<2>(m, slot0, out, bar);
+}
+
+// The solve as PCG preconditioned by B, on the system scaled by the size of g: for systems where
+// refinement gains too little, or whose size is outside the range of its sums. Returns false when
+// a barrier's wait ran out.
+template <int K, bool MIXED>
+__device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const LatCtx<K, MIXED>& L,
+                                     typename LatT<MIXED>::V* p, Barrier& bar, LatScal<typename LatT<MIXED>::A>& sc,
+                                     typename LatT<MIXED>::Acc (*scr)[kLatThreads], int& it) {
+  using T = LatT<MIXED>;
   using V = typename T::V;
   using A = typename T::A;
   using Acc = typename T::Acc;
   using Z = typename T::Z;
   constexpr int NL = K + 1, VS = LatCtx<K, MIXED>::VS;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ LatScal<A> sc;
-  LatCtx<K, MIXED> L;
-  L.N = m.lat_N;
-  L.logn = m.lat_logn;
-  L.NK = L.N / 2 + 1;
-  L.ntj = (L.N + kLatTJ - 1) / kLatTJ;
-  L.pow2 = (L.N & (L.N - 1)) == 0;
-  L.grp = m.lat_grp;
-  L.tw = reinterpret_cast<C2*>(smem_raw);
-  L.bufa = L.tw + L.N;
-  L.scr = L.bufa + m.lat_bufsz;
-  L.X = reinterpret_cast<C2*>(m.lat_x);
-  L.S = reinterpret_cast<const C2*>(m.lat_sinv);
-  L.split = m.lat_split != 0;
-  L.tw2 = reinterpret_cast<C2*>(smem_raw) + m.lat_tw2_off;
-  L.X2 = reinterpret_cast<C2*>(m.lat_x2);
-  V* p;
-  if constexpr (MIXED) {
-    L.lam = m.lam_df;
-    L.g = m.lv_g;
-    L.r = m.lv_r;
-    L.q = m.lv_q;
-    L.z = m.lv_z;
-    p = m.lv_p;
-  } else {
-    L.lam = m.lam;
-    L.g = m.g;
-    L.r = m.r;
-    L.q = m.q;
-    L.z = m.z;
-    p = m.pa;
-  }
-  for (int t = threadIdx.x; t < L.N; t += blockDim.x) L.tw[t] = C2{R(m.lat_tw[2 * t]), R(m.lat_tw[2 * t + 1])};
-  if (L.split)
-    for (int t = threadIdx.x; t < L.N / 2; t += blockDim.x)
-      L.tw2[t] = C2{R(m.lat_tw[4 * t]), R(m.lat_tw[4 * t + 1])};
-  __syncthreads();
   const int nF = m.n_facet;
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
-  Barrier bar(m.bar);
   // g from both sides of every facet and the warm start lam0. With a history (the same stage
   // of earlier steps), lam0 = c1 hist1 + c2 hist2 and r = g - S lam0 in the same pass (every
   // facet forms its neighbours' lam0 from the history, which this launch only reads until
@@ -944,8 +1195,8 @@ __global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveAr
   }
   double gg[2];
   {
-    const double gv2[2] = {ga, acc_val(g0)};
-    if (!lat_reduce<2>(m, 4, gv2, bar, gg)) return;
+    // FP64 sums (the squares of any g fit), through the double slots of the scratch
+    if (!grid_reduce_pair(m, bar, 4, ga, acc_val(g0), gg)) return false;
   }
   const double c0 = gg[1] / double(nF);
   const double gnorm0 = sqrt(fmax(gg[0] - gg[1] * gg[1] / double(nF), 0.0));
@@ -961,7 +1212,6 @@ __global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveAr
   // once an iteration no longer halves the residual and it is below floor_rtol, the
   // solve is accepted there
   const double floor2 = (a.floor_rtol * gnorm) * (a.floor_rtol * gnorm);
-  int it = 0;
   bool conv = false;
   double relres = 0.0;
   if (gnorm == 0.0) {
@@ -991,7 +1241,7 @@ __global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveAr
         for (int j = 0; j < NL; ++j) y[j] = gv[j] - y[j];
         stf<NL, VS>(L.r + o, y);
       }
-      if (!grid_sync(bar, m.stats)) return;
+      if (!grid_sync(bar, m.stats)) return false;
     }
     // z = M r
     // The constant multiplier is in the kernel of S and of the preconditioner, so PCG cannot
@@ -1001,25 +1251,47 @@ __global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveAr
     // The first row pass scales r by sigma and removes the constant component of g from it:
     // r = sigma (g - c0 1 - S lam0).
     Acc rra[2] = {acc_zero(Acc{}), acc_zero(Acc{})};
-    rows_forward<K, MIXED>(L, false, A(0), A(0), A(c0), p, rra[0], rra[1], A(sigma), hist1, hist2);
+    {
+      const A cm = A(c0), scale = A(sigma);
+      rows_forward<K, MIXED>(L, [&](size_t o, A (&rv)[NL]) {
+        rv[0] = rv[0] - cm;
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+          rv[j] = scale * rv[j];
+          mad(rra[0], rv[j], rv[j]);
+        }
+        acc_add(rra[1], rv[0]);
+        stf<NL, VS>(L.r + o, rv);
+        if (hist1) {
+          A hv[NL];
+          ldf<NL, VS>(hist1 + o, hv);
+          stf<NL, VS>(hist2 + o, hv);
+        }
+      });
+    }
     double rr[2];
-    if (!lat_reduce<2>(m, 6, rra, bar, rr)) return;
+    if (!lat_sums<2>(m, bar, 6, rra, scr, sc, rr)) return false;
     double cmode = rr[1] / double(nF);
     rr[0] = fmax(rr[0] - rr[1] * rr[1] / double(nF), 0.0);
     columns<K, MIXED>(L);
-    if (!grid_sync(bar, m.stats)) return;
+    if (!grid_sync(bar, m.stats)) return false;
     Acc rza[2] = {acc_zero(Acc{}), acc_zero(Acc{})};
-    rows_inverse<K, MIXED>(L, false, rza[0], rza[1]);
+    rows_inverse<K, MIXED>(L, [&](size_t o, const Z (&zv)[NL]) {
+      A rv[NL];
+      ldf<NL, VS>(L.r + o, rv);
+#pragma unroll
+      for (int j = 0; j < NL; ++j) mad(rza[0], rv[j], zv[j]);
+    });
     double rz[2];
     {
       const Acc rz1[1] = {rza[0]};
       double rzt[1];
-      if (!lat_reduce<1>(m, 1, rz1, bar, rzt)) return;
+      if (!lat_sums<1>(m, bar, 1, rz1, scr, sc, rzt)) return false;
       rz[0] = rzt[0];
     }
     double rho = rz[0], rrv = rr[0];
     double beta = 0.0;
-    for (;; ++it) {
+    for (int n = 0;; ++it, ++n) {
       // convergence and the scalars of this step, once per block
       if (threadIdx.x == 0) {
         sc.done = 0;
@@ -1051,22 +1323,22 @@ __global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveAr
         Z zz[NL];
         spmv_lat<NL, VS, MIXED>(m, f, L.z, Z{}, y);
         ldf<NL, VS>(L.z + o, zz);
-        if (it > 0) {
+        if (n > 0) {
           ldf<NL, VS>(p + o, pv);
           ldf<NL, VS>(L.q + o, qv);
         }
 #pragma unroll
         for (int j = 0; j < NL; ++j) {
           const A zv = as_a(zz[j]);
-          pv[j] = (it == 0) ? zv : zv + bt * pv[j];
-          qv[j] = (it == 0) ? y[j] : y[j] + bt * qv[j];
+          pv[j] = (n == 0) ? zv : zv + bt * pv[j];
+          qv[j] = (n == 0) ? y[j] : y[j] + bt * qv[j];
           mad(pqa[0], pv[j], qv[j]);
         }
         stf<NL, VS>(p + o, pv);
         stf<NL, VS>(L.q + o, qv);
       }
       double pq[1];
-      if (!lat_reduce<1>(m, 0, pqa, bar, pq)) return;
+      if (!lat_sums<1>(m, bar, 0, pqa, scr, sc, pq)) return false;
       if (threadIdx.x == 0) {
         sc.done = 0;
         if (!(pq[0] > 0.0)) {
@@ -1083,8 +1355,27 @@ __global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveAr
       // r -= alpha q, lam += alpha p, and the forward row pass of z = M r
       rra[0] = acc_zero(Acc{});
       rra[1] = acc_zero(Acc{});
-      rows_forward<K, MIXED>(L, true, sc.alpha, sc.alpha_lam, A(cmode), p, rra[0], rra[1], A(1), nullptr, nullptr);
-      if (!lat_reduce<2>(m, 6, rra, bar, rr)) return;
+      {
+        const A al = sc.alpha, all = sc.alpha_lam, cm = A(cmode);
+        rows_forward<K, MIXED>(L, [&](size_t o, A (&rv)[NL]) {
+          A qv[NL], lv[NL], pv[NL];
+          ldf<NL, VS>(L.q + o, qv);
+          ldf<NL, VS>(L.lam + o, lv);
+          ldf<NL, VS>(p + o, pv);
+#pragma unroll
+          for (int j = 0; j < NL; ++j) {
+            rv[j] = rv[j] - al * qv[j];
+            lv[j] = lv[j] + all * pv[j];
+          }
+          rv[0] = rv[0] - cm;   // the constant-multiplier component measured last pass
+#pragma unroll
+          for (int j = 0; j < NL; ++j) mad(rra[0], rv[j], rv[j]);
+          acc_add(rra[1], rv[0]);
+          stf<NL, VS>(L.r + o, rv);
+          stf<NL, VS>(L.lam + o, lv);
+        });
+      }
+      if (!lat_sums<2>(m, bar, 6, rra, scr, sc, rr)) return false;
       cmode = rr[1] / double(nF);
       const double rr_prev = rrv;
       rrv = fmax(rr[0] - rr[1] * rr[1] / double(nF), 0.0);
@@ -1107,25 +1398,123 @@ __global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveAr
         break;
       }
       columns<K, MIXED>(L);
-      if (!grid_sync(bar, m.stats)) return;
+      if (!grid_sync(bar, m.stats)) return false;
       rza[0] = acc_zero(Acc{});
       rza[1] = acc_zero(Acc{});
-      rows_inverse<K, MIXED>(L, true, rza[0], rza[1]);
-      if (!lat_reduce<2>(m, 1, rza, bar, rz)) return;
+      rows_inverse<K, MIXED>(L, [&](size_t o, const Z (&zv)[NL]) {
+        A rv[NL];
+        Z zo[NL];
+        ldf<NL, VS>(L.r + o, rv);
+        ldf<NL, VS>(L.z + o, zo);
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+          mad(rza[1], rv[j], zo[j]);
+          mad(rza[0], rv[j], zv[j]);
+        }
+      });
+      if (!lat_sums<2>(m, bar, 1, rza, scr, sc, rz)) return false;
       // flexible (Polak-Ribiere) beta: the FP32 preconditioner is symmetric only up to rounding
       beta = (rz[0] - rz[1]) / rho;
       rho = rz[0];
     }
+  }
+  if (a.hist_new) {
+    V* hnew = static_cast<V*>(a.hist_new);
+    if (!grid_sync(bar, m.stats)) return false;
+    for (int f = gtid; f < nF; f += gsz) {
+      A lv[NL];
+      ldf<NL, VS>(L.lam + size_t(f) * VS, lv);
+      stf<NL, VS>(hnew + size_t(f) * VS, lv);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    sc.conv = conv ? 1 : 0;
+    sc.relres = relres;
+  }
+  return true;
+}
+
+// One solve: refinement, and PCG where it does not do.
+template <int K, bool MIXED>
+__global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveArgs a) {
+  using T = LatT<MIXED>;
+  using C2 = typename T::C2;
+  using R = typename T::R;
+  using V = typename T::V;
+  using A = typename T::A;
+  using Acc = typename T::Acc;
+  constexpr int NL = K + 1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ LatScal<A> sc;
+  __shared__ __align__(16) V stencil[kLatStencils * 5 * NL * NL];
+  LatCtx<K, MIXED> L;
+  L.N = m.lat_N;
+  L.logn = m.lat_logn;
+  L.NK = L.N / 2 + 1;
+  L.ntj = (L.N + kLatTJ - 1) / kLatTJ;
+  L.pow2 = (L.N & (L.N - 1)) == 0;
+  L.r1 = dft_factor(L.N);
+  L.grp = m.lat_grp;
+  L.tw = reinterpret_cast<C2*>(smem_raw);
+  L.bufa = L.tw + L.N;
+  L.scr = L.bufa + m.lat_bufsz;
+  // the reductions run while the transform buffers are free
+  Acc(*scr)[kLatThreads] = reinterpret_cast<Acc(*)[kLatThreads]>(L.bufa);
+  L.X = reinterpret_cast<C2*>(m.lat_x);
+  L.S = reinterpret_cast<const C2*>(m.lat_sinv);
+  L.split = m.lat_split != 0;
+  L.tw2 = reinterpret_cast<C2*>(smem_raw) + m.lat_tw2_off;
+  L.X2 = reinterpret_cast<C2*>(m.lat_x2);
+  V* p;
+  if constexpr (MIXED) {
+    L.lam = m.lam_df;
+    L.g = m.lv_g;
+    L.r = m.lv_r;
+    L.q = m.lv_q;
+    L.z = m.lv_z;
+    p = m.lv_p;
+  } else {
+    L.lam = m.lam;
+    L.g = m.g;
+    L.r = m.r;
+    L.q = m.q;
+    L.z = m.z;
+    p = m.pa;
+  }
+  for (int t = threadIdx.x; t < L.N; t += blockDim.x) L.tw[t] = C2{R(m.lat_tw[2 * t]), R(m.lat_tw[2 * t + 1])};
+  if (L.split)
+    for (int t = threadIdx.x; t < L.N / 2; t += blockDim.x)
+      L.tw2[t] = C2{R(m.lat_tw[4 * t]), R(m.lat_tw[4 * t + 1])};
+  const V* S;   // (a uniform torus has three classes; more are read from global memory)
+  if constexpr (MIXED) S = m.st_blk_df;
+  else S = m.st_blk;
+  if (m.n_stencil <= kLatStencils) {
+    for (int t = threadIdx.x; t < m.n_stencil * 5 * NL * NL; t += blockDim.x) stencil[t] = __ldg(&S[t]);
+    S = stencil;
+  }
+  __syncthreads();
+  Barrier bar(m.bar);
+  int it = 0;
+  const int how = lat_refine<K, MIXED>(m, a, L, S, bar, sc, scr, it);
+  if (how < 0) return;
+  if (how > 0) {
+    SolveArgs b = a;
+    if (how == 2) {
+      b.hist1 = nullptr;
+      b.warm_scale = 1.0;
+    }
+    if (!grid_sync(bar, m.stats) || !lat_pcg<K, MIXED>(m, b, L, p, bar, sc, scr, it)) return;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     DevStats* st = m.stats;
     st->last_iters = it;
     st->total_iters += it;
     st->solves += 1;
-    st->last_relres = relres;
+    st->last_relres = sc.relres;
     st->last_sweeps = 1;
     st->total_sweeps += 1;
-    if (!conv) atomicOr(&st->flags, kFlagNotConverged);
+    if (!sc.conv) atomicOr(&st->flags, kFlagNotConverged);
   }
 }
 

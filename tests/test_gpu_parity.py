@@ -610,3 +610,25 @@ def test_multilevel_solver_forms_match_the_host_v_cycle(g, N, k, walls, perturb,
     r[:, 0] -= r[:, 0].mean()
     host = g.host_multilevel(vid, X, k, r=r.reshape(1, -1))["z"][0]
     assert rel(mesh.test_multilevel_apply(r.ravel()), host) < (1e-5 if precision else 1e-12)
+
+
+@pytest.mark.parametrize("N,k,precision", [(1, 2, 0), (2, 3, 1), (6, 1, 1), (13, 2, 1), (35, 1, 0), (66, 2, 1), (77, 3, 1),
+                                           (127, 1, 1)])
+@pytest.mark.parametrize("size", [1.0, 1e-14, 1e7])
+def test_lattice_solver_forms_match_block_jacobi(g, N, k, precision, size):
+    # the lattice solver's transforms (primes, two factors, the split column pass at 66) and both
+    # of its methods: refinement, and PCG where the size of g is outside the range of refinement's
+    # sums (1e-14, 1e7 in the mixed form). The block-Jacobi solver, which shares neither, meets the
+    # same rtol, so that the projections differ by rtol times sqrt(cond(S)) (below 1e3 N), with a
+    # factor of ten to spare; steps on top run the warm starts from the history
+    vid, X = synth.split_square_mesh(N, L=1.0)
+    v = size * random_lattice(2 * N * N, k, N)
+    out = []
+    for pc in (g.PRECOND_AUTO, g.PRECOND_BLOCK_JACOBI):
+        mesh = g.DGMesh(vid, X, k, 0.0, precision=precision, precond=pc)
+        assert mesh.solver_stats()["preconditioner"] == ("lattice FFT" if pc == g.PRECOND_AUTO else "block Jacobi")
+        mesh.set_velocity(v)
+        mesh.project_divfree()
+        mesh.rk3_step(1e-3 / (N * size), 3)
+        out.append(mesh.get_velocity())
+    assert rel(out[0], out[1]) < 1e-13 * 1e3 * N * 10 / 1e3
