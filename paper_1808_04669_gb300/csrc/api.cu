@@ -477,7 +477,7 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
       if ((rc = upload(M, &d.inflow_q, uq)) || (rc = upload(M, &d.inflow_d, dm))) return cleanup(rc);
     }
   }
-  if (d.elem_df && d.n_class <= dgdf::kDnClasses) {
+  if (d.n_class <= dgdf::kDnClasses) {
     // normal derivatives of the basis at the facet points, per class
     const int nqf = ref.nqf, ns = hm.ns;
     std::vector<double> dn(size_t(d.n_class) * 3 * nqf * ns);
@@ -493,65 +493,68 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
           }
       }
     }
-    // paired image for k_stage_df2: rows of ns values as ceil(ns/2) pairs
-    // {hi_j, hi_j+1, lo_j, lo_j+1} (a missing j+1 is 0), in the order of PairTables<K>
-    const int ns2 = (ns + 1) / 2, nq = ref.nq;
-    std::vector<float> pt;
-    auto split = [](double v, float& h, float& l) {
-      h = float(v);
-      l = float(v - double(h));
-    };
-    // value (r, j) = src[r * rstride + j * jstride]
-    auto rows = [&](const double* src, int nrow, int rstride, int jstride) {
-      for (int r = 0; r < nrow; ++r)
-        for (int jp = 0; jp < ns2; ++jp) {
-          float h0, l0, h1 = 0.f, l1 = 0.f;
-          const int j = 2 * jp;
-          split(src[size_t(r) * rstride + size_t(j) * jstride], h0, l0);
-          if (j + 1 < ns) split(src[size_t(r) * rstride + size_t(j + 1) * jstride], h1, l1);
-          pt.insert(pt.end(), {h0, h1, l0, l1});
-        }
-    };
-    rows(ref.vphi.data(), nq, ns, 1);                  // vphi[q][j]
-    rows(ref.vdphi.data(), nq, 2 * ns, 2);             // d/dxi1 psi_j at q
-    rows(ref.vdphi.data() + 1, nq, 2 * ns, 2);         // d/dxi2
-    rows(ref.fphi.data(), 3 * nqf, ns, 1);             // fphi[e][q][j]
-    {
-      std::vector<double> dnfull(size_t(dgdf::kDnClasses) * 3 * nqf * ns, 0.0);
-      std::copy(dn.begin(), dn.end(), dnfull.begin());
-      rows(dnfull.data(), dgdf::kDnClasses * 3 * nqf, ns, 1);
-    }
-    for (int q = 0; q < nq; ++q) {
-      float h, l;
-      split(ref.vw[q], h, l);
-      pt.push_back(h);
-      pt.push_back(l);
-    }
-    for (int q = 0; q < nqf; ++q) {
-      float h, l;
-      split(ref.fw[q], h, l);
-      pt.push_back(h);
-      pt.push_back(l);
-    }
-    while (pt.size() % 4) pt.push_back(0.f);
-    d.ptab_words = int(pt.size() / 4);
-    // class operators, pairs of consecutive columns
-    auto pairs = [&](const std::vector<double>& Mx, int nrow) {
-      std::vector<float> out;
-      const int nc2 = nd / 2;
-      for (int c = 0; c < d.n_class; ++c)
+    if ((rc = upload(M, &d.dn64, dn))) return cleanup(rc);
+    if (d.elem_df) {
+      // paired image for k_stage_df2: rows of ns values as ceil(ns/2) pairs
+      // {hi_j, hi_j+1, lo_j, lo_j+1} (a missing j+1 is 0), in the order of PairTables<K>
+      const int ns2 = (ns + 1) / 2, nq = ref.nq;
+      std::vector<float> pt;
+      auto split = [](double v, float& h, float& l) {
+        h = float(v);
+        l = float(v - double(h));
+      };
+      // value (r, j) = src[r * rstride + j * jstride]
+      auto rows = [&](const double* src, int nrow, int rstride, int jstride) {
         for (int r = 0; r < nrow; ++r)
-          for (int jp = 0; jp < nc2; ++jp) {
-            float h0, l0, h1, l1;
-            split(Mx[(size_t(c) * nrow + r) * nd + 2 * jp], h0, l0);
-            split(Mx[(size_t(c) * nrow + r) * nd + 2 * jp + 1], h1, l1);
-            out.insert(out.end(), {h0, h1, l0, l1});
+          for (int jp = 0; jp < ns2; ++jp) {
+            float h0, l0, h1 = 0.f, l1 = 0.f;
+            const int j = 2 * jp;
+            split(src[size_t(r) * rstride + size_t(j) * jstride], h0, l0);
+            if (j + 1 < ns) split(src[size_t(r) * rstride + size_t(j + 1) * jstride], h1, l1);
+            pt.insert(pt.end(), {h0, h1, l0, l1});
           }
-      return out;
-    };
-    std::vector<float> p2 = pairs(P, nd), g2 = pairs(G, L3);
-    if ((rc = upload_f4(M, &d.ptab, pt)) || (rc = upload_f4(M, &d.P2, p2)) || (rc = upload_f4(M, &d.G2, g2)))
-      return cleanup(rc);
+      };
+      rows(ref.vphi.data(), nq, ns, 1);                  // vphi[q][j]
+      rows(ref.vdphi.data(), nq, 2 * ns, 2);             // d/dxi1 psi_j at q
+      rows(ref.vdphi.data() + 1, nq, 2 * ns, 2);         // d/dxi2
+      rows(ref.fphi.data(), 3 * nqf, ns, 1);             // fphi[e][q][j]
+      {
+        std::vector<double> dnfull(size_t(dgdf::kDnClasses) * 3 * nqf * ns, 0.0);
+        std::copy(dn.begin(), dn.end(), dnfull.begin());
+        rows(dnfull.data(), dgdf::kDnClasses * 3 * nqf, ns, 1);
+      }
+      for (int q = 0; q < nq; ++q) {
+        float h, l;
+        split(ref.vw[q], h, l);
+        pt.push_back(h);
+        pt.push_back(l);
+      }
+      for (int q = 0; q < nqf; ++q) {
+        float h, l;
+        split(ref.fw[q], h, l);
+        pt.push_back(h);
+        pt.push_back(l);
+      }
+      while (pt.size() % 4) pt.push_back(0.f);
+      d.ptab_words = int(pt.size() / 4);
+      // class operators, pairs of consecutive columns
+      auto pairs = [&](const std::vector<double>& Mx, int nrow) {
+        std::vector<float> out;
+        const int nc2 = nd / 2;
+        for (int c = 0; c < d.n_class; ++c)
+          for (int r = 0; r < nrow; ++r)
+            for (int jp = 0; jp < nc2; ++jp) {
+              float h0, l0, h1, l1;
+              split(Mx[(size_t(c) * nrow + r) * nd + 2 * jp], h0, l0);
+              split(Mx[(size_t(c) * nrow + r) * nd + 2 * jp + 1], h1, l1);
+              out.insert(out.end(), {h0, h1, l0, l1});
+            }
+        return out;
+      };
+      std::vector<float> p2 = pairs(P, nd), g2 = pairs(G, L3);
+      if ((rc = upload_f4(M, &d.ptab, pt)) || (rc = upload_f4(M, &d.P2, p2)) || (rc = upload_f4(M, &d.G2, g2)))
+        return cleanup(rc);
+    }
   }
   if (d.elem_df && d.ptab && d.n_class <= 2) {
     // tensor-core recovery: per class, tiles of 128 triangles, and the class operator

@@ -96,6 +96,7 @@ struct DevMesh {
   // P2 [n_class][nd][nd/2] and G2 [n_class][3(k+1)][nd/2] (pairs of consecutive columns:
   // both leading words, then both trailing words)
   const float4 *ptab, *P2, *G2;
+  const double* dn64;   // the same normal derivatives in FP64, [n_class][3][nqf][ns] (NULL: more classes)
   int ptab_words;   // float4 words of ptab
   // facet-system stencil
   const int32_t *facet_nbr, *facet_stencil, *facet_tri;

@@ -1,5 +1,5 @@
-// Element kernels: stage residual + condensation (K1-K3), recovery (K5), pressure,
-// lattice conversion and diagnostics. One thread per triangle; the reference
+// Element kernels: recovery (K5), pressure, lattice conversion and diagnostics (the FP64 stage kernel
+// is in k_stage64.cu, the mixed form's in k_stage_df.cu). One thread per triangle; the reference
 // tables sit in shared memory and are read as warp broadcasts.
 #include "device.cuh"
 #include "dfloat.cuh"
@@ -7,398 +7,6 @@
 #include "ktables.cuh"
 
 namespace dgdf {
-
-// Convective term of eq. (7) on boundary facet e of triangle t when it is an inflow or
-// outflow facet (Sec. 2.5): the flux (u.n) u^up with u.n the average of the interior trace and
-// the exterior state, which is u_in on an inflow facet (stored at the facet points in the
-// canonical direction: our point q is point q there when the triangle runs the facet the
-// canonical way, else point NQF-1-q) and the interior trace on an outflow facet. The viscous
-// form has no boundary terms (natural conditions on every boundary facet).
-template <int K, typename R>
-__device__ void boundary_flux(const DevMesh& m, const SmemTables<K, R>& T, int t, int e, const R (&Ji)[4], R s,
-                              const R (&up)[Dims<K>::ND], R (&acc)[Dims<K>::ND]) {
-  using D = Dims<K>;
-  constexpr int NS = D::NS;
-  const int f = m.tri_facet[size_t(t) * 3 + e];
-  const int kd = m.facet_kind[f];
-  if (kd == kFacetWall) return;
-  const bool canon = m.tri_orient[size_t(t) * 3 + e] > 0;
-  const double* geo = m.geo + size_t(m.tri_class[t]) * kGeo;
-  const R n0 = R(geo[G_NRM + 2 * e]), n1 = R(geo[G_NRM + 2 * e + 1]);
-  const R len = R(geo[G_FLEN + e]);
-#pragma unroll 1
-  for (int q = 0; q < D::NQF; ++q) {
-    R ui0 = 0, ui1 = 0;
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-      const R ph = T.fphi[e][q][j];
-      ui0 += ph * up[j];
-      ui1 += ph * up[NS + j];
-    }
-    ui0 *= s;
-    ui1 *= s;
-    R uo0 = ui0, uo1 = ui1;
-    if (kd == kFacetInflow) {
-      const double* uq = m.inflow_q + (size_t(f) * D::NQF + (canon ? q : D::NQF - 1 - q)) * 2;
-      uo0 = R(uq[0]);
-      uo1 = R(uq[1]);
-    }
-    const R vn = R(0.5) * ((ui0 + uo0) * n0 + (ui1 + uo1) * n1);
-    const R w0 = vn >= R(0) ? ui0 : uo0, w1 = vn >= R(0) ? ui1 : uo1;
-    const R w = T.fw[q] * len * s;
-    const R A0 = -w * vn * w0, A1 = -w * vn * w1;
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-      const R ph = T.fphi[e][q][j];
-      acc[j] += A0 * ph;
-      acc[NS + j] += A1 * ph;
-    }
-  }
-}
-
-// acc[i] = L(u)(phi_i) on triangle t: -C_h(u;u,phi_i) - B_h(u,phi_i) (eq. (7), eq. (18)).
-// Volume: int (u x u - nu grad u) : grad phi. Facets: the upwind flux with u.n the
-// average of both traces, and the SIPG consistency, symmetry and penalty terms,
-// at the facet Gauss points (the neighbour traverses the facet the other way,
-// so its point q is our point NQF-1-q). ug is the global coefficient array of u.
-template <int K, typename R>
-__device__ void element_residual(const DevMesh& m, const SmemTables<K, R>& T, int t, const double* __restrict__ ug,
-                                 const R (&up)[Dims<K>::ND], R (&acc)[Dims<K>::ND]) {
-  using D = Dims<K>;
-  constexpr int NS = D::NS;
-  const R nu = R(m.nu);
-  const double* geo = m.geo + size_t(m.tri_class[t]) * kGeo;
-  const R Ji[4] = {R(geo[G_JINV + 0]), R(geo[G_JINV + 1]), R(geo[G_JINV + 2]), R(geo[G_JINV + 3])};
-  const R det = R(geo[G_DET]), s = R(geo[G_S]);
-#pragma unroll
-  for (int i = 0; i < D::ND; ++i) acc[i] = R(0);
-  // ---- volume terms
-#pragma unroll 1
-  for (int q = 0; q < D::NQ; ++q) {
-    R u0 = 0, u1 = 0, a00 = 0, a01 = 0, a10 = 0, a11 = 0;
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-      const R ph = T.vphi[q][j], d0 = T.vdphi[q][j][0], d1 = T.vdphi[q][j][1];
-      u0 += ph * up[j];
-      u1 += ph * up[NS + j];
-      a00 += d0 * up[j];
-      a01 += d1 * up[j];
-      a10 += d0 * up[NS + j];
-      a11 += d1 * up[NS + j];
-    }
-    u0 *= s;
-    u1 *= s;
-    // physical gradient du_c/dx_d = s sum_r a_cr Jinv[r][d]
-    const R g00 = s * (a00 * Ji[0] + a01 * Ji[2]), g01 = s * (a00 * Ji[1] + a01 * Ji[3]);
-    const R g10 = s * (a10 * Ji[0] + a11 * Ji[2]), g11 = s * (a10 * Ji[1] + a11 * Ji[3]);
-    const R F00 = u0 * u0 - nu * g00, F01 = u0 * u1 - nu * g01;
-    const R F10 = u1 * u0 - nu * g10, F11 = u1 * u1 - nu * g11;
-    const R w = T.vw[q] * det * s;
-    // H_cr = sum_d F_cd Jinv[r][d]
-    const R H00 = w * (F00 * Ji[0] + F01 * Ji[1]), H01 = w * (F00 * Ji[2] + F01 * Ji[3]);
-    const R H10 = w * (F10 * Ji[0] + F11 * Ji[1]), H11 = w * (F10 * Ji[2] + F11 * Ji[3]);
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-      const R d0 = T.vdphi[q][j][0], d1 = T.vdphi[q][j][1];
-      acc[j] += H00 * d0 + H01 * d1;
-      acc[NS + j] += H10 * d0 + H11 * d1;
-    }
-  }
-  // ---- facet terms
-#pragma unroll 1
-  for (int e = 0; e < 3; ++e) {
-    const int tn = m.tri_nbr[size_t(t) * 3 + e];
-    if (tn < 0) {
-      // a wall adds no term (u.n = 0 there; SIPG on interior facets only); inflow and outflow
-      // facets add the convective flux against the exterior state (Sec. 2.5)
-      if (m.facet_kind) boundary_flux<K, R>(m, T, t, e, Ji, s, up, acc);
-      continue;
-    }
-    const int en = m.tri_nbr_loc[size_t(t) * 3 + e];
-    const double* geon = m.geo + size_t(m.tri_class[tn]) * kGeo;
-    const R sn = R(geon[G_S]);
-    const R n0 = R(geo[G_NRM + 2 * e]), n1 = R(geo[G_NRM + 2 * e + 1]);
-    const R len = R(geo[G_FLEN + e]);
-    const R sig = R(m.facet_sigma[m.tri_facet[size_t(t) * 3 + e]]);
-    // normal derivative in reference gradients: d_n psi = s sum_r d_r psihat (Jinv n)_r
-    const R mo0 = Ji[0] * n0 + Ji[1] * n1, mo1 = Ji[2] * n0 + Ji[3] * n1;
-    const R mn0 = R(geon[G_JINV + 0]) * n0 + R(geon[G_JINV + 1]) * n1;
-    const R mn1 = R(geon[G_JINV + 2]) * n0 + R(geon[G_JINV + 3]) * n1;
-    R un[D::ND];
-    load_coef<D::ND>(ug + size_t(tn) * D::ND, un);
-#pragma unroll 1
-    for (int q = 0; q < D::NQF; ++q) {
-      const int qn = D::NQF - 1 - q;
-      R ui0 = 0, ui1 = 0, di0 = 0, di1 = 0, uo0 = 0, uo1 = 0, do0 = 0, do1 = 0;
-#pragma unroll
-      for (int j = 0; j < NS; ++j) {
-        const R ph = T.fphi[e][q][j];
-        const R dn = T.fdphi[e][q][j][0] * mo0 + T.fdphi[e][q][j][1] * mo1;
-        ui0 += ph * up[j];
-        ui1 += ph * up[NS + j];
-        di0 += dn * up[j];
-        di1 += dn * up[NS + j];
-        const R phn = T.fphi[en][qn][j];
-        const R dnn = T.fdphi[en][qn][j][0] * mn0 + T.fdphi[en][qn][j][1] * mn1;
-        uo0 += phn * un[j];
-        uo1 += phn * un[NS + j];
-        do0 += dnn * un[j];
-        do1 += dnn * un[NS + j];
-      }
-      ui0 *= s;
-      ui1 *= s;
-      di0 *= s;
-      di1 *= s;
-      uo0 *= sn;
-      uo1 *= sn;
-      do0 *= sn;
-      do1 *= sn;
-      const R vn = R(0.5) * ((ui0 + uo0) * n0 + (ui1 + uo1) * n1);
-      const R w0 = vn >= R(0) ? ui0 : uo0, w1 = vn >= R(0) ? ui1 : uo1;
-      const R j0 = ui0 - uo0, j1 = ui1 - uo1;
-      const R w = T.fw[q] * len * s;
-      const R A0 = w * (-vn * w0 + nu * R(0.5) * (di0 + do0) - nu * sig * j0);
-      const R A1 = w * (-vn * w1 + nu * R(0.5) * (di1 + do1) - nu * sig * j1);
-      const R B0 = w * R(0.5) * nu * j0, B1 = w * R(0.5) * nu * j1;
-#pragma unroll
-      for (int j = 0; j < NS; ++j) {
-        const R ph = T.fphi[e][q][j];
-        const R dn = T.fdphi[e][q][j][0] * mo0 + T.fdphi[e][q][j][1] * mo1;
-        acc[j] += A0 * ph + B0 * dn;
-        acc[NS + j] += A1 * ph + B1 * dn;
-      }
-    }
-  }
-}
-
-// Transposed Jacobian of the residual (adjoint of the stage functional): for the
-// state u and a functional w (coefficients), out = c_w w + c_J J_L(u)^T w with
-//   (J_L(u)^T w)_j = d/du_j L(u)(w)
-//     volume : int psi_j [(u.grad) w + (grad w)^T u]_c - nu int grad psi_j . grad w_c
-//     facets : -int psi_j [n_c (u^up . [w]) / 2 + max(u.n, 0) [w]_c]        (upwind flux in its
-//              1/2 (u.n)(u+ + u-) + 1/2 |u.n| (u+ - u-) form, sign(0) = 0)
-//              + nu int [psi_j ({d_n w}_c - sigma [w]_c) + 1/2 d_n psi_j [w]_c]  (SIPG, symmetric)
-// with [w] = w_T - w_neighbour and n the outward normal of T. The viscous part is the
-// SIPG residual of w itself (eq. (18) is symmetric). Block partials of
-// <u, dL/dnu(u)> = B_h(u, w)/nu with the sign of L, i.e. the nu-derivative of
-// L(u)(w), go to red[blockIdx].
-template <int K>
-__device__ void element_adjoint(const DevMesh& m, const SmemTables<K, double>& T, int t, const double* __restrict__ ug,
-                                const double* __restrict__ wg, double (&acc)[Dims<K>::ND], double& nupart) {
-  using D = Dims<K>;
-  constexpr int NS = D::NS, ND = D::ND;
-  const double nu = m.nu;
-  const double* geo = m.geo + size_t(m.tri_class[t]) * kGeo;
-  const double Ji[4] = {geo[G_JINV + 0], geo[G_JINV + 1], geo[G_JINV + 2], geo[G_JINV + 3]};
-  const double det = geo[G_DET], s = geo[G_S];
-  double uc[ND], wc[ND];
-  load_coef<ND>(ug + size_t(t) * ND, uc);
-  load_coef<ND>(wg + size_t(t) * ND, wc);
-#pragma unroll
-  for (int i = 0; i < ND; ++i) acc[i] = 0.0;
-  nupart = 0.0;
-#pragma unroll 1
-  for (int q = 0; q < D::NQ; ++q) {
-    double u0 = 0, u1 = 0, a[2][2] = {{0, 0}, {0, 0}}, b[2][2] = {{0, 0}, {0, 0}};
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-      const double ph = T.vphi[q][j], d0 = T.vdphi[q][j][0], d1 = T.vdphi[q][j][1];
-      u0 += ph * uc[j];
-      u1 += ph * uc[NS + j];
-      a[0][0] += d0 * wc[j];
-      a[0][1] += d1 * wc[j];
-      a[1][0] += d0 * wc[NS + j];
-      a[1][1] += d1 * wc[NS + j];
-      b[0][0] += d0 * uc[j];
-      b[0][1] += d1 * uc[j];
-      b[1][0] += d0 * uc[NS + j];
-      b[1][1] += d1 * uc[NS + j];
-    }
-    u0 *= s;
-    u1 *= s;
-    double gw[2][2], gu[2][2];   // physical gradients d w_c / d x_d, d u_c / d x_d
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      gw[c][0] = s * (a[c][0] * Ji[0] + a[c][1] * Ji[2]);
-      gw[c][1] = s * (a[c][0] * Ji[1] + a[c][1] * Ji[3]);
-      gu[c][0] = s * (b[c][0] * Ji[0] + b[c][1] * Ji[2]);
-      gu[c][1] = s * (b[c][0] * Ji[1] + b[c][1] * Ji[3]);
-    }
-    const double w = T.vw[q] * det;
-    // value-type test terms A_c = (u.grad) w_c + sum_d u_d d_c w_d
-    const double A0 = w * s * (u0 * gw[0][0] + u1 * gw[0][1] + u0 * gw[0][0] + u1 * gw[1][0]);
-    const double A1 = w * s * (u0 * gw[1][0] + u1 * gw[1][1] + u0 * gw[0][1] + u1 * gw[1][1]);
-    // gradient-type test terms: -nu grad w_c . grad psi_j, written through reference gradients
-    const double H00 = -w * s * nu * (gw[0][0] * Ji[0] + gw[0][1] * Ji[1]);
-    const double H01 = -w * s * nu * (gw[0][0] * Ji[2] + gw[0][1] * Ji[3]);
-    const double H10 = -w * s * nu * (gw[1][0] * Ji[0] + gw[1][1] * Ji[1]);
-    const double H11 = -w * s * nu * (gw[1][0] * Ji[2] + gw[1][1] * Ji[3]);
-    nupart -= w * (gu[0][0] * gw[0][0] + gu[0][1] * gw[0][1] + gu[1][0] * gw[1][0] + gu[1][1] * gw[1][1]);
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-      const double ph = T.vphi[q][j], d0 = T.vdphi[q][j][0], d1 = T.vdphi[q][j][1];
-      acc[j] += A0 * ph + H00 * d0 + H01 * d1;
-      acc[NS + j] += A1 * ph + H10 * d0 + H11 * d1;
-    }
-  }
-#pragma unroll 1
-  for (int e = 0; e < 3; ++e) {
-    const int tn = m.tri_nbr[size_t(t) * 3 + e];
-    if (tn < 0) continue;   // walls: no term in the forward residual, none in its transpose
-    const int en = m.tri_nbr_loc[size_t(t) * 3 + e];
-    const double* geon = m.geo + size_t(m.tri_class[tn]) * kGeo;
-    const double sn = geon[G_S];
-    const double n0 = geo[G_NRM + 2 * e], n1 = geo[G_NRM + 2 * e + 1];
-    const double len = geo[G_FLEN + e];
-    const double sig = m.facet_sigma[m.tri_facet[size_t(t) * 3 + e]];
-    const double mo0 = Ji[0] * n0 + Ji[1] * n1, mo1 = Ji[2] * n0 + Ji[3] * n1;
-    const double mn0 = geon[G_JINV + 0] * n0 + geon[G_JINV + 1] * n1;
-    const double mn1 = geon[G_JINV + 2] * n0 + geon[G_JINV + 3] * n1;
-    double un[ND], wn[ND];
-    load_coef<ND>(ug + size_t(tn) * ND, un);
-    load_coef<ND>(wg + size_t(tn) * ND, wn);
-#pragma unroll 1
-    for (int q = 0; q < D::NQF; ++q) {
-      const int qn = D::NQF - 1 - q;
-      double ui[2] = {0, 0}, uo[2] = {0, 0}, wi[2] = {0, 0}, wo[2] = {0, 0};
-      double dwi[2] = {0, 0}, dwo[2] = {0, 0}, dui[2] = {0, 0};
-#pragma unroll
-      for (int j = 0; j < NS; ++j) {
-        const double ph = T.fphi[e][q][j];
-        const double dn = T.fdphi[e][q][j][0] * mo0 + T.fdphi[e][q][j][1] * mo1;
-        const double phn = T.fphi[en][qn][j];
-        const double dnn = T.fdphi[en][qn][j][0] * mn0 + T.fdphi[en][qn][j][1] * mn1;
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          ui[c] += ph * uc[c * NS + j];
-          wi[c] += ph * wc[c * NS + j];
-          dwi[c] += dn * wc[c * NS + j];
-          dui[c] += dn * uc[c * NS + j];
-          uo[c] += phn * un[c * NS + j];
-          wo[c] += phn * wn[c * NS + j];
-          dwo[c] += dnn * wn[c * NS + j];
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        ui[c] *= s;
-        wi[c] *= s;
-        dwi[c] *= s;
-        dui[c] *= s;
-        uo[c] *= sn;
-        wo[c] *= sn;
-        dwo[c] *= sn;
-      }
-      const double vn = 0.5 * ((ui[0] + uo[0]) * n0 + (ui[1] + uo[1]) * n1);
-      const double sg = vn > 0.0 ? 1.0 : (vn < 0.0 ? -1.0 : 0.0);
-      const double up0 = 0.5 * ((ui[0] + uo[0]) + sg * (ui[0] - uo[0]));
-      const double up1 = 0.5 * ((ui[1] + uo[1]) + sg * (ui[1] - uo[1]));
-      const double jw0 = wi[0] - wo[0], jw1 = wi[1] - wo[1];
-      const double upj = up0 * jw0 + up1 * jw1;
-      const double vp = vn > 0.0 ? vn : 0.0;
-      const double w = T.fw[q] * len;
-      // value-type: convective adjoint + SIPG consistency and penalty of w (nu)
-      // u.n is the average of both traces: d(u.n)/du_T = n/2
-      const double A0 = w * s * (-(0.5 * n0 * upj + vp * jw0) + nu * (0.5 * (dwi[0] + dwo[0]) - sig * jw0));
-      const double A1 = w * s * (-(0.5 * n1 * upj + vp * jw1) + nu * (0.5 * (dwi[1] + dwo[1]) - sig * jw1));
-      // normal-derivative test: SIPG symmetry term
-      const double B0 = w * s * 0.5 * nu * jw0, B1 = w * s * 0.5 * nu * jw1;
-      nupart += w * (ui[0] * (0.5 * (dwi[0] + dwo[0]) - sig * jw0) + ui[1] * (0.5 * (dwi[1] + dwo[1]) - sig * jw1) +
-                     0.5 * (dui[0] * jw0 + dui[1] * jw1));
-#pragma unroll
-      for (int j = 0; j < NS; ++j) {
-        const double ph = T.fphi[e][q][j];
-        const double dn = T.fdphi[e][q][j][0] * mo0 + T.fdphi[e][q][j][1] * mo1;
-        acc[j] += A0 * ph + B0 * dn;
-        acc[NS + j] += A1 * ph + B1 * dn;
-      }
-    }
-  }
-}
-
-template <int K>
-__global__ void __launch_bounds__(128) k_adjoint(DevMesh m, const double* u, const double* w, double* out, double cw,
-                                                 double cj, int accumulate) {
-  using D = Dims<K>;
-  constexpr int ND = D::ND;
-  __shared__ SmemTables<K, double> T;
-  load_tables<K, double>(m, T);
-  __syncthreads();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  double nupart = 0.0;
-  if (t < m.n_tri) {
-    double acc[ND];
-    element_adjoint<K>(m, T, t, u, w, acc, nupart);
-#pragma unroll
-    for (int i = 0; i < ND; ++i) {
-      const size_t o = size_t(t) * ND + i;
-      const double v = cw * w[o] + cj * acc[i];
-      out[o] = accumulate ? out[o] + v : v;
-    }
-  }
-  nupart = block_sum(nupart);
-  if (threadIdx.x == 0) m.red[blockIdx.x] = nupart;
-}
-
-// acc_dev += coef * (sum of the k_adjoint block partials), in fixed order.
-__global__ void k_nu_accumulate(DevMesh m, int nparts, double coef, double* acc_dev) {
-  if (threadIdx.x >= 32) return;
-  double v = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += 32) v += m.red[i];
-  v = warp_sum(v);
-  if (threadIdx.x == 0) *acc_dev += coef * v;
-}
-
-// Stage kernel, FP64 form (the mixed form's is k_stage_df in k_stage_df.cu).
-// Modes (StageMode): the stage functional and its condensation (h = P f,
-// gl = G f), the residual alone, the pressure functional, or the projection
-// functional.
-template <int K, typename R>
-__global__ void __launch_bounds__(128) k_stage(DevMesh m, StageArgs a) {
-  using D = Dims<K>;
-  constexpr int ND = D::ND, L3 = 3 * D::NL;
-  __shared__ SmemTables<K, R> T;
-  load_tables<K, R>(m, T);
-  __syncthreads();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m.n_tri) return;
-  R up[ND];
-  load_coef<ND>(a.up + size_t(t) * ND, up);
-  R f[ND];
-  if (a.mode == MODE_PROJECT) {
-#pragma unroll
-    for (int i = 0; i < ND; ++i) f[i] = up[i];
-  } else {
-    element_residual<K, R>(m, T, t, a.up, up, f);
-    if (a.mode == MODE_STAGE) {
-      R un[ND];
-      load_coef<ND>(a.un + size_t(t) * ND, un);
-      const R ca = R(a.a), cb = R(a.b), cc = R(a.c);
-#pragma unroll
-      for (int i = 0; i < ND; ++i) f[i] = ca * un[i] + cb * up[i] + cc * f[i];
-    }
-  }
-  if (a.mode == MODE_RESIDUAL || a.mode == MODE_PRESSURE) {
-#pragma unroll
-    for (int i = 0; i < ND; ++i) m.h[size_t(t) * ND + i] = double(f[i]);
-  }
-  if (a.mode == MODE_RESIDUAL) return;
-  const int c = m.tri_class[t];
-  if (a.mode != MODE_PRESSURE) {
-    for (int i = 0; i < ND; ++i) {
-      R v = R(0);
-#pragma unroll
-      for (int j = 0; j < ND; ++j) v += m.P[(size_t(c) * ND + i) * ND + j] * f[j];
-      m.h[size_t(t) * ND + i] = double(v);
-    }
-  }
-  for (int i = 0; i < L3; ++i) {
-    R v = R(0);
-#pragma unroll
-    for (int j = 0; j < ND; ++j) v += m.G[(size_t(c) * L3 + i) * ND + j] * f[j];
-    m.gl[size_t(t) * L3 + i] = double(v);
-  }
-}
 
 // Recovery (eq. (12) eliminated locally): u_T = P_T f_T - G_T^T lam_T, with
 // lam_T the multipliers of T's three facets mapped to T's own orientation.
@@ -805,12 +413,6 @@ cudaError_t launch_coef_to_lattice(const DevMesh& m, const double* coef, double*
   return cudaGetLastError();
 }
 
-cudaError_t launch_stage(const DevMesh& m, const StageArgs& a, cudaStream_t s) {
-  if (m.elem_df) return launch_stage_df(m, a, s);
-  DGDF_DISPATCH_K(m.k, (k_stage<K, double><<<blocks_for(m.n_tri, 128), 128, 0, s>>>(m, a)));
-  return cudaGetLastError();
-}
-
 cudaError_t launch_recover(const DevMesh& m, double* out, float2* out_df, cudaStream_t s) {
   if (m.elem_df) return launch_recover_df(m, out, out_df, s);
   DGDF_DISPATCH_K(m.k, (k_recover<K><<<blocks_for(m.n_tri, 128), 128, 0, s>>>(m, out)));
@@ -834,14 +436,6 @@ cudaError_t launch_diagnostics(const DevMesh& m, const double* coef, cudaStream_
   if (nb > kMaxSolverBlocks) nb = kMaxSolverBlocks;
   DGDF_DISPATCH_K(m.k, (k_diagnostics<K><<<nb, 128, 0, s>>>(m, coef)));
   k_diag_finish<<<1, 32, 0, s>>>(m, nb);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_adjoint(const DevMesh& m, const double* u, const double* w, double* out, double cw, double cj,
-                           int accumulate, double nu_coef, double* nu_acc, cudaStream_t s) {
-  const int nb = blocks_for(m.n_tri, 128);
-  DGDF_DISPATCH_K(m.k, (k_adjoint<K><<<nb, 128, 0, s>>>(m, u, w, out, cw, cj, accumulate)));
-  k_nu_accumulate<<<1, 32, 0, s>>>(m, nb, nu_coef, nu_acc);
   return cudaGetLastError();
 }
 

@@ -632,3 +632,16 @@ def test_lattice_solver_forms_match_block_jacobi(g, N, k, precision, size):
         mesh.rk3_step(1e-3 / (N * size), 3)
         out.append(mesh.get_velocity())
     assert rel(out[0], out[1]) < 1e-13 * 1e3 * N * 10 / 1e3
+
+
+@pytest.mark.parametrize("N,k,nu,perturb", [(1, 3, 0.0, 0.0), (4, 1, 1e-3, 0.0), (13, 2, 1e-3, 0.1), (13, 3, 0.0, 0.1),
+                                            (18, 1, 0.0, 0.0), (25, 3, 1e-3, 0.0), (35, 2, 0.0, 0.0), (71, 1, 1e-3, 0.1)])
+def test_fp64_residual_tiles_match_the_oracle(g, N, k, nu, perturb):
+    # the tiles of the FP64 residual kernel from 1 to 16 triangles, with a ragged last one, and its
+    # three ways with the viscous terms (none, per-class table, reference gradients). Sums of some
+    # hundred FP64 products either way: 1e-12
+    mesh, d, X = pair(g, N, k, nu, perturb=perturb, seed=N)
+    v = random_lattice(mesh.n_tri, k, 3 * N)
+    mesh.set_velocity(v)
+    U = d.from_lattice(v)
+    assert rel(mesh.eval_residual(), d.to_lattice(d.riesz(d.residual(U)))) < TOL64
