@@ -214,6 +214,20 @@ int dg3_mesh_create(int64_t n_tet, const int64_t* tet_vertex_ids, const double* 
       (rc = upload3(M, &d.face_loc, hm.face_loc)) || (rc = upload3(M, &d.st_blk, hm.stencil_blocks)) ||
       (rc = upload3(M, &d.st_binv, hm.stencil_binv)))
     return cleanup(rc);
+  if (d.n_class <= dgdf::kDnClasses3) {
+    const int rows = ref.nqf * hm.ns;
+    std::vector<double> dn(size_t(d.n_class) * 4 * rows);
+    for (int c = 0; c < d.n_class; ++c)
+      for (int e = 0; e < 4; ++e) {
+        const dgdf::Class3& co = hm.classes[c];
+        const double* g = &ref.fdphi[size_t(e * 6 + co.perm[e]) * rows * 3];
+        double mo[3];
+        for (int r = 0; r < 3; ++r)
+          mo[r] = co.Jinv[3 * r] * co.normal[e][0] + co.Jinv[3 * r + 1] * co.normal[e][1] + co.Jinv[3 * r + 2] * co.normal[e][2];
+        for (int i = 0; i < rows; ++i) dn[size_t(c * 4 + e) * rows + i] = g[3 * i] * mo[0] + g[3 * i + 1] * mo[1] + g[3 * i + 2] * mo[2];
+      }
+    if ((rc = upload3(M, &d.dn, dn))) return cleanup(rc);
+  }
   const size_t nT = size_t(d.n_tet), nF = size_t(d.n_face), nl = size_t(hm.nl);
   if ((rc = dalloc3(M, &d.u, nT * nd)) || (rc = dalloc3(M, &d.ustage, nT * nd)) || (rc = dalloc3(M, &d.h, nT * nd)) ||
       (rc = dalloc3(M, &d.gl, nT * L4)) || (rc = dalloc3(M, &d.lam, nF * nl)) || (rc = dalloc3(M, &d.g, nF * nl)) ||

@@ -12,6 +12,7 @@ namespace dgdf {
 // Per-class geometry record (doubles): Jinv[9] row-major (d xi_r / d x_d), det = 6|T|,
 // s = 1/sqrt(det), outward normals [4][3], face areas [4], face perm indices [4]; padded to 32.
 constexpr int kGeo3 = 32;
+constexpr int kDnClasses3 = 64;
 enum Geo3Slot { G3_JINV = 0, G3_DET = 9, G3_S = 10, G3_NRM = 11, G3_AREA = 23, G3_PERM = 27 };
 
 struct DevMesh3 {
@@ -23,6 +24,8 @@ struct DevMesh3 {
   // lattice interpolation [ns][ns] and its inverse
   const double *vw, *vphi, *vdphi, *fw, *fphi, *fdphi, *lat_phi, *lat_inv;
   const double* geo;                  // [n_class][kGeo3]
+  const double* dn;                   // derivatives of the basis along the outward normals at the face points,
+                                      // [n_class][4][nqf][ns] (NULL: more than kDnClasses3 classes)
   const double *P, *G;                // [n_class][nd][nd], [n_class][4 nl][nd]
   const double *W, *WC;               // pressure rows [n_class][nw][nd], [n_class][nw][4 nl]
   const double *plat_phi, *mu_lat;    // P^(k-1) basis at the (k-1)-lattice [nw][nw]; face basis

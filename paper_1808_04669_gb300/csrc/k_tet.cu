@@ -1,7 +1,6 @@
 // Kernels of the three-dimensional path (closed tetrahedral meshes, FP64): the stage residual +
 // condensation, the recovery, the face-system PCG and the lattice / diagnostics helpers.
-// One thread per tetrahedron in the element kernels; the volume tables sit in shared memory,
-// the face tables (four local faces x six vertex orderings) are read through the L1 cache.
+// The volume tables sit in shared memory, the face tables (four local faces x six vertex orderings) are read through the L1 cache.
 // Conventions (canonical face coordinates, perm index, face rule): setup3.hpp.
 #include <algorithm>
 
@@ -41,186 +40,259 @@ __device__ void load_vol3(const DevMesh3& m, VolTables3<K>& T) {
   for (int i = threadIdx.x; i < D::NQ * D::NS * 3; i += blockDim.x) (&T.vdphi[0][0][0])[i] = m.vdphi[i];
 }
 
-// acc[i] = L(u)(phi_i) on tetrahedron t: -C_h(u; u, phi_i) - B_h(u, phi_i) (eq. (7), eq. (18)).
-// Volume: int (u x u - nu grad u) : grad phi. Faces: the upwind flux with u.n the average of both
-// traces, and the SIPG consistency, symmetry and penalty terms, at the shared face points (both
-// sides evaluate at the same canonical points, so point q is point q on either side).
-template <int K>
-__device__ void tet_residual(const DevMesh3& m, const VolTables3<K>& T, int t, const double* __restrict__ ug,
-                             const double (&up)[Dims3<K>::ND], double (&acc)[Dims3<K>::ND]) {
-  using D = Dims3<K>;
-  constexpr int NS = D::NS, ND = D::ND;
-  const double nu = m.nu;
-  const double* geo = m.geo + size_t(__ldg(&m.tet_class[t])) * kGeo3;
-  double Ji[9];
+// How the stage kernel takes the viscous terms: none (nu = 0), with the normal derivatives of the
+// basis at the face points from a per-class table (m.dn, at most kDnClasses3 classes), or from
+// reference gradients.
+enum Visc3 { VISC3_NONE, VISC3_TABLE, VISC3_GENERAL };
+
+// Values v and derivatives d along our normal of the field with coefficients U at face point q: ph,
+// fd the basis values and reference gradients of its (local face, vertex order), tab its row of the
+// table of derivatives along its own outward normal (sgn times ours), mm = Jinv n.
+template <int K, int V>
+__device__ __forceinline__ void face_trace3(const double* __restrict__ ph, const double* __restrict__ fd,
+                                            const double* __restrict__ tab, const double* U, double s, double sgn,
+                                            const double (&mm)[3], double (&v)[3], double (&d)[3]) {
+  constexpr int NS = Dims3<K>::NS;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) Ji[i] = geo[G3_JINV + i];
-  const double det = geo[G3_DET], s = geo[G3_S];
+  for (int c = 0; c < 3; ++c) v[c] = d[c] = 0.0;
 #pragma unroll
-  for (int i = 0; i < ND; ++i) acc[i] = 0.0;
-  // ---- volume terms
-#pragma unroll 1
-  for (int q = 0; q < D::NQ; ++q) {
-    double u[3], a[3][3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      u[c] = 0.0;
-      a[c][0] = a[c][1] = a[c][2] = 0.0;
-    }
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-      const double ph = T.vphi[q][j];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const double x = up[c * NS + j];
-        u[c] += ph * x;
-#pragma unroll
-        for (int r = 0; r < 3; ++r) a[c][r] += T.vdphi[q][j][r] * x;
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) u[c] *= s;
-    const double w = T.vw[q] * det * s;
-    double H[3][3];
+  for (int j = 0; j < NS; ++j) {
+    const double p = __ldg(&ph[j]);
+    double g = 0.0;
+    if constexpr (V == VISC3_TABLE) g = __ldg(&tab[j]);
+    if constexpr (V == VISC3_GENERAL) g = __ldg(&fd[3 * j]) * mm[0] + __ldg(&fd[3 * j + 1]) * mm[1] + __ldg(&fd[3 * j + 2]) * mm[2];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      double F[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        // physical gradient du_c/dx_d = s sum_r a_cr Jinv[r][d]
-        const double g = s * (a[c][0] * Ji[0 * 3 + d] + a[c][1] * Ji[1 * 3 + d] + a[c][2] * Ji[2 * 3 + d]);
-        F[d] = u[c] * u[d] - nu * g;
-      }
-#pragma unroll
-      for (int r = 0; r < 3; ++r) H[c][r] = w * (F[0] * Ji[r * 3 + 0] + F[1] * Ji[r * 3 + 1] + F[2] * Ji[r * 3 + 2]);
+      const double x = U[c * NS + j];
+      v[c] += p * x;
+      if constexpr (V != VISC3_NONE) d[c] += g * x;
     }
-#pragma unroll
-    for (int j = 0; j < NS; ++j)
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        acc[c * NS + j] += H[c][0] * T.vdphi[q][j][0] + H[c][1] * T.vdphi[q][j][1] + H[c][2] * T.vdphi[q][j][2];
   }
-  // ---- face terms
-#pragma unroll 1
-  for (int e = 0; e < 4; ++e) {
-    const int tn = __ldg(&m.tet_nbr[size_t(t) * 4 + e]);
-    const int en = __ldg(&m.tet_nbr_loc[size_t(t) * 4 + e]);
-    const double* geon = m.geo + size_t(__ldg(&m.tet_class[tn])) * kGeo3;
-    const double sn = geon[G3_S];
-    const int pe = int(geo[G3_PERM + e]), pn = int(geon[G3_PERM + en]);
-    const double n[3] = {geo[G3_NRM + 3 * e], geo[G3_NRM + 3 * e + 1], geo[G3_NRM + 3 * e + 2]};
-    const double area = geo[G3_AREA + e];
-    const double sig = __ldg(&m.face_sigma[__ldg(&m.tet_face[size_t(t) * 4 + e])]);
-    // normal derivative in reference gradients: d_n psi = s sum_r d_r psihat (Jinv n)_r, with our
-    // normal n for both sides
-    double mo[3], mn[3];
+  const double sd = V == VISC3_TABLE ? sgn * s : s;
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      mo[r] = Ji[r * 3] * n[0] + Ji[r * 3 + 1] * n[1] + Ji[r * 3 + 2] * n[2];
-      mn[r] = geon[G3_JINV + r * 3] * n[0] + geon[G3_JINV + r * 3 + 1] * n[1] + geon[G3_JINV + r * 3 + 2] * n[2];
-    }
-    double un[ND];
-#pragma unroll
-    for (int i = 0; i < ND; ++i) un[i] = __ldg(&ug[size_t(tn) * ND + i]);
-    const double* fo = m.fphi + size_t(e * 6 + pe) * D::NQF * NS;
-    const double* fdo = m.fdphi + size_t(e * 6 + pe) * D::NQF * NS * 3;
-    const double* fn = m.fphi + size_t(en * 6 + pn) * D::NQF * NS;
-    const double* fdn = m.fdphi + size_t(en * 6 + pn) * D::NQF * NS * 3;
-#pragma unroll 1
-    for (int q = 0; q < D::NQF; ++q) {
-      double ui[3] = {0, 0, 0}, di[3] = {0, 0, 0}, uo[3] = {0, 0, 0}, dn[3] = {0, 0, 0};
-#pragma unroll
-      for (int j = 0; j < NS; ++j) {
-        const double ph = __ldg(&fo[q * NS + j]);
-        const double* g = &fdo[(q * NS + j) * 3];
-        const double dno = __ldg(&g[0]) * mo[0] + __ldg(&g[1]) * mo[1] + __ldg(&g[2]) * mo[2];
-        const double phn = __ldg(&fn[q * NS + j]);
-        const double* gn = &fdn[(q * NS + j) * 3];
-        const double dnn = __ldg(&gn[0]) * mn[0] + __ldg(&gn[1]) * mn[1] + __ldg(&gn[2]) * mn[2];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          ui[c] += ph * up[c * NS + j];
-          di[c] += dno * up[c * NS + j];
-          uo[c] += phn * un[c * NS + j];
-          dn[c] += dnn * un[c * NS + j];
-        }
-      }
-      double vn = 0.0;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        ui[c] *= s;
-        di[c] *= s;
-        uo[c] *= sn;
-        dn[c] *= sn;
-        vn += (ui[c] + uo[c]) * n[c];
-      }
-      vn *= 0.5;
-      const double w = __ldg(&m.fw[q]) * 2.0 * area * s;
-      double A[3], B[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const double wup = vn >= 0.0 ? ui[c] : uo[c];
-        const double jc = ui[c] - uo[c];
-        A[c] = w * (-vn * wup + nu * 0.5 * (di[c] + dn[c]) - nu * sig * jc);
-        B[c] = w * 0.5 * nu * jc;
-      }
-#pragma unroll
-      for (int j = 0; j < NS; ++j) {
-        const double ph = __ldg(&fo[q * NS + j]);
-        const double* g = &fdo[(q * NS + j) * 3];
-        const double dno = __ldg(&g[0]) * mo[0] + __ldg(&g[1]) * mo[1] + __ldg(&g[2]) * mo[2];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) acc[c * NS + j] += A[c] * ph + B[c] * dno;
-      }
-    }
+  for (int c = 0; c < 3; ++c) {
+    v[c] *= s;
+    d[c] *= sd;
   }
 }
+
+// Words of a tetrahedron in a tile: own and neighbours' coefficients, the point terms (volume, then
+// faces) and the functional; odd row lengths against bank conflicts.
+template <int K, int V>
+struct Tile3 {
+  using D = Dims3<K>;
+  static constexpr int NF = 4 * D::NQF, NA = V == VISC3_NONE ? 3 : (V == VISC3_TABLE ? 6 : 12);
+  static constexpr int LU = D::ND + 1, LN = 4 * D::ND + 1, LF = D::ND + 1;
+  static constexpr int LH = (D::NQ * 9 > NF * NA ? D::NQ * 9 : NF * NA) | 1;
+  static constexpr int words = LU + LN + LH + LF;
+};
 
 // Stage kernel (modes as StageMode): f = a u^n + b u' + c L(u') (MODE_STAGE), L(u') alone
 // (MODE_RESIDUAL: h = f, the Riesz representer since M = I; MODE_PRESSURE: h = f and gl = G f),
 // or f = u' (MODE_PROJECT); then h = P f and gl = G f per class.
-template <int K>
-__global__ void __launch_bounds__(kTetThreads) k_stage3(DevMesh3 m, StageArgs a) {
+// L(u)(phi) = -C_h(u; u, phi) - B_h(u, phi) (eq. (7), eq. (18)). Volume: int (u x u - nu grad u) :
+// grad phi. Faces: the upwind flux with u.n the average of both traces, and the SIPG consistency,
+// symmetry and penalty terms, at the shared face points (both sides evaluate at the same canonical
+// points, so point q is point q on either side).
+// Bound: the FP64 pipes (an instruction of a warp takes a quarter of an SM 64 cycles). A thread a
+// tetrahedron held 255 registers and spilled, and 24576 tetrahedra left the last wave a quarter
+// full; here a block takes a tile of E = 2^log_e through shared memory and deals out volume points,
+// face points, test functions and operator rows to all its threads, in phases. 16^3 cubes, BDM_2:
+// 2.09 -> 1.05 ms a launch.
+template <int K, int V>
+__global__ void __launch_bounds__(kTetThreads) k_stage3(DevMesh3 m, StageArgs a, int log_e) {
   using D = Dims3<K>;
-  constexpr int ND = D::ND, L4 = 4 * D::NL;
+  using L = Tile3<K, V>;
+  constexpr int NS = D::NS, ND = D::ND, NQ = D::NQ, NQF = D::NQF, L4 = 4 * D::NL;
   __shared__ VolTables3<K> T;
+  extern __shared__ double tile3_smem[];
+  const int E = 1 << log_e;
+  double* U = tile3_smem;
+  double* N = U + E * L::LU;
+  double* H = N + E * L::LN;   // volume terms, then face terms
+  double* F = H + E * L::LH;
   load_vol3<K>(m, T);
-  __syncthreads();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m.n_tet) return;
-  double up[ND], f[ND];
-#pragma unroll
-  for (int i = 0; i < ND; ++i) up[i] = a.up[size_t(t) * ND + i];
-  if (a.mode == MODE_PROJECT) {
-#pragma unroll
-    for (int i = 0; i < ND; ++i) f[i] = up[i];
-  } else {
-    tet_residual<K>(m, T, t, a.up, up, f);
-    if (a.mode == MODE_STAGE) {
-#pragma unroll
-      for (int i = 0; i < ND; ++i) f[i] = a.a * a.un[size_t(t) * ND + i] + a.b * up[i] + a.c * f[i];
+  const double nu = m.nu;
+  const int ntiles = (m.n_tet + E - 1) >> log_e;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int t0 = tile << log_e;
+    auto tet = [&](int el) { return min(t0 + el, m.n_tet - 1); };
+    __syncthreads();
+    for (int i = threadIdx.x; i < E * ND; i += blockDim.x) {
+      const int el = i / ND, j = i - el * ND;
+      U[el * L::LU + j] = a.up[size_t(tet(el)) * ND + j];
     }
-  }
-  if (a.mode == MODE_RESIDUAL || a.mode == MODE_PRESSURE) {
+    const bool res = a.mode != MODE_PROJECT;
+    if (res)
+      for (int i = threadIdx.x; i < E * 4 * ND; i += blockDim.x) {
+        const int el = i / (4 * ND), r = i - el * 4 * ND, e = r / ND, j = r - e * ND;
+        N[el * L::LN + r] = a.up[size_t(__ldg(&m.tet_nbr[size_t(tet(el)) * 4 + e])) * ND + j];
+      }
+    __syncthreads();
+    if (res) {
+      // volume points: H[c][r], the flux in reference directions times the weight
+      for (int i = threadIdx.x; i < (NQ << log_e); i += blockDim.x) {
+        const int el = i & (E - 1), q = i >> log_e;
+        const double* up = U + el * L::LU;
+        const double* geo = m.geo + size_t(__ldg(&m.tet_class[tet(el)])) * kGeo3;
+        double Ji[9];
 #pragma unroll
-    for (int i = 0; i < ND; ++i) m.h[size_t(t) * ND + i] = f[i];
-    if (a.mode == MODE_RESIDUAL) return;
-  }
-  const int cls = m.tet_class[t];
-  const double* P = m.P + size_t(cls) * ND * ND;
-  const double* G = m.G + size_t(cls) * L4 * ND;
-  if (a.mode != MODE_PRESSURE)
-    for (int i = 0; i < ND; ++i) {
-      double v = 0.0;
+        for (int x = 0; x < 9; ++x) Ji[x] = __ldg(&geo[G3_JINV + x]);
+        const double s = __ldg(&geo[G3_S]);
+        double u[3], g[3][3];
 #pragma unroll
-      for (int j = 0; j < ND; ++j) v += __ldg(&P[i * ND + j]) * f[j];
-      m.h[size_t(t) * ND + i] = v;
+        for (int c = 0; c < 3; ++c) u[c] = g[c][0] = g[c][1] = g[c][2] = 0.0;
+#pragma unroll
+        for (int j = 0; j < NS; ++j) {
+          const double ph = T.vphi[q][j];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const double x = up[c * NS + j];
+            u[c] += ph * x;
+            if constexpr (V != VISC3_NONE)
+#pragma unroll
+              for (int r = 0; r < 3; ++r) g[c][r] += T.vdphi[q][j][r] * x;
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) u[c] *= s;
+        const double w = T.vw[q] * __ldg(&geo[G3_DET]) * s, ns = nu * s;
+        double* h = H + el * L::LH + q * 9;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          double f[3];
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            f[d] = u[c] * u[d];
+            // physical gradient du_c/dx_d = s sum_r g_cr Jinv[r][d]
+            if constexpr (V != VISC3_NONE)
+              f[d] -= ns * (g[c][0] * Ji[d] + g[c][1] * Ji[3 + d] + g[c][2] * Ji[6 + d]);
+          }
+#pragma unroll
+          for (int r = 0; r < 3; ++r) h[3 * c + r] = w * (f[0] * Ji[3 * r] + f[1] * Ji[3 * r + 1] + f[2] * Ji[3 * r + 2]);
+        }
+      }
+      __syncthreads();
+      for (int i = threadIdx.x; i < (ND << log_e); i += blockDim.x) {
+        const int el = i & (E - 1), r = i >> log_e, c = r / NS, j = r - c * NS;
+        const double* h = H + el * L::LH + 3 * c;
+        double x = 0.0, y = 0.0, z = 0.0;
+#pragma unroll 9
+        for (int q = 0; q < NQ; ++q) {
+          x += h[9 * q] * T.vdphi[q][j][0];
+          y += h[9 * q + 1] * T.vdphi[q][j][1];
+          z += h[9 * q + 2] * T.vdphi[q][j][2];
+        }
+        F[el * L::LF + r] = x + y + z;
+      }
+      __syncthreads();
+      // face points: A[c] against phi_c, B[c] against its normal derivative (general: B (Jinv n)_r
+      // against its reference gradient)
+      for (int i = threadIdx.x; i < (L::NF << log_e); i += blockDim.x) {
+        const int el = i & (E - 1), p = i >> log_e, e = p / NQF, q = p - e * NQF, t = tet(el);
+        const int tn = __ldg(&m.tet_nbr[size_t(t) * 4 + e]), en = __ldg(&m.tet_nbr_loc[size_t(t) * 4 + e]);
+        const int co = __ldg(&m.tet_class[t]), cn = __ldg(&m.tet_class[tn]);
+        const double *geo = m.geo + size_t(co) * kGeo3, *geon = m.geo + size_t(cn) * kGeo3;
+        const int ro = (e * 6 + int(__ldg(&geo[G3_PERM + e]))) * NQF + q;
+        const int rn = (en * 6 + int(__ldg(&geon[G3_PERM + en]))) * NQF + q;
+        const double n[3] = {__ldg(&geo[G3_NRM + 3 * e]), __ldg(&geo[G3_NRM + 3 * e + 1]), __ldg(&geo[G3_NRM + 3 * e + 2])};
+        const double s = __ldg(&geo[G3_S]), sn = __ldg(&geon[G3_S]);
+        double mo[3] = {0, 0, 0}, mn[3] = {0, 0, 0};
+        if constexpr (V == VISC3_GENERAL)
+#pragma unroll
+          for (int r = 0; r < 3; ++r) {
+            mo[r] = __ldg(&geo[G3_JINV + 3 * r]) * n[0] + __ldg(&geo[G3_JINV + 3 * r + 1]) * n[1] + __ldg(&geo[G3_JINV + 3 * r + 2]) * n[2];
+            mn[r] = __ldg(&geon[G3_JINV + 3 * r]) * n[0] + __ldg(&geon[G3_JINV + 3 * r + 1]) * n[1] +
+                    __ldg(&geon[G3_JINV + 3 * r + 2]) * n[2];
+          }
+        const double *to = nullptr, *tb = nullptr;
+        if constexpr (V == VISC3_TABLE) {
+          to = m.dn + (size_t(co * 4 + e) * NQF + q) * NS;
+          tb = m.dn + (size_t(cn * 4 + en) * NQF + q) * NS;
+        }
+        double ui[3], di[3], uo[3], dn[3];
+        face_trace3<K, V>(m.fphi + size_t(ro) * NS, m.fdphi + size_t(ro) * NS * 3, to, U + el * L::LU, s, 1.0, mo, ui, di);
+        face_trace3<K, V>(m.fphi + size_t(rn) * NS, m.fdphi + size_t(rn) * NS * 3, tb, N + el * L::LN + e * ND, sn, -1.0,
+                          mn, uo, dn);
+        const double vn = 0.5 * ((ui[0] + uo[0]) * n[0] + (ui[1] + uo[1]) * n[1] + (ui[2] + uo[2]) * n[2]);
+        const double w = __ldg(&m.fw[q]) * 2.0 * __ldg(&geo[G3_AREA + e]) * s, wv = w * vn, wn = w * nu;
+        const bool own = vn >= 0.0;
+        double* out = H + el * L::LH + p * L::NA;
+        double sig = 0.0;
+        if constexpr (V != VISC3_NONE) sig = __ldg(&m.face_sigma[__ldg(&m.tet_face[size_t(t) * 4 + e])]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          double x = -wv * (own ? ui[c] : uo[c]);
+          if constexpr (V != VISC3_NONE) {
+            const double jc = ui[c] - uo[c], B = 0.5 * wn * jc;
+            x += wn * (0.5 * (di[c] + dn[c]) - sig * jc);
+            if constexpr (V == VISC3_TABLE) {
+              out[3 + c] = B;
+            } else {
+#pragma unroll
+              for (int r = 0; r < 3; ++r) out[3 + 3 * c + r] = B * mo[r];
+            }
+          }
+          out[c] = x;
+        }
+      }
+      __syncthreads();
     }
-  for (int i = 0; i < L4; ++i) {
-    double v = 0.0;
+    for (int i = threadIdx.x; i < (ND << log_e); i += blockDim.x) {
+      const int el = i & (E - 1), r = i >> log_e, c = r / NS, j = r - c * NS, t = tet(el);
+      double f = U[el * L::LU + r];
+      if (res) {
+        const int co = __ldg(&m.tet_class[t]);
+        const double* geo = m.geo + size_t(co) * kGeo3;
+        const double* h = H + el * L::LH;
+        double x = F[el * L::LF + r], y = 0.0;
+#pragma unroll 1
+        for (int e = 0; e < 4; ++e) {
+          const int ro = (e * 6 + int(__ldg(&geo[G3_PERM + e]))) * NQF;
+          const double* ph = m.fphi + size_t(ro) * NS + j;
+          const double* fd = m.fdphi + (size_t(ro) * NS + j) * 3;
+          const double* tab = V == VISC3_TABLE ? m.dn + size_t(co * 4 + e) * NQF * NS + j : nullptr;
+          const double* A = h + e * NQF * L::NA;
+#pragma unroll 8
+          for (int q = 0; q < NQF; ++q) {
+            x += A[q * L::NA + c] * __ldg(&ph[q * NS]);
+            if constexpr (V == VISC3_TABLE) y += A[q * L::NA + 3 + c] * __ldg(&tab[q * NS]);
+            if constexpr (V == VISC3_GENERAL) {
+              y += A[q * L::NA + 3 + 3 * c] * __ldg(&fd[q * NS * 3]);
+              y += A[q * L::NA + 4 + 3 * c] * __ldg(&fd[q * NS * 3 + 1]);
+              y += A[q * L::NA + 5 + 3 * c] * __ldg(&fd[q * NS * 3 + 2]);
+            }
+          }
+        }
+        x += y;
+        f = a.mode == MODE_STAGE ? a.a * a.un[size_t(t) * ND + r] + a.b * f + a.c * x : x;
+      }
+      F[el * L::LF + r] = f;
+    }
+    __syncthreads();
+    if (a.mode == MODE_RESIDUAL || a.mode == MODE_PRESSURE)
+      for (int i = threadIdx.x; i < E * ND; i += blockDim.x) {
+        const int el = i / ND, r = i - el * ND;
+        if (t0 + el < m.n_tet) m.h[size_t(t0 + el) * ND + r] = F[el * L::LF + r];
+      }
+    if (a.mode == MODE_RESIDUAL) continue;
+    const int r0 = a.mode == MODE_PRESSURE ? ND : 0;
+    for (int i = threadIdx.x + (r0 << log_e); i < ((ND + L4) << log_e); i += blockDim.x) {
+      const int el = i & (E - 1), r = i >> log_e, t = tet(el);
+      const size_t cls = __ldg(&m.tet_class[t]);
+      const double* row = r < ND ? m.P + (cls * ND + r) * ND : m.G + (cls * L4 + r - ND) * ND;
+      const double* f = F + el * L::LF;
+      double x = 0.0, y = 0.0;
 #pragma unroll
-    for (int j = 0; j < ND; ++j) v += __ldg(&G[i * ND + j]) * f[j];
-    m.gl[size_t(t) * L4 + i] = v;
+      for (int j = 0; j < ND; j += 2) {
+        x += __ldg(&row[j]) * f[j];
+        y += __ldg(&row[j + 1]) * f[j + 1];
+      }
+      if (t0 + el < m.n_tet) {
+        if (r < ND) m.h[size_t(t) * ND + r] = x + y;
+        else m.gl[size_t(t) * L4 + r - ND] = x + y;
+      }
+    }
   }
 }
 
@@ -658,9 +730,34 @@ bool tet_tables_match(int k, int nq, int nqf) {
   }
 }
 
-cudaError_t launch_stage3(const DevMesh3& m, const StageArgs& a, cudaStream_t s) {
-  DGDF_DISPATCH_K3(m.k, (k_stage3<K><<<blocks3(m.n_tet), kTetThreads, 0, s>>>(m, a)));
+namespace {
+// Tiles of up to eight tetrahedra that fit in the 48 KB of shared memory beside the volume tables and
+// leave every SM two; a block takes several.
+template <int K, int V>
+cudaError_t stage3(const DevMesh3& m, const StageArgs& a, cudaStream_t st) {
+  using L = Tile3<K, V>;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const size_t room = 48 * 1024 - sizeof(VolTables3<K>) - 64;
+  int log_e = 3;
+  while (log_e > 0 && ((m.n_tet >> log_e) < 2 * sms || (size_t(L::words) << log_e) * 8 > room)) --log_e;
+  const int tiles = (m.n_tet + (1 << log_e) - 1) >> log_e;
+  k_stage3<K, V><<<std::min(tiles, 8 * sms), kTetThreads, (size_t(L::words) << log_e) * 8, st>>>(m, a, log_e);
   return cudaGetLastError();
+}
+template <int K>
+cudaError_t stage3_visc(const DevMesh3& m, const StageArgs& a, cudaStream_t s) {
+  // nu = 0 leaves out every gradient and normal derivative: they would be multiplied by zero
+  if (m.nu == 0.0) return stage3<K, VISC3_NONE>(m, a, s);
+  return m.dn ? stage3<K, VISC3_TABLE>(m, a, s) : stage3<K, VISC3_GENERAL>(m, a, s);
+}
+}  // namespace
+
+cudaError_t launch_stage3(const DevMesh3& m, const StageArgs& a, cudaStream_t s) {
+  DGDF_DISPATCH_K3(m.k, return stage3_visc<K>(m, a, s));
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_recover3(const DevMesh3& m, double* out, cudaStream_t s) {

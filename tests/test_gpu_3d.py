@@ -225,3 +225,23 @@ def test_rk3_warm_start_history_across_step_sizes(g, precond):
         U = d.rk3_step(U, h, n)
         assert rel(m.get_velocity(), d.to_lattice(U)) < TOL, (n, h)
     assert its[1] < its[0], its
+
+
+@pytest.mark.parametrize("N,k,nu,perturb", [(2, 1, 0.0, 0.0), (2, 2, 1e-2, 0.1), (3, 1, 1e-2, 0.1), (3, 2, 0.0, 0.1),
+                                            (5, 1, 1e-2, 0.0), (7, 2, 1e-2, 0.0)])
+def test_residual_tiles_match_the_oracle(g, N, k, nu, perturb):
+    # the tiles of the residual kernel (one to eight tetrahedra, a ragged last one at 7^3) and its
+    # three ways with the viscous terms: none, per-class table, reference gradients (perturbed: every
+    # tetrahedron its own class). Sums of a few hundred FP64 products either way: 1e-12
+    from synth.mesh3 import kuhn_cube_mesh, lattice_points3
+    from oracle.dg3 import Discretization3
+    vid, X = kuhn_cube_mesh(N)
+    if perturb:
+        h = 2 * np.pi / N
+        X = X + perturb * h * np.random.default_rng(N).uniform(-1, 1, size=(N ** 3, 3))[vid]
+    mesh = g.DGMesh3(vid, X, k, nu)
+    v = np.random.default_rng(k).standard_normal((mesh.n_tet, mesh.n_lat, 3))
+    mesh.set_velocity(v)
+    d = Discretization3(vid, X, k, nu)
+    ref = d.to_lattice(d.riesz(d.residual(d.from_lattice(v))))
+    assert np.linalg.norm(mesh.eval_residual() - ref) < 1e-12 * np.linalg.norm(ref)
