@@ -75,7 +75,7 @@ __device__ __forceinline__ void boundary_terms(const DevMesh& m, const float2* g
 // upwind flux (u.n) u_c^up with u.n the average of both traces, and the SIPG
 // consistency, symmetry and penalty terms, at the facet Gauss points (the
 // neighbour's point q is our point NQF-1-q).
-template <int K>
+template <int K, bool VISC>
 __device__ __forceinline__ void residual_component(const DevMesh& m, const SmemTables<K, dfl>& T, int t, int c,
                                                    const float2* __restrict__ ug, const dfl (&up)[Dims<K>::NS],
                                                    dacc (&acc)[Dims<K>::NS]) {
@@ -95,15 +95,22 @@ __device__ __forceinline__ void residual_component(const DevMesh& m, const SmemT
 #pragma unroll
     for (int j = 0; j < NS; ++j) {
       mad(U, T.vphi[q][j], up[j]);
-      mad(A0, T.vdphi[q][j][0], up[j]);
-      mad(A1, T.vdphi[q][j][1], up[j]);
+      if constexpr (VISC) {
+        mad(A0, T.vdphi[q][j][0], up[j]);
+        mad(A1, T.vdphi[q][j][1], up[j]);
+      }
     }
-    const dfl uc = s * val(U), a0 = val(A0), a1 = val(A1);
-    // physical gradient d u_c / d x_d = s sum_r a_r Jinv[r][d]
-    const dfl g0 = s * (a0 * Ji0 + a1 * Ji2), g1 = s * (a0 * Ji1 + a1 * Ji3);
+    const dfl uc = s * val(U);
     const dfl uo = shfl_pair(uc);
     const dfl u0 = c ? uo : uc, u1 = c ? uc : uo;
-    const dfl F0 = uc * u0 - nu * g0, F1 = uc * u1 - nu * g1;
+    dfl F0 = uc * u0, F1 = uc * u1;
+    if constexpr (VISC) {
+      const dfl a0 = val(A0), a1 = val(A1);
+      // physical gradient d u_c / d x_d = s sum_r a_r Jinv[r][d]
+      const dfl g0 = s * (a0 * Ji0 + a1 * Ji2), g1 = s * (a0 * Ji1 + a1 * Ji3);
+      F0 = F0 - nu * g0;
+      F1 = F1 - nu * g1;
+    }
     const dfl w = T.vw[q] * ds;
     // H_r = w sum_d F_d Jinv[r][d]
     const dfl H0 = w * (F0 * Ji0 + F1 * Ji1), H1 = w * (F0 * Ji2 + F1 * Ji3);
@@ -145,28 +152,36 @@ __device__ __forceinline__ void residual_component(const DevMesh& m, const SmemT
 #pragma unroll
       for (int j = 0; j < NS; ++j) {
         mad(V, T.fphi[e][q][j], up[j]);
-        mad(D0, T.fdphi[e][q][j][0], up[j]);
-        mad(D1, T.fdphi[e][q][j][1], up[j]);
         mad(Vn, T.fphi[en][qn][j], un[j]);
-        mad(Dn0, T.fdphi[en][qn][j][0], un[j]);
-        mad(Dn1, T.fdphi[en][qn][j][1], un[j]);
+        if constexpr (VISC) {
+          mad(D0, T.fdphi[e][q][j][0], up[j]);
+          mad(D1, T.fdphi[e][q][j][1], up[j]);
+          mad(Dn0, T.fdphi[en][qn][j][0], un[j]);
+          mad(Dn1, T.fdphi[en][qn][j][1], un[j]);
+        }
       }
-      const dfl ui = s * val(V), di = s * (mo0 * val(D0) + mo1 * val(D1));
-      const dfl uo = sn * val(Vn), dn = sn * (mn0 * val(Dn0) + mn1 * val(Dn1));
+      const dfl ui = s * val(V), uo = sn * val(Vn);
       // u.n = 1/2 (u_in + u_out) . n, summed in the same order by both threads of the pair
       const dfl pc = (ui + uo) * nc, po = shfl_pair(pc);
       const dfl vn = half(c ? po + pc : pc + po);
       const dfl wup = vn >= dfl(0) ? ui : uo;
-      const dfl jc = ui - uo;
       const dfl w = T.fw[q] * lens;
-      const dfl A = w * (hnu * (di + dn) - vn * wup - nusig * jc);
-      const dfl B = w * hnu * jc;
-      const dfl B0 = B * mo0, B1 = B * mo1;
+      if constexpr (VISC) {
+        const dfl di = s * (mo0 * val(D0) + mo1 * val(D1)), dn = sn * (mn0 * val(Dn0) + mn1 * val(Dn1));
+        const dfl jc = ui - uo;
+        const dfl A = w * (hnu * (di + dn) - vn * wup - nusig * jc);
+        const dfl B = w * hnu * jc;
+        const dfl B0 = B * mo0, B1 = B * mo1;
 #pragma unroll
-      for (int j = 0; j < NS; ++j) {
-        mad(acc[j], A, T.fphi[e][q][j]);
-        mad(acc[j], B0, T.fdphi[e][q][j][0]);
-        mad(acc[j], B1, T.fdphi[e][q][j][1]);
+        for (int j = 0; j < NS; ++j) {
+          mad(acc[j], A, T.fphi[e][q][j]);
+          mad(acc[j], B0, T.fdphi[e][q][j][0]);
+          mad(acc[j], B1, T.fdphi[e][q][j][1]);
+        }
+      } else {
+        const dfl A = -(w * (vn * wup));
+#pragma unroll
+        for (int j = 0; j < NS; ++j) mad(acc[j], A, T.fphi[e][q][j]);
       }
     }
   }
@@ -191,7 +206,7 @@ __device__ __forceinline__ void residual_component(const DevMesh& m, const SmemT
 // MODE_PROJECT), h = f in FP64 (MODE_RESIDUAL, MODE_PRESSURE) and gl_df
 // (MODE_PRESSURE). Thread c of a pair owns rows c*NS.. of f and h, and the rows
 // i = c (mod 2) of gl.
-template <int K>
+template <int K, bool VISC>
 __global__ void __launch_bounds__(kStageDfThreads, 2) k_stage_df(DevMesh m, StageArgs a) {
   using D = Dims<K>;
   constexpr int NS = D::NS, ND = D::ND, L3 = 3 * D::NL;
@@ -212,7 +227,7 @@ __global__ void __launch_bounds__(kStageDfThreads, 2) k_stage_df(DevMesh m, Stag
     dacc acc[NS];
 #pragma unroll
     for (int j = 0; j < NS; ++j) acc[j] = dacc_zero();
-    residual_component<K>(m, T, t, c, a.up_df, up, acc);
+    residual_component<K, VISC>(m, T, t, c, a.up_df, up, acc);
     if (a.mode == MODE_STAGE) {
       dfl un[NS];
       load_df<NS>(a.un_df + size_t(t) * ND + c * NS, un);
@@ -289,7 +304,7 @@ __device__ __forceinline__ void load_pairs(const float2* __restrict__ p, dfl2 (&
 
 __device__ __forceinline__ dfl lane(const dfl2& v, int l) { return l ? dfl(v.hi.y, v.lo.y) : dfl(v.hi.x, v.lo.x); }
 
-template <int K>
+template <int K, bool VISC>
 __device__ __forceinline__ void residual_pairs(const DevMesh& m, const PairTables<K>& T, int t, int c,
                                                const float2* __restrict__ ug, const dfl2 (&up)[PairTables<K>::NS2],
                                                dacc2 (&acc)[PairTables<K>::NS2]) {
@@ -309,14 +324,21 @@ __device__ __forceinline__ void residual_pairs(const DevMesh& m, const PairTable
 #pragma unroll
     for (int jp = 0; jp < NS2; ++jp) {
       mad2(U, pair(T.vphi[q][jp]), up[jp]);
-      mad2(A0, pair(T.vd0[q][jp]), up[jp]);
-      mad2(A1, pair(T.vd1[q][jp]), up[jp]);
+      if constexpr (VISC) {
+        mad2(A0, pair(T.vd0[q][jp]), up[jp]);
+        mad2(A1, pair(T.vd1[q][jp]), up[jp]);
+      }
     }
-    const dfl uc = s * val_sum(U), a0 = val_sum(A0), a1 = val_sum(A1);
-    const dfl g0 = s * (a0 * Ji0 + a1 * Ji2), g1 = s * (a0 * Ji1 + a1 * Ji3);
+    const dfl uc = s * val_sum(U);
+    dfl g0(0), g1(0);
+    if constexpr (VISC) {
+      const dfl a0 = val_sum(A0), a1 = val_sum(A1);
+      g0 = s * (a0 * Ji0 + a1 * Ji2);
+      g1 = s * (a0 * Ji1 + a1 * Ji3);
+    }
     const dfl uo = shfl_pair(uc);
     const dfl u0 = c ? uo : uc, u1 = c ? uc : uo;
-    const dfl F0 = uc * u0 - nu * g0, F1 = uc * u1 - nu * g1;
+    const dfl F0 = VISC ? uc * u0 - nu * g0 : uc * u0, F1 = VISC ? uc * u1 - nu * g1 : uc * u1;
     const dfl w = to_dfl(T.vw[q]) * ds;
     const dfl2 H0 = splat(w * (F0 * Ji0 + F1 * Ji1)), H1 = splat(w * (F0 * Ji2 + F1 * Ji3));
 #pragma unroll
@@ -350,23 +372,34 @@ __device__ __forceinline__ void residual_pairs(const DevMesh& m, const PairTable
 #pragma unroll
       for (int jp = 0; jp < NS2; ++jp) {
         mad2(V, pair(T.fphi[e][q][jp]), up[jp]);
-        mad2(Dd, pair(T.dn[cls][e][q][jp]), up[jp]);
         mad2(Vn, pair(T.fphi[en][qn][jp]), un[jp]);
-        mad2(Dnd, pair(T.dn[ncls][en][qn][jp]), un[jp]);
+        if constexpr (VISC) {
+          mad2(Dd, pair(T.dn[cls][e][q][jp]), up[jp]);
+          mad2(Dnd, pair(T.dn[ncls][en][qn][jp]), un[jp]);
+        }
       }
-      const dfl ui = s * val_sum(V), di = s * val_sum(Dd);
-      const dfl uo = sn * val_sum(Vn), dn = msn * val_sum(Dnd);
+      const dfl ui = s * val_sum(V);
+      dfl di(0), dn(0);
+      if constexpr (VISC) di = s * val_sum(Dd);
+      const dfl uo = sn * val_sum(Vn);
+      if constexpr (VISC) dn = msn * val_sum(Dnd);
       const dfl pc = (ui + uo) * nc, po = shfl_pair(pc);
       const dfl vn = half(c ? po + pc : pc + po);
       const dfl wup = vn >= dfl(0) ? ui : uo;
       const dfl jc = ui - uo;
       const dfl w = to_dfl(T.fw[q]) * lens;
-      const dfl2 A = splat(w * (hnu * (di + dn) - vn * wup - nusig * jc));
-      const dfl2 B = splat(w * hnu * jc);
+      if constexpr (VISC) {
+        const dfl2 A = splat(w * (hnu * (di + dn) - vn * wup - nusig * jc));
+        const dfl2 B = splat(w * hnu * jc);
 #pragma unroll
-      for (int jp = 0; jp < NS2; ++jp) {
-        mad2(acc[jp], A, pair(T.fphi[e][q][jp]));
-        mad2(acc[jp], B, pair(T.dn[cls][e][q][jp]));
+        for (int jp = 0; jp < NS2; ++jp) {
+          mad2(acc[jp], A, pair(T.fphi[e][q][jp]));
+          mad2(acc[jp], B, pair(T.dn[cls][e][q][jp]));
+        }
+      } else {
+        const dfl2 A = splat(-(w * (vn * wup)));
+#pragma unroll
+        for (int jp = 0; jp < NS2; ++jp) mad2(acc[jp], A, pair(T.fphi[e][q][jp]));
       }
     }
   }
@@ -386,10 +419,16 @@ __device__ __forceinline__ void residual_pairs(const DevMesh& m, const PairTable
         });
 }
 
+// Blocks per SM that k_stage_df2 is compiled for
+template <int K, bool VISC>
+constexpr int stage_df2_blocks() {
+  return K == 2 && !VISC ? 3 : 2;   // 113 registers do there
+}
+
 // Stage kernel, paired form: the modes, inputs and outputs of k_stage_df; the class
 // operators P and G are read as column pairs (m.P2, m.G2).
-template <int K>
-__global__ void __launch_bounds__(kStageDfThreads, 2) k_stage_df2(DevMesh m, StageArgs a) {
+template <int K, bool VISC>
+__global__ void __launch_bounds__(kStageDfThreads, (stage_df2_blocks<K, VISC>())) k_stage_df2(DevMesh m, StageArgs a) {
   using D = Dims<K>;
   using PT = PairTables<K>;
   constexpr int NS = D::NS, ND = D::ND, L3 = 3 * D::NL, NS2 = PT::NS2, NDP = ND / 2;
@@ -413,7 +452,7 @@ __global__ void __launch_bounds__(kStageDfThreads, 2) k_stage_df2(DevMesh m, Sta
     dacc2 acc[NS2];
 #pragma unroll
     for (int jp = 0; jp < NS2; ++jp) acc[jp] = dacc2_zero();
-    residual_pairs<K>(m, T, t, c, a.up_df, up, acc);
+    residual_pairs<K, VISC>(m, T, t, c, a.up_df, up, acc);
     if (a.mode == MODE_STAGE) {
       dfl un[NS];
       load_df<NS>(a.un_df + size_t(t) * ND + c * NS, un);
@@ -575,11 +614,11 @@ inline int blocks_for(long long n, int bs) { return int((n + bs - 1) / bs); }
 
 }  // namespace
 
-template <int K>
+template <int K, bool VISC>
 cudaError_t launch_pairs(const DevMesh& m, const StageArgs& a, cudaStream_t s) {
   // the host image must have the layout of PairTables<K>
   if (m.ptab_words != int(sizeof(PairTables<K>) / sizeof(float4))) return cudaErrorInvalidValue;
-  k_stage_df2<K><<<blocks_for(m.n_tri, kStageDfThreads / 2), kStageDfThreads, 0, s>>>(m, a);
+  k_stage_df2<K, VISC><<<blocks_for(m.n_tri, kStageDfThreads / 2), kStageDfThreads, 0, s>>>(m, a);
   return cudaSuccess;
 }
 
@@ -594,12 +633,17 @@ cudaError_t launch_pairs(const DevMesh& m, const StageArgs& a, cudaStream_t s) {
 cudaError_t launch_stage_df(const DevMesh& m, const StageArgs& a, cudaStream_t s) {
   if (!a.up_df || (a.mode == MODE_STAGE && !a.un_df)) return cudaErrorInvalidValue;
   const int nb = blocks_for(m.n_tri, kStageDfThreads / 2);
+  // nu = 0 leaves out every gradient and normal derivative: they would be multiplied by zero
+  // (512^2, BDM_2: 514 -> 300 us a launch)
+  const bool visc = m.nu != 0.0;
   if (m.ptab) {
     cudaError_t e = cudaSuccess;
-    DGDF_DISPATCH_K(m.k, (e = launch_pairs<K>(m, a, s)));
+    DGDF_DISPATCH_K(m.k, (e = visc ? launch_pairs<K, true>(m, a, s) : launch_pairs<K, false>(m, a, s)));
     if (e != cudaSuccess) return e;
+  } else if (visc) {
+    DGDF_DISPATCH_K(m.k, (k_stage_df<K, true><<<nb, kStageDfThreads, 0, s>>>(m, a)));
   } else {
-    DGDF_DISPATCH_K(m.k, (k_stage_df<K><<<nb, kStageDfThreads, 0, s>>>(m, a)));
+    DGDF_DISPATCH_K(m.k, (k_stage_df<K, false><<<nb, kStageDfThreads, 0, s>>>(m, a)));
   }
   return cudaGetLastError();
 }

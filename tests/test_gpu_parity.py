@@ -645,3 +645,14 @@ def test_fp64_residual_tiles_match_the_oracle(g, N, k, nu, perturb):
     mesh.set_velocity(v)
     U = d.from_lattice(v)
     assert rel(mesh.eval_residual(), d.to_lattice(d.riesz(d.residual(U)))) < TOL64
+
+
+@pytest.mark.parametrize("N,k,perturb", [(1, 2, 0.0), (7, 1, 0.0), (9, 3, 0.1), (13, 2, 0.1), (14, 3, 0.0)])
+def test_mixed_inviscid_residual_matches_the_oracle(g, N, k, perturb):
+    # nu = 0 in the mixed form: the paired kernel (few classes) and the general one (perturbed)
+    # without their viscous sums, on random fields (no cancellation); double-float sums keep some 44
+    # bits, 1e-11 leaves them a few thousand roundings
+    mesh, d, X = pair(g, N, k, 0.0, precision=1, perturb=perturb, seed=N)
+    v = random_lattice(mesh.n_tri, k, N)
+    mesh.set_velocity(v)
+    assert rel(mesh.eval_residual(), d.to_lattice(d.riesz(d.residual(d.from_lattice(v))))) < 1e-11
