@@ -70,11 +70,11 @@ struct dg_mesh {
   std::vector<void*> allocs;
   int solver_blocks[2] = {1, 1};
   bool use_lattice = false;
-  int lattice_blocks = 0;
+  int lattice_blocks = 0, lattice_work = 0;
   bool tc_available = false;      // the tensor-core recovery is set up (mixed form, <= 2 classes)
   bool use_ml = false;            // multilevel-preconditioned PCG (k_multilevel.cu)
   int grid_div = 1;               // solver grid divided by this while a batch runs lanes
-  int ml_blocks = 0;
+  int ml_blocks = 0, ml_fit = 0;
   std::string lattice_why;
   double last_c = 0.0;            // coefficient of L(u') in the last stage solved
   long long gen = 0;              // bumped by every setter that changes a kernel argument
@@ -284,12 +284,13 @@ void forget_history(dg_mesh* M) {
   for (int s = 0; s < dg_mesh::kMaxStages; ++s) M->hist_n[s] = 0;
 }
 
-// Persistent solver blocks: the mesh's maximum, divided by the ensemble's lanes while a batch
+// Persistent solver blocks: those that fit on the device, divided by the ensemble's lanes while a batch
 // runs members on parallel graph branches (so that every solver grid that can run at the
 // same time fits on the device together, and no grid barrier waits for another grid's blocks).
-int capped(const dg_mesh* M, int nb) {
+// work: blocks that the solve has work for.
+int capped(const dg_mesh* M, int nb, int work) {
   if (M->grid_div > 1) nb = std::max(1, nb / M->grid_div);
-  return nb;
+  return std::min(nb, work);
 }
 
 int solve(dg_mesh* M, double warm_scale, int stage = -1, double dt = 0.0, bool homog = false) {
@@ -326,15 +327,15 @@ int solve(dg_mesh* M, double warm_scale, int stage = -1, double dt = 0.0, bool h
   a.inner_maxit = M->p.cg_maxit;
   a.floor_rtol = 1e-9;
   if (M->use_lattice) {
-    const int nb = capped(M, M->lattice_blocks);
+    const int nb = capped(M, M->lattice_blocks, M->lattice_work);
     return launch(M, a.mixed ? KC_SOLVE_LAT32 : KC_SOLVE_LAT64,
                   [&] { return dgdf::launch_solve_lattice(M->dm, a, nb, a.mixed, M->stream); });
   }
   if (M->use_ml) {
-    const int nb = capped(M, M->ml_blocks);
+    const int nb = capped(M, M->ml_fit, M->ml_blocks);
     return launch(M, KC_SOLVE_ML, [&] { return dgdf::launch_solve_ml(M->dm, a, nb, M->stream); });
   }
-  const int nb = capped(M, M->solver_blocks[a.mixed]);
+  const int nb = capped(M, M->solver_blocks[a.mixed], M->solver_blocks[a.mixed]);
   return launch(M, a.mixed ? KC_SOLVE_MIXED : KC_SOLVE64, [&] { return dgdf::launch_solve(M->dm, a, nb, M->stream); });
 }
 
@@ -684,7 +685,7 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
     d.ml_nlev = int(mlh.lv.size());
     d.ml_nc = mlh.nc;
     M->use_ml = d.ml_nlev >= 1;
-    M->ml_blocks = dgdf::solver_ml_blocks(d);
+    M->ml_blocks = dgdf::solver_ml_blocks(d, &M->ml_fit);
     if (M->use_ml && M->ml_blocks < 1) return cleanup(fail(DG_ERR_CUDA, "multilevel solver does not fit"));
   }
   if (lat.ok && lat_blocks > 0) {
@@ -837,6 +838,7 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
     d.lat_logn = logn;
     M->use_lattice = true;
     M->lattice_blocks = lat_blocks;
+    M->lattice_work = dgdf::lattice_work_blocks(hm.k, N);
   }
   // multiplier history of the stages (warm starts), in the layout of the solver's lam: two
   // entries on the lattice path (its solves take two PCG iterations from the linear
@@ -1614,7 +1616,7 @@ int dg_get_solver_stats(dg_mesh* M, double out[8]) {
   out[4] = s.last_sweeps;
   out[5] = double(s.total_sweeps);
   out[6] = M->use_lattice ? 1.0 : (M->use_ml ? 2.0 : 0.0);
-  out[7] = M->use_lattice ? M->lattice_blocks
+  out[7] = M->use_lattice ? std::min(M->lattice_blocks, M->lattice_work)
                           : (M->use_ml ? M->ml_blocks : M->solver_blocks[M->p.precision == DG_PRECISION_MIXED]);
   return DG_OK;
 }

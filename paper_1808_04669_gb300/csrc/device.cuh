@@ -248,7 +248,7 @@ cudaError_t launch_energy_watch(const double* u, long long n, double* watch, dou
 cudaError_t launch_solve(const DevMesh& m, const SolveArgs& a, int nblocks, cudaStream_t s);
 // FP64 PCG with the multilevel preconditioner (k_multilevel.cu)
 cudaError_t launch_solve_ml(const DevMesh& m, const SolveArgs& a, int nblocks, cudaStream_t s);
-int solver_ml_blocks(const DevMesh& m);
+int solver_ml_blocks(const DevMesh& m, int* fit);   // blocks with work; fit: that fit on the device at once
 int ml_grid_threads();   // threads of the solver's full grid on the current device
 // whether the operators of ncls stencil classes (nl modes, nb blocks) fit in shared memory
 bool ml_class_tables_fit(int nl, int nb, bool fp32, int ncls);
@@ -261,7 +261,8 @@ int lattice_group_rows(int k, int N, int fp32);          // rows per transform g
 size_t lattice_symbol_elems(int k, int N, int fp32);   // complex entries of the stored inverse symbol
 size_t lattice_spectrum_elems(int k, int N);   // complex entries of the spectrum work array
 size_t lattice_buffer_elems(int k, int N, int fp32);
-int lattice_blocks(int k, int N, int fp32);
+int lattice_blocks(int k, int N, int fp32);   // that fit on the device at once
+int lattice_work_blocks(int k, int N);         // that a solve has work for
 cudaError_t launch_solve_lattice(const DevMesh& m, const SolveArgs& a, int nblocks, int fp32, cudaStream_t s);
 long long noalloc_max_dofs();
 cudaError_t solve_noalloc(int k, int n_facet, const int32_t* facet_nbr, const int32_t* stencil, const double* blocks,

@@ -37,6 +37,34 @@ __global__ void __launch_bounds__(128) k_recover(DevMesh m, double* out) {
   }
 }
 
+// The same with a thread per coefficient, for meshes of fewer than kRecoverSmall triangles: below
+// that a thread per triangle leaves SM quarters without a warp (FP64 instructions take one 64 cycles),
+// above it the shared multipliers win. 8^2, BDM_2: 10.4 us a thread per triangle, 6.0 per coefficient;
+// 64^2, BDM_2: 11.1, 8.3; 128^2, BDM_3: 22.9, 28.7.
+constexpr int kRecoverSmall = 608 * 32;
+template <int K>
+__global__ void __launch_bounds__(128) k_recover_coef(DevMesh m, double* out) {
+  using D = Dims<K>;
+  constexpr int ND = D::ND, NL = D::NL, L3 = 3 * NL;
+  const int o = blockIdx.x * blockDim.x + threadIdx.x;
+  if (o >= m.n_tri * ND) return;
+  const int t = o / ND, i = o - t * ND;
+  const double* G = m.G + size_t(__ldg(&m.tri_class[t])) * L3 * ND + i;
+  double v = m.h[o], w = 0.0;
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    const double* lam = m.lam + size_t(__ldg(&m.tri_facet[size_t(t) * 3 + e])) * NL;
+    const bool flip = __ldg(&m.tri_orient[size_t(t) * 3 + e]) < 0;
+#pragma unroll
+    for (int mm = 0; mm < NL; ++mm) {
+      const double g = __ldg(&G[(e * NL + mm) * ND]);
+      if (mm & 1) w -= (flip ? -g : g) * lam[mm];
+      else v -= g * lam[mm];
+    }
+  }
+  out[o] = v + w;
+}
+
 // Element pressure w_T = W_T f_T - (W C^T)_T lam_T; block partial sums of the
 // integral of w for the L^2_0 shift go to red[0][block].
 template <int K>
@@ -121,54 +149,35 @@ __global__ void __launch_bounds__(128) k_pressure_lattice(DevMesh m, const doubl
   }
 }
 
-// Lattice values -> orthonormal coefficients: coef = sqrt(det) Vhat^-1 vals per component.
+// Lattice values -> orthonormal coefficients: coef = sqrt(det) Vhat^-1 vals per component; a thread
+// per value, as the recovery.
 template <int K>
-__global__ void k_lattice_to_coef(DevMesh m, const double* vals, double* coef) {
-  using D = Dims<K>;
-  constexpr int NS = D::NS;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m.n_tri) return;
-  const double sq = 1.0 / m.geo[size_t(m.tri_class[t]) * kGeo + G_S];
-  double v[NS][2];
+__global__ void __launch_bounds__(128) k_lattice_to_coef(DevMesh m, const double* __restrict__ vals,
+                                                         double* __restrict__ coef) {
+  constexpr int NS = Dims<K>::NS, ND = 2 * NS;
+  const long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (o >= (long long)m.n_tri * ND) return;
+  const int t = int(o / ND), r = int(o - (long long)t * ND), c = r / NS, j = r - c * NS;
+  const double* v = vals + size_t(t) * ND + c;
+  double x = 0.0;
 #pragma unroll
-  for (int p = 0; p < NS; ++p) {
-    v[p][0] = vals[(size_t(t) * NS + p) * 2];
-    v[p][1] = vals[(size_t(t) * NS + p) * 2 + 1];
-  }
-#pragma unroll
-  for (int j = 0; j < NS; ++j) {
-    double c0 = 0.0, c1 = 0.0;
-#pragma unroll
-    for (int p = 0; p < NS; ++p) {
-      c0 += m.lat_inv[j * NS + p] * v[p][0];
-      c1 += m.lat_inv[j * NS + p] * v[p][1];
-    }
-    coef[size_t(t) * 2 * NS + j] = sq * c0;
-    coef[size_t(t) * 2 * NS + NS + j] = sq * c1;
-  }
+  for (int p = 0; p < NS; ++p) x += __ldg(&m.lat_inv[j * NS + p]) * v[2 * p];
+  const double* geo = m.geo + size_t(__ldg(&m.tri_class[t])) * kGeo;
+  coef[o] = __ldg(&geo[G_DET]) * __ldg(&geo[G_S]) * x;   // sqrt(det) = det / sqrt(det): no FP64 division
 }
 
 template <int K>
-__global__ void k_coef_to_lattice(DevMesh m, const double* coef, double* vals) {
-  using D = Dims<K>;
-  constexpr int NS = D::NS;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m.n_tri) return;
-  const double s = m.geo[size_t(m.tri_class[t]) * kGeo + G_S];
-  double c[2 * NS];
+__global__ void __launch_bounds__(128) k_coef_to_lattice(DevMesh m, const double* __restrict__ coef,
+                                                         double* __restrict__ vals) {
+  constexpr int NS = Dims<K>::NS, ND = 2 * NS;
+  const long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (o >= (long long)m.n_tri * ND) return;
+  const int t = int(o / ND), r = int(o - (long long)t * ND), p = r >> 1, c = r & 1;
+  const double* u = coef + size_t(t) * ND + c * NS;
+  double x = 0.0;
 #pragma unroll
-  for (int i = 0; i < 2 * NS; ++i) c[i] = coef[size_t(t) * 2 * NS + i];
-#pragma unroll
-  for (int p = 0; p < NS; ++p) {
-    double v0 = 0.0, v1 = 0.0;
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-      v0 += m.lat_phi[p * NS + j] * c[j];
-      v1 += m.lat_phi[p * NS + j] * c[NS + j];
-    }
-    vals[(size_t(t) * NS + p) * 2] = s * v0;
-    vals[(size_t(t) * NS + p) * 2 + 1] = s * v1;
-  }
+  for (int j = 0; j < NS; ++j) x += __ldg(&m.lat_phi[p * NS + j]) * u[j];
+  vals[o] = __ldg(&m.geo[size_t(__ldg(&m.tri_class[t])) * kGeo + G_S]) * x;
 }
 
 // The same conversions for the mixed form, in double-float arithmetic on the FP32 pipes (the
@@ -401,7 +410,7 @@ cudaError_t launch_lattice_to_coef(const DevMesh& m, const double* vals, double*
   if (m.elem_df)
     DGDF_DISPATCH_K(m.k, (k_lattice_to_coef_df<K><<<blocks_for(m.n_tri, kConvTris), kConvTris, 0, s>>>(m, vals, coef)))
   else
-    DGDF_DISPATCH_K(m.k, (k_lattice_to_coef<K><<<blocks_for(m.n_tri, 128), 128, 0, s>>>(m, vals, coef)))
+    DGDF_DISPATCH_K(m.k, (k_lattice_to_coef<K><<<blocks_for((long long)m.n_tri * m.nd, 128), 128, 0, s>>>(m, vals, coef)))
   return cudaGetLastError();
 }
 
@@ -409,13 +418,17 @@ cudaError_t launch_coef_to_lattice(const DevMesh& m, const double* coef, double*
   if (m.elem_df)
     DGDF_DISPATCH_K(m.k, (k_coef_to_lattice_df<K><<<blocks_for(m.n_tri, kConvTris), kConvTris, 0, s>>>(m, coef, vals)))
   else
-    DGDF_DISPATCH_K(m.k, (k_coef_to_lattice<K><<<blocks_for(m.n_tri, 128), 128, 0, s>>>(m, coef, vals)))
+    DGDF_DISPATCH_K(m.k, (k_coef_to_lattice<K><<<blocks_for((long long)m.n_tri * m.nd, 128), 128, 0, s>>>(m, coef, vals)))
   return cudaGetLastError();
 }
 
 cudaError_t launch_recover(const DevMesh& m, double* out, float2* out_df, cudaStream_t s) {
   if (m.elem_df) return launch_recover_df(m, out, out_df, s);
-  DGDF_DISPATCH_K(m.k, (k_recover<K><<<blocks_for(m.n_tri, 128), 128, 0, s>>>(m, out)));
+  if (m.n_tri < kRecoverSmall) {
+    DGDF_DISPATCH_K(m.k, (k_recover_coef<K><<<blocks_for((long long)m.n_tri * m.nd, 128), 128, 0, s>>>(m, out)));
+  } else {
+    DGDF_DISPATCH_K(m.k, (k_recover<K><<<blocks_for(m.n_tri, 128), 128, 0, s>>>(m, out)));
+  }
   return cudaGetLastError();
 }
 

@@ -1,6 +1,8 @@
 // Host side of the lattice facet solver (the kernel is in k_lattice_kernel.cuh): sizes of its
 // shared-memory buffers and of the stored symbol, the launch shape and the launch. Each
 // instantiation k_solve_lat<K, MIXED> lives in its own object file (k_lattice_inst.cu).
+#include <algorithm>
+
 #include "k_lattice_kernel.cuh"
 
 namespace dgdf {
@@ -123,6 +125,15 @@ int lattice_blocks(int k, int N, int fp32) {
   int nb = sms * (per_sm < 2 ? per_sm : 2);
   if (nb > kMaxSolverBlocks) nb = kMaxSolverBlocks;
   return nb;
+}
+
+// Blocks that the widest pass has work for: a lane per value of the facet passes, a tile of the row
+// passes, a column or half of one. Fewer blocks make the barriers cheaper (N = 8, BDM_2, FP64: 304 ->
+// 6 blocks, 55 -> 50 us a solve; N = 65, BDM_1, mixed: 304 -> 100 blocks, 66 -> 62).
+int lattice_work_blocks(int k, int N) {
+  const long long lanes = 3ll * N * N * (k == 1 ? 2 : 4);
+  return std::max({int(std::min<long long>((lanes + kLatThreads - 1) / kLatThreads, kMaxSolverBlocks)),
+                   3 * ((N + kLatTJ - 1) / kLatTJ), (lattice_split(N) ? 2 : 1) * (N / 2 + 1)});
 }
 
 cudaError_t launch_solve_lattice(const DevMesh& m, const SolveArgs& a, int nblocks, int fp32, cudaStream_t s) {

@@ -985,7 +985,7 @@ MLSys<R> ml_system(const DevMesh3& m, const DevMesh& v) {
 
 // Blocks of the solver's grid: one per SM, fewer on meshes that would leave a block less than
 // two warps of facet lanes. Also lets the kernel use its shared memory. 0: it does not fit.
-int ml_blocks(const void* fn, int threads, int nl, int nb, bool fp32, int ncls, int n) {
+int ml_blocks(const void* fn, int threads, int nl, int nb, bool fp32, int ncls, int n, int* fit = nullptr) {
   int dev = 0, sms = 0, per_sm = 0, idx = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -996,6 +996,7 @@ int ml_blocks(const void* fn, int threads, int nl, int nb, bool fp32, int ncls, 
     cudaGetLastError();
     return 0;
   }
+  if (fit) *fit = sms;
   return blocks;
 }
 
@@ -1056,10 +1057,10 @@ cudaError_t launch_ml_apply(const DevMesh& m, const double* r, double* z, int nb
   return cudaErrorInvalidValue;
 }
 
-int solver_ml_blocks(const DevMesh& m) {
+int solver_ml_blocks(const DevMesh& m, int* fit) {
   const bool fp32 = m.ml_lv_f != nullptr;
   ML_K2(m.k, fp32, return ml_blocks((const void*)k_solve_ml<NL, 5, R, DevMesh>, ml_threads<NL, R>(), NL, 5, fp32,
-                                m.ml_ncls, m.n_facet));
+                                m.ml_ncls, m.n_facet, fit));
   return 0;
 }
 

@@ -296,27 +296,26 @@ __global__ void __launch_bounds__(kTetThreads) k_stage3(DevMesh3 m, StageArgs a,
   }
 }
 
-// Recovery u = P f - G^T lam_T (eq. (12) condensed): h holds P f.
+// Recovery u = P f - G^T lam_T (eq. (12) condensed): h holds P f. A thread per coefficient.
 template <int K>
 __global__ void __launch_bounds__(kTetThreads) k_recover3(DevMesh3 m, double* out) {
   using D = Dims3<K>;
   constexpr int ND = D::ND, NL = D::NL, L4 = 4 * NL;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m.n_tet) return;
-  double lam[L4];
+  const long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (o >= (long long)m.n_tet * ND) return;
+  const int t = int(o / ND), i = int(o - (long long)t * ND);
+  const double* G = m.G + size_t(__ldg(&m.tet_class[t])) * L4 * ND + i;
+  double v = m.h[o], w = 0.0;
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    const int f = m.tet_face[size_t(t) * 4 + e];
+    const double* lam = m.lam + size_t(__ldg(&m.tet_face[size_t(t) * 4 + e])) * NL;
 #pragma unroll
-    for (int j = 0; j < NL; ++j) lam[e * NL + j] = m.lam[size_t(f) * NL + j];
+    for (int j = 0; j < NL; ++j) {
+      if (j & 1) w -= __ldg(&G[(e * NL + j) * ND]) * lam[j];
+      else v -= __ldg(&G[(e * NL + j) * ND]) * lam[j];
+    }
   }
-  const double* G = m.G + size_t(m.tet_class[t]) * L4 * ND;
-  for (int i = 0; i < ND; ++i) {
-    double v = m.h[size_t(t) * ND + i];
-#pragma unroll
-    for (int l = 0; l < L4; ++l) v -= __ldg(&G[l * ND + i]) * lam[l];
-    out[size_t(t) * ND + i] = v;
-  }
+  out[o] = v + w;
 }
 
 // Element pressure of eq. (12) (h = f of MODE_PRESSURE, lam the solve's multipliers):
@@ -604,17 +603,17 @@ __global__ void k_lattice_to_coef3(DevMesh3 m, const double* vals, double* coef)
 }
 
 template <int K>
-__global__ void k_coef_to_lattice3(DevMesh3 m, const double* coef, double* vals) {
-  constexpr int NS = Dims3<K>::NS;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m.n_tet) return;
-  const double s = m.geo[size_t(m.tet_class[t]) * kGeo3 + G3_S];
-  for (int p = 0; p < NS; ++p)
-    for (int c = 0; c < 3; ++c) {
-      double v = 0.0;
-      for (int j = 0; j < NS; ++j) v += m.lat_phi[p * NS + j] * coef[size_t(t) * 3 * NS + c * NS + j];
-      vals[(size_t(t) * NS + p) * 3 + c] = s * v;
-    }
+__global__ void __launch_bounds__(kTetThreads) k_coef_to_lattice3(DevMesh3 m, const double* __restrict__ coef,
+                                                                  double* __restrict__ vals) {
+  constexpr int NS = Dims3<K>::NS, ND = 3 * NS;
+  const long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (o >= (long long)m.n_tet * ND) return;
+  const int t = int(o / ND), r = int(o - (long long)t * ND), p = r / 3, c = r - 3 * p;
+  const double* u = coef + size_t(t) * ND + c * NS;
+  double v = 0.0;
+#pragma unroll
+  for (int j = 0; j < NS; ++j) v += __ldg(&m.lat_phi[p * NS + j]) * u[j];
+  vals[o] = __ldg(&m.geo[size_t(__ldg(&m.tet_class[t])) * kGeo3 + G3_S]) * v;
 }
 
 // Diagnostics partials per block: energy, enstrophy (|curl u|^2), max |div u| at the volume
@@ -702,7 +701,7 @@ __global__ void k_diag_finish3(DevMesh3 m, int nparts) {
   }
 }
 
-int blocks3(int n) { return (n + kTetThreads - 1) / kTetThreads; }
+int blocks3(long long n) { return int((n + kTetThreads - 1) / kTetThreads); }
 
 template <int K>
 int solve3_blocks_for() {
@@ -761,7 +760,7 @@ cudaError_t launch_stage3(const DevMesh3& m, const StageArgs& a, cudaStream_t s)
 }
 
 cudaError_t launch_recover3(const DevMesh3& m, double* out, cudaStream_t s) {
-  DGDF_DISPATCH_K3(m.k, (k_recover3<K><<<blocks3(m.n_tet), kTetThreads, 0, s>>>(m, out)));
+  DGDF_DISPATCH_K3(m.k, (k_recover3<K><<<blocks3((long long)m.n_tet * m.nd), kTetThreads, 0, s>>>(m, out)));
   return cudaGetLastError();
 }
 
@@ -771,7 +770,7 @@ cudaError_t launch_lattice_to_coef3(const DevMesh3& m, const double* vals, doubl
 }
 
 cudaError_t launch_coef_to_lattice3(const DevMesh3& m, const double* coef, double* vals, cudaStream_t s) {
-  DGDF_DISPATCH_K3(m.k, (k_coef_to_lattice3<K><<<blocks3(m.n_tet), kTetThreads, 0, s>>>(m, coef, vals)));
+  DGDF_DISPATCH_K3(m.k, (k_coef_to_lattice3<K><<<blocks3((long long)m.n_tet * m.nd), kTetThreads, 0, s>>>(m, coef, vals)));
   return cudaGetLastError();
 }
 
