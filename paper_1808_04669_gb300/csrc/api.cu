@@ -495,6 +495,36 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
       }
     }
     if ((rc = upload(M, &d.dn64, dn))) return cleanup(rc);
+    // the viscous terms that a triangle's own coefficients enter linearly, as matrices on them:
+    // vown = -int grad phi_j . grad phi_i + sum over the facets of vfac, and
+    // vfac[e] = int_e (phi_j d_n phi_i + d_n phi_j phi_i) / 2
+    const int ns_ = hm.ns;
+    std::vector<double> vown(size_t(d.n_class) * ns_ * ns_, 0.0), vfac(size_t(d.n_class) * 3 * ns_ * ns_, 0.0);
+    for (int c = 0; c < d.n_class; ++c) {
+      const dgdf::ClassOps& co = hm.classes[c];
+      const double s2 = 1.0 / co.det;
+      for (int j = 0; j < ns_; ++j)
+        for (int i = 0; i < ns_; ++i) {
+          double v = 0.0;
+          for (int q = 0; q < ref.nq; ++q) {
+            const double *gj = &ref.vdphi[(size_t(q) * ns_ + j) * 2], *gi = &ref.vdphi[(size_t(q) * ns_ + i) * 2];
+            for (int x = 0; x < 2; ++x)
+              v -= ref.vw[q] * co.det * s2 * (gj[0] * co.Jinv[x] + gj[1] * co.Jinv[2 + x]) *
+                   (gi[0] * co.Jinv[x] + gi[1] * co.Jinv[2 + x]);
+          }
+          for (int e = 0; e < 3; ++e) {
+            double f = 0.0;
+            for (int q = 0; q < nqf; ++q) {
+              const double *ph = &ref.fphi[(size_t(e) * nqf + q) * ns_], *dq = &dn[((size_t(c) * 3 + e) * nqf + q) * ns_];
+              f += ref.fw[q] * co.flen[e] * s2 * 0.5 * (ph[j] * dq[i] + dq[j] * ph[i]);
+            }
+            vfac[((size_t(c) * 3 + e) * ns_ + j) * ns_ + i] = f;
+            v += f;
+          }
+          vown[(size_t(c) * ns_ + j) * ns_ + i] = v;
+        }
+    }
+    if ((rc = upload(M, &d.vown64, vown)) || (rc = upload(M, &d.vfac64, vfac))) return cleanup(rc);
     if (d.elem_df) {
       // paired image for k_stage_df2: rows of ns values as ceil(ns/2) pairs
       // {hi_j, hi_j+1, lo_j, lo_j+1} (a missing j+1 is 0), in the order of PairTables<K>
@@ -523,6 +553,9 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
         std::vector<double> dnfull(size_t(dgdf::kDnClasses) * 3 * nqf * ns, 0.0);
         std::copy(dn.begin(), dn.end(), dnfull.begin());
         rows(dnfull.data(), dgdf::kDnClasses * 3 * nqf, ns, 1);
+        std::vector<double> vfull(size_t(dgdf::kDnClasses) * ns * ns, 0.0);
+        std::copy(vown.begin(), vown.end(), vfull.begin());
+        rows(vfull.data(), dgdf::kDnClasses * ns, ns, 1);   // vown[cls][i][j]
       }
       for (int q = 0; q < nq; ++q) {
         float h, l;
@@ -553,6 +586,13 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
         return out;
       };
       std::vector<float> p2 = pairs(P, nd), g2 = pairs(G, L3);
+      std::vector<float> main_tab;
+      main_tab.swap(pt);
+      rows(vfac.data(), d.n_class * 3 * ns, ns, 1);
+      std::vector<float> vf2;
+      vf2.swap(pt);
+      pt.swap(main_tab);
+      if ((rc = upload_f4(M, &d.vfac2, vf2))) return cleanup(rc);
       if ((rc = upload_f4(M, &d.ptab, pt)) || (rc = upload_f4(M, &d.P2, p2)) || (rc = upload_f4(M, &d.G2, g2)))
         return cleanup(rc);
     }

@@ -26,7 +26,9 @@ constexpr int kTileThreads = 128;
 
 // How a kernel takes the viscous terms: none (nu = 0), with the normal derivatives of the basis at
 // the facet points from a per-class table (m.dn64, at most kDnClasses classes), or from reference
-// gradients.
+// gradients. The stage kernel with tables takes the terms that a triangle's own coefficients enter
+// linearly (volume, own consistency and symmetry) as one matrix per class (m.vown64): its volume
+// points then need no gradients, its facet points no own normal derivative.
 enum Visc { VISC_NONE, VISC_TABLE, VISC_GENERAL };
 
 template <int K>
@@ -144,6 +146,7 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
   using L = StageTile<K, V>;
   constexpr int NS = D::NS, ND = D::ND, NQ = D::NQ, NQF = D::NQF, NF = 3 * NQF, L3 = 3 * D::NL;
   __shared__ SmemTables<K, double> T;
+  __shared__ int info[16];   // 8 x class + a bit per boundary facet
   extern __shared__ double tile_smem[];
   const int E = 1 << log_e;
   double* U = tile_smem;
@@ -153,8 +156,10 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
   double* F = A + E * L::LA;
   double* dn = F + E * L::LF;
   load_tables<K, double>(m, T);
-  if constexpr (V == VISC_TABLE)
+  if constexpr (V == VISC_TABLE) {
     for (int i = threadIdx.x; i < m.n_class * NF * NS; i += blockDim.x) dn[i] = __ldg(&m.dn64[i]);
+    for (int i = threadIdx.x; i < m.n_class * NS * NS; i += blockDim.x) dn[m.n_class * NF * NS + i] = __ldg(&m.vown64[i]);
+  }
   const double nu = m.nu;
   const int ntiles = (m.n_tri + E - 1) >> log_e;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -162,6 +167,13 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
     __syncthreads();
     const bool res = a.mode != MODE_PROJECT;
     load_tile<K>(m, a.up, t0, E, U, res ? N : nullptr);
+    if (int(threadIdx.x) < E) {
+      const int t = min(t0 + int(threadIdx.x), m.n_tri - 1);
+      int v = __ldg(&m.tri_class[t]) * 8;
+#pragma unroll
+      for (int e = 0; e < 3; ++e) v |= __ldg(&m.tri_nbr[size_t(t) * 3 + e]) < 0 ? 1 << e : 0;
+      info[threadIdx.x] = v;
+    }
     __syncthreads();
     if (res) {
       // 1: points
@@ -178,7 +190,7 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
             const double ph = T.vphi[pt][j], x = u[j], y = u[NS + j];
             u0 += ph * x;
             u1 += ph * y;
-            if constexpr (V != VISC_NONE) {
+            if constexpr (V == VISC_GENERAL) {
               const double d0 = T.vdphi[pt][j][0], d1 = T.vdphi[pt][j][1];
               a00 += d0 * x;
               a01 += d1 * x;
@@ -189,7 +201,7 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
           u0 *= s;
           u1 *= s;
           double F00 = u0 * u0, F01 = u0 * u1, F11 = u1 * u1, F10 = F01;
-          if constexpr (V != VISC_NONE) {
+          if constexpr (V == VISC_GENERAL) {
             // physical gradient du_c/dx_d = s sum_r a_cr Jinv[r][d]
             const double ns = nu * s;
             F00 -= ns * (a00 * J0 + a01 * J2);
@@ -218,7 +230,7 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
           facet_geo<K, V>(m, t, e, tn, g);
           double ui[2], di[2], uo[2], dd[2];
           if (tn >= 0) {
-            facet_trace<K, V, true>(T, dn, u, e, q, g.cls, g.s, 1.0, g.mo0, g.mo1, ui, di);
+            facet_trace<K, V, V == VISC_GENERAL>(T, dn, u, e, q, g.cls, g.s, 1.0, g.mo0, g.mo1, ui, di);
             facet_trace<K, V, true>(T, dn, N + el * L::LN + e * ND, g.en, NQF - 1 - q, g.ncls, g.sn, -1.0, g.mn0, g.mn1,
                                     uo, dd);
           } else {
@@ -245,8 +257,13 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
               double B = 0.0;
               if (tn >= 0) {
                 const double jc = ui[c] - uo[c], wn = w * nu;
-                x += wn * (0.5 * (di[c] + dd[c]) - g.sig * jc);
-                B = 0.5 * wn * jc;
+                if constexpr (V == VISC_TABLE) {
+                  x += wn * (0.5 * dd[c] - g.sig * jc);
+                  B = -0.5 * wn * uo[c];
+                } else {
+                  x += wn * (0.5 * (di[c] + dd[c]) - g.sig * jc);
+                  B = 0.5 * wn * jc;
+                }
               }
               out[c] = x;
               if constexpr (V == VISC_TABLE) {
@@ -282,9 +299,21 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
           }
         }
         if constexpr (V == VISC_TABLE) {
-          const double* tab = dn + __ldg(&m.tri_class[t]) * NF * NS + j;
+          const int cls = info[el] >> 3, walls = info[el] & 7;
+          const double *tab = dn + cls * NF * NS + j, *vo = dn + m.n_class * NF * NS + (cls * NS + j) * NS;
+          const double* u = U + el * L::LU + c * NS;
 #pragma unroll
           for (int p = 0; p < NF; ++p) y += A_[p * L::NA + 2 + c] * tab[p * NS];
+          double z = 0.0;
+#pragma unroll
+          for (int k = 0; k < NS; ++k) z += vo[k] * u[k];
+          for (int e = 0; walls >> e; ++e)
+            if (walls >> e & 1) {   // a boundary facet has no viscous terms
+              const double* vf = m.vfac64 + ((size_t(cls) * 3 + e) * NS + j) * NS;
+#pragma unroll
+              for (int k = 0; k < NS; ++k) z -= __ldg(&vf[k]) * u[k];
+            }
+          x += nu * z;
         }
         x += y;
         f = a.mode == MODE_STAGE ? a.a * a.un[size_t(t) * ND + r] + a.b * f + a.c * x : x;
@@ -302,7 +331,7 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
     const int r0 = a.mode == MODE_PRESSURE ? ND : 0;
     for (int i = threadIdx.x + (r0 << log_e); i < ((ND + L3) << log_e); i += blockDim.x) {
       const int el = i & (E - 1), r = i >> log_e, t = min(t0 + el, m.n_tri - 1);
-      const size_t cls = __ldg(&m.tri_class[t]);
+      const size_t cls = info[el] >> 3;
       const double* row = r < ND ? m.P + (cls * ND + r) * ND : m.G + (cls * L3 + r - ND) * ND;
       const double* f = F + el * L::LF;
       double x = 0.0, y = 0.0;
@@ -512,7 +541,8 @@ cudaError_t tile_shape(const DevMesh& m, TileShape& s) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const size_t table = V == VISC_TABLE ? size_t(m.n_class) * 3 * Dims<K>::NQF * Dims<K>::NS : 0;
+  const size_t table =
+      V == VISC_TABLE ? size_t(m.n_class) * (3 * Dims<K>::NQF + Dims<K>::NS) * Dims<K>::NS : 0;
   const size_t room = 48 * 1024 - sizeof(SmemTables<K, double>) - 512;
   s.log_e = 4;
   while (s.log_e > 0 && ((m.n_tri >> s.log_e) < 2 * sms || ((size_t(T::words) << s.log_e) + table) * 8 > room)) --s.log_e;

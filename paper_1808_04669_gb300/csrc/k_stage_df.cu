@@ -277,7 +277,10 @@ __global__ void __launch_bounds__(kStageDfThreads, 2) k_stage_df(DevMesh m, Stag
 // once in the packed FP32x2 instructions (dacc2 / mad2), with the tables laid out as
 // pairs {hi_j, hi_j+1, lo_j, lo_j+1}. The terms and the per-point arithmetic are those of
 // k_stage_df; only the order of summation inside each dot product differs (even and odd
-// j apart).
+// j apart). The viscous terms that a triangle's own coefficients enter linearly (volume, own
+// consistency and symmetry) are one matrix per class (PairTables::visc): the volume points
+// need no gradients, the facet points no own normal derivative, and the symmetry term keeps the
+// neighbour's trace alone. 4080 -> 3340 multiply-adds a triangle at k = 3: 256^2 287 -> @V256@ us.
 template <int K>
 struct PairTables {
   static constexpr int NS2 = (Dims<K>::NS + 1) / 2, NQ = Dims<K>::NQ, NQF = Dims<K>::NQF;
@@ -286,6 +289,7 @@ struct PairTables {
   float4 vd1[NQ][NS2];   // d/dxi2
   float4 fphi[3][NQF][NS2];
   float4 dn[kDnClasses][3][NQF][NS2];   // d/dn of the basis at the facet points, per class
+  float4 visc[kDnClasses][Dims<K>::NS][NS2];   // the viscous terms of the own coefficients, per class
   float2 vw[NQ], fw[NQF];
 };
 
@@ -320,25 +324,13 @@ __device__ __forceinline__ void residual_pairs(const DevMesh& m, const PairTable
   // ---- volume terms
 #pragma unroll 1
   for (int q = 0; q < D::NQ; ++q) {
-    dacc2 U = dacc2_zero(), A0 = dacc2_zero(), A1 = dacc2_zero();
+    dacc2 U = dacc2_zero();
 #pragma unroll
-    for (int jp = 0; jp < NS2; ++jp) {
-      mad2(U, pair(T.vphi[q][jp]), up[jp]);
-      if constexpr (VISC) {
-        mad2(A0, pair(T.vd0[q][jp]), up[jp]);
-        mad2(A1, pair(T.vd1[q][jp]), up[jp]);
-      }
-    }
+    for (int jp = 0; jp < NS2; ++jp) mad2(U, pair(T.vphi[q][jp]), up[jp]);
     const dfl uc = s * val_sum(U);
-    dfl g0(0), g1(0);
-    if constexpr (VISC) {
-      const dfl a0 = val_sum(A0), a1 = val_sum(A1);
-      g0 = s * (a0 * Ji0 + a1 * Ji2);
-      g1 = s * (a0 * Ji1 + a1 * Ji3);
-    }
     const dfl uo = shfl_pair(uc);
     const dfl u0 = c ? uo : uc, u1 = c ? uc : uo;
-    const dfl F0 = VISC ? uc * u0 - nu * g0 : uc * u0, F1 = VISC ? uc * u1 - nu * g1 : uc * u1;
+    const dfl F0 = uc * u0, F1 = uc * u1;
     const dfl w = to_dfl(T.vw[q]) * ds;
     const dfl2 H0 = splat(w * (F0 * Ji0 + F1 * Ji1)), H1 = splat(w * (F0 * Ji2 + F1 * Ji3));
 #pragma unroll
@@ -368,20 +360,16 @@ __device__ __forceinline__ void residual_pairs(const DevMesh& m, const PairTable
 #pragma unroll 1
     for (int q = 0; q < D::NQF; ++q) {
       const int qn = D::NQF - 1 - q;
-      dacc2 V = dacc2_zero(), Dd = dacc2_zero(), Vn = dacc2_zero(), Dnd = dacc2_zero();
+      dacc2 V = dacc2_zero(), Vn = dacc2_zero(), Dnd = dacc2_zero();
 #pragma unroll
       for (int jp = 0; jp < NS2; ++jp) {
         mad2(V, pair(T.fphi[e][q][jp]), up[jp]);
         mad2(Vn, pair(T.fphi[en][qn][jp]), un[jp]);
-        if constexpr (VISC) {
-          mad2(Dd, pair(T.dn[cls][e][q][jp]), up[jp]);
-          mad2(Dnd, pair(T.dn[ncls][en][qn][jp]), un[jp]);
-        }
+        if constexpr (VISC) mad2(Dnd, pair(T.dn[ncls][en][qn][jp]), un[jp]);
       }
       const dfl ui = s * val_sum(V);
-      dfl di(0), dn(0);
-      if constexpr (VISC) di = s * val_sum(Dd);
       const dfl uo = sn * val_sum(Vn);
+      dfl dn(0);
       if constexpr (VISC) dn = msn * val_sum(Dnd);
       const dfl pc = (ui + uo) * nc, po = shfl_pair(pc);
       const dfl vn = half(c ? po + pc : pc + po);
@@ -389,8 +377,8 @@ __device__ __forceinline__ void residual_pairs(const DevMesh& m, const PairTable
       const dfl jc = ui - uo;
       const dfl w = to_dfl(T.fw[q]) * lens;
       if constexpr (VISC) {
-        const dfl2 A = splat(w * (hnu * (di + dn) - vn * wup - nusig * jc));
-        const dfl2 B = splat(w * hnu * jc);
+        const dfl2 A = splat(w * (hnu * dn - vn * wup - nusig * jc));
+        const dfl2 B = splat(-(w * hnu * uo));
 #pragma unroll
         for (int jp = 0; jp < NS2; ++jp) {
           mad2(acc[jp], A, pair(T.fphi[e][q][jp]));
@@ -400,6 +388,26 @@ __device__ __forceinline__ void residual_pairs(const DevMesh& m, const PairTable
         const dfl2 A = splat(-(w * (vn * wup)));
 #pragma unroll
         for (int jp = 0; jp < NS2; ++jp) mad2(acc[jp], A, pair(T.fphi[e][q][jp]));
+      }
+    }
+  }
+  // the viscous terms of the own coefficients; a boundary facet has none
+  if constexpr (VISC) {
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      const dfl2 x = splat(nu * lane(up[i / 2], i & 1));
+#pragma unroll
+      for (int jp = 0; jp < NS2; ++jp) mad2(acc[jp], x, pair(T.visc[cls][i][jp]));
+    }
+#pragma unroll 1
+    for (int e = 0; e < 3; ++e) {
+      if (__ldg(&m.tri_nbr[size_t(t) * 3 + e]) >= 0) continue;
+      const float4* vf = m.vfac2 + (size_t(cls) * 3 + e) * NS * NS2;
+#pragma unroll
+      for (int i = 0; i < NS; ++i) {
+        const dfl2 x = splat(-(nu * lane(up[i / 2], i & 1)));
+#pragma unroll
+        for (int jp = 0; jp < NS2; ++jp) mad2(acc[jp], x, pair(__ldg(&vf[i * NS2 + jp])));
       }
     }
   }
