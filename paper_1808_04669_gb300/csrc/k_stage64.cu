@@ -11,8 +11,8 @@
 //   3  a row of the class operators P and G
 // Operands come from shared memory, which the slow pipes leave idle. E is a power of two, at most
 // 16 and small enough to give every SM two tiles. Time per launch, a thread a triangle -> tasks:
-// 8^2 BDM_2 107 -> 19 us, 48^2 perturbed BDM_2 113 -> 39, 64^2 BDM_2 107 -> 51, 128^2 BDM_3 438 -> 320
-// (0.88 of 2 FMA a clock and SM); the adjoint's at 64^2 BDM_2 about 130 -> 52.
+// 8^2 BDM_2 107 -> 18 us, 48^2 perturbed BDM_2 113 -> 39, 64^2 BDM_2 107 -> 44, 128^2 BDM_3 438 -> 282
+// (320 of that before the own viscous terms became a matrix); the adjoint's at 64^2 BDM_2 130 -> 52.
 #include <algorithm>
 
 #include "device.cuh"

@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(kStageDfThreads, 2) k_stage_df(DevMesh m, Stag
 // j apart). The viscous terms that a triangle's own coefficients enter linearly (volume, own
 // consistency and symmetry) are one matrix per class (PairTables::visc): the volume points
 // need no gradients, the facet points no own normal derivative, and the symmetry term keeps the
-// neighbour's trace alone. 4080 -> 3340 multiply-adds a triangle at k = 3: 256^2 287 -> @V256@ us.
+// neighbour's trace alone. 4080 -> 3340 multiply-adds a triangle at k = 3: 256^2 287 -> 233 us.
 template <int K>
 struct PairTables {
   static constexpr int NS2 = (Dims<K>::NS + 1) / 2, NQ = Dims<K>::NQ, NQF = Dims<K>::NQF;
