@@ -41,7 +41,7 @@ L2_FLUSH_BYTES = 512 << 20
 # over the three stages of a step (the first stage reads one state, the others two), from the
 # ncu capture summarised in profiles/; used only while the stage-kernel sources still hash to
 # the captured `sha`, else the line reports null.
-NCU_TRAFFIC = {"stage_residual": {"sha": "62f71c3ca9c15082", "n_tri": 131072, "bytes": 40963755,
+NCU_TRAFFIC = {"stage_residual": {"sha": "606d4b9243dd1631", "n_tri": 131072, "bytes": 40762283,
                                   "source": "profiles/k_stage_df2_shear_n256_k3.md"}}
 
 
@@ -209,39 +209,42 @@ def element_kernel_sha():
 
 
 def stage_flops_per_triangle(k, tabulated=True):
-    """Flops of the stage kernel per triangle (FMA = 2), counted from its loops: the volume rule
-    has 3, 7, 16 points for k = 1, 2, 3 (fully symmetric, degree 3k - 1). With
-    `tabulated` (meshes of at most 4 geometry classes, mixed form) the facet normal derivatives
-    of the basis come from per-class tables: two sums per trace and per test instead of three."""
+    """Flops of the viscous stage kernel per triangle (FMA = 2), counted from its loops: the volume
+    rule has 3, 7, 16 points for k = 1, 2, 3 (fully symmetric, degree 3k - 1). With `tabulated`
+    (meshes of at most 4 geometry classes) the viscous terms of the triangle's own coefficients are
+    one matrix per class, and the facet normal derivatives of the basis come from per-class tables:
+    per volume point the trace and its test, per facet point both traces, the neighbour's normal
+    derivative and two tests. Otherwise gradients (volume) and three sums per trace and per test."""
     ns = (k + 1) * (k + 2) // 2
     nd = 2 * ns
     nq = {1: 3, 2: 7, 3: 16}[k]
     nqf = (3 * k + 2) // 2
-    vol = nq * (2 * (6 * ns + 4 * ns) + 40)              # trace/gradient sums, flux, test sums
-    per_pt = (8 * ns + 4 * ns) if tabulated else (12 * ns + 6 * ns)
+    vol = nq * (2 * ((2 if tabulated else 6) * ns + 4 * ns) + 40)   # trace (gradient) sums, flux, test sums
+    per_pt = (6 * ns + 4 * ns) if tabulated else (12 * ns + 6 * ns)
     fac = 3 * nqf * (2 * per_pt + 30)                      # both traces, flux, test sums
+    own = 2 * nd * ns if tabulated else 0                  # the own viscous matrix
     out = 3 * nd + 2 * nd * nd + 2 * 3 * (k + 1) * nd    # stage combination, P f, G f
-    return vol + fac + out
+    return vol + fac + own + out
 
 
 def lattice_solver_bytes(n_facet, k, iters, solves):
-    """Algorithmic DRAM bytes of the mixed-form lattice (Fourier-preconditioned) facet solves.
+    """Algorithmic DRAM bytes of the mixed-form lattice facet solves (refinement with the
+    Fourier-space inverse).
 
     Vectors are double-float (8 B per DOF), z is FP32 (4 B); the spectrum holds half the
     wavenumbers (4 B per DOF per pass) and the FP32 deflated eigen form of the symbol
     (C + 1 + C(C+1)/2 complex entries per wavenumber: 4 (C + 1 + C(C+1)/2) / C B per DOF),
-    C = 3(k+1). Per DOF and CG iteration: SpMV pass 36 B (read z, p, q; write p, q); update +
-    forward rows 52 B (read r, q, lam, p; write r, lam, spectrum); columns 8 B + symbol; inverse
-    rows 20 B (read spectrum, r, z_old; write z); plus 20 B of stencil ids per facet. Per solve:
-    g assembly with the warm-start history (read two entries, shift one), the first residual and
-    one more preconditioner application, 124 B + symbol per DOF; the new multipliers are copied
-    into the history, 16 B per DOF.
+    C = 3(k+1). Per DOF and iteration: forward rows 12 B (read r; write the spectrum); columns
+    8 B + symbol; inverse rows 32 B (read the spectrum, lam; write z, lam, the history entry);
+    residual 20 B (read r, z; write r); plus 20 B of stencil ids per facet. Per solve: g from both
+    sides, the warm start from two history entries and the first residual 48 B, and the history
+    shift 16 B per DOF, plus 28 B of ids per facet.
     """
     nl = n_facet * (k + 1)
     C = 3 * (k + 1)
     sym = 4 * (C + 1 + C * (C + 1) // 2) / C
-    per_iter = nl * (36 + 52 + 8 + sym + 20) + 20 * n_facet
-    per_solve = nl * (124 + 16 + sym) + 20 * n_facet
+    per_iter = nl * (12 + 8 + sym + 32 + 20) + 20 * n_facet
+    per_solve = nl * (48 + 16) + 28 * n_facet
     return iters * per_iter + solves * per_solve
 
 
@@ -455,7 +458,7 @@ def run_ours(args):
     roof64 = {"kernel": name64, "ms_per_launch": per64_s * 1e3,
               "share_of_device_time": ms64 / sum(v[0] for v in prof64.values())}
     if name64.startswith("stage_residual"):
-        a64 = stage_flops_per_triangle(k, tabulated=False) * fp64.n_tri / per64_s / 1e12
+        a64 = stage_flops_per_triangle(k, tabulated=fp64.n_class <= 4) * fp64.n_tri / per64_s / 1e12
         p64 = fp64_peak_tflops(sm_mhz, sms)
         b64 = stage_bytes_per_triangle(k) * fp64.n_tri
         roof64.update({"bound": "alu", "achieved": a64, "peak": p64, "unit": "TFLOP/s", "frac": a64 / p64,

@@ -164,8 +164,8 @@ int dg_project_divfree(dg_mesh* mesh);
  * forms F = a M u^n + b [M u' + dt L(u')] and solves eq. (12) for the next
  * stage velocity. With DG_PRECISION_MIXED the facet system of each stage is
  * solved with FP32 preconditioning: FP32 PCG inside FP64 iterative refinement
- * (block Jacobi), or PCG on double-float vectors with the FP32 Fourier-space
- * preconditioner (lattice meshes), to the same cg_rtol; the element residual,
+ * (block Jacobi), or on double-float vectors by refinement with the FP32 Fourier-space
+ * inverse, PCG where that gains too little (lattice meshes), to the same cg_rtol; the element residual,
  * condensation and recovery run in double-float arithmetic (FP32 pairs, about
  * 48 significant bits) in the mixed form and in FP64 in the FP64 form.
  * Each stage's solve starts from an extrapolation of the same stage's multipliers in
@@ -266,7 +266,8 @@ int dg_eval_residual(dg_mesh* mesh, double* vals, int on_device);
 int dg_get_diagnostics(dg_mesh* mesh, double out[8]);
 
 /* Facet-solver counters: out[0] CG iterations of the last solve (inner FP32
- * iterations summed over refinement sweeps in the mixed form), out[1] total
+ * iterations summed over refinement sweeps in the mixed form; refinement iterations
+ * on lattice meshes), out[1] total
  * iterations, out[2] solves, out[3] final relative residual of the last solve,
  * out[4] refinement sweeps of the last solve, out[5] total sweeps, out[6] 1 if
  * the Fourier-space (lattice) preconditioner is in use, 2 for the multilevel

@@ -593,14 +593,15 @@ def test_iteration_cap_reports_not_converged(g):
 
 
 @pytest.mark.parametrize("N,k,walls,perturb", [(3, 1, True, 0.0), (17, 2, True, 0.0), (22, 3, False, 0.1),
-                                               (45, 1, False, 0.1), (97, 2, True, 0.0), (300, 1, True, 0.0)])
+                                               (45, 1, False, 0.1), (97, 2, True, 0.0), (420, 1, True, 0.0)])
 @pytest.mark.parametrize("precision", [0, 1])
 def test_multilevel_solver_forms_match_the_host_v_cycle(g, N, k, walls, perturb, precision):
     # the forms a V-cycle takes on the device against the host's: fewer facets than one block's
     # lanes, the coarsest level taking in the level above (17^2, 45^2), operators per stencil class
-    # (walls) and per facet (perturbed), fused levels, and at 300^2 a facet-constant level too large
-    # to fuse above fused ones. FP64: sums of some hundred terms through five levels, 1e-12; FP32:
-    # the same at 2^-24, amplified by the cycle as in the tests above, 1e-5
+    # (walls) and per facet (perturbed), fused levels, and at 420^2 a facet-constant level too large
+    # to fuse above fused ones, with neighbour lists too long for shared memory. FP64: sums of some
+    # hundred terms through five levels, 1e-12; FP32: the same at 2^-24, amplified by the cycle as in
+    # the tests above, 1e-5
     vid, X = synth.split_square_mesh(N, L=1.0, periodic=not walls)
     if perturb:
         rng = np.random.default_rng(N)
