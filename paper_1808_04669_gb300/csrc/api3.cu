@@ -271,7 +271,10 @@ int dg3_mesh_create(int64_t n_tet, const int64_t* tet_vertex_ids, const double* 
       return rc2;
     };
     dgdf::DevMesh& v = M->mv;
-    const bool tables = dgdf::ml_class_tables_fit(hm.nl, 7, true, d.n_stencil);
+    const int slots = dgdf::ml_class_tables_fit(hm.nl, 7, true, d.n_stencil)
+                          ? d.n_stencil
+                          : dgdf::ml_class_slots(hm.nl, 7, true, d.n_stencil, d.n_face, hm.face_stencil.data());
+    const bool tables = slots > 0;
     auto table = [&](int word) {
       return dgdf::ml_operator_table(tables, hm.nl, 7, d.n_stencil, d.n_face, hm.face_stencil.data(),
                                      hm.stencil_blocks.data(), word);
@@ -279,6 +282,7 @@ int dg3_mesh_create(int64_t n_tet, const int64_t* tet_vertex_ids, const double* 
     const std::vector<double> tab4 = table(4);
     std::vector<dgdf::MLLevelT<float>> lv;
     v.ml_ncls = tables ? d.n_stencil : 0;
+    d.ml_nslot = slots;
     if ((rc = upload3(M, &v.ml_tab, table(8))) ||
         (rc = upload3(M, &v.ml_tab_f, std::vector<float>(tab4.begin(), tab4.end()))) ||
         (rc = dgdf::ml_fill<float>(mlh, lv, up, al, d.r, d.z, &v.ml_cpinv_f, &v.ml_xc_f, &v.ml_bc_f, &v.ml_ld)) ||

@@ -34,6 +34,7 @@ struct DevMesh3 {
   const int8_t* tet_nbr_loc;
   const double* face_sigma;           // [n_face]
   const int32_t *face_tet, *face_nbr, *face_stencil;   // [n_face][2], [n_face][6], [n_face]
+  int ml_nslot;                                        // multilevel solver: classes a block holds in shared memory
   const int8_t* face_loc;             // [n_face][2]
   const double *st_blk, *st_binv;     // [n_stencil][7][nl][nl], [n_stencil][nl][nl]
   double *u, *ustage, *h, *gl;        // [n_tet][nd] x3, [n_tet][4 nl]
@@ -60,6 +61,9 @@ cudaError_t launch_pressure3(const DevMesh3& m, double* pe, double* pf, double* 
 // FP64 PCG with the multilevel preconditioner of an assembled hierarchy (k_multilevel.cu): mv
 // holds the hierarchy (ml_*), the PCG vectors r and z, red, bar and stats
 int solver3_ml_blocks(const DevMesh3& m, const DevMesh& mv);
+// where the operators of all face classes don't fit in shared memory: classes a block of the solver
+// holds for its own faces (0: tables per face). cls: [n]
+int ml_class_slots(int nl, int nb, bool fp32, int ncls, int n, const int32_t* cls);
 cudaError_t launch_solve3_ml(const DevMesh3& m, const DevMesh& mv, const SolveArgs& a, int nblocks, cudaStream_t s);
 
 }  // namespace dgdf

@@ -25,13 +25,16 @@
 //   - a facet's modes go to 2 or 4 lanes, one output mode a lane (3-D: three): neighbours' values are
 //     one vector load shared by the lanes, and a phase is a dozen instructions deep;
 //   - each block owns a contiguous run of facets, whose neighbour lists stay in shared memory
-//     for the whole solve, as do the stencil classes' operators (structured meshes have a few
-//     classes; otherwise the facets' own operators are read transposed, coalesced);
+//     for the whole solve, as do the operators of the stencil classes, of all (structured 2-D
+//     meshes have a few) or of its own facets; otherwise the facets' own operators are read
+//     transposed, coalesced;
 //   - fused coarse levels: at 128^2, BDM_3, 13 phases a V-cycle instead of 27.
 // Measured (walls, 128^2, BDM_3, mixed form, per solve of 14.3 iterations): 2.89 ms
 // with a thread a row, 193 blocks of 256 threads and unfused levels; 1.16 ms in this form, of which
 // the barriers take a third, the FP64 pass S p 13 of 74 us an iteration (7.3 of the FP64 pipes).
+#include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "device.cuh"
 #include "device3.cuh"
@@ -53,12 +56,14 @@ constexpr int ml_threads() {
 }
 constexpr int kMLSmemMax = 200 * 1024;   // dynamic shared memory a block may ask for
 constexpr int kMLIdxMax = 64 * 1024;     // of which neighbour lists
+constexpr int kMLMapMax = 2 * (3 * kMLThreads + 192);   // classes a block can number (ints of the scratch)
 
 // The system and the hierarchy as the kernel takes them.
 template <typename R>
 struct MLSys {
   int n;                      // facets
   int ncls;                   // operator tables: classes (0: per facet)
+  int nslot;                  // of which a block holds in shared memory (ncls: all; fewer: ml_context)
   int idx_smem;               // 1: the block's neighbour lists fit in shared memory
   int nlev, nc, ld;
   int has_kernel;
@@ -143,7 +148,7 @@ __device__ __host__ constexpr int ml_vs(int bs) {
 }
 
 // Per-block context: the block's facets [f0, f1), its neighbour lists (shared or global memory,
-// indexed from f0) and the operator tables (shared memory, or per facet in global memory).
+// indexed from f0) and the operator tables (classes in shared memory, or per facet in global memory).
 template <int NL, int NB, typename R>
 struct MLCtx {
   static constexpr int LP = ml_lanes(NL) * ml_modes(NL), RS = ml_row_stride(NL);
@@ -153,7 +158,24 @@ struct MLCtx {
   const int32_t *nbr, *cls;
   const double* tab64;
   const R* tab;
+  const double* gtab64;        // tables of all classes in global memory
+  const R* gtab;
 };
+
+// operators of the class of the block's facet fl (class tables). On faces of tetrahedra c.cls is a
+// slot of the shared tables, or ~class of a class that found no slot
+template <int NL, int NB, typename R, typename T>
+__device__ __forceinline__ const T* ml_class_tab(const MLCtx<NL, NB, R>& c, const T* tab, int fl) {
+  const int s = c.cls[fl];
+  if constexpr (NB == 7) {
+    if (s < 0) {
+      if constexpr (std::is_same<T, R>::value) tab = c.gtab;
+      else tab = c.gtab64;
+      return tab + ~s * ml_class_stride(NL, NB, sizeof(T));
+    }
+  }
+  return tab + s * ml_class_stride(NL, NB, sizeof(T));
+}
 
 // y[q] = (A x)_(i + q) of facet f on the leading BS modes, for the ml_modes(BS) modes of a lane
 template <int NL, int NB, int BS, typename R, typename T>
@@ -171,7 +193,7 @@ __device__ __forceinline__ void ml_apply_row(const MLCtx<NL, NB, R>& c, const T*
 #pragma unroll
   for (int q = 0; q < MP; ++q) y[q] = T(0);
   if (c.classes) {
-    const T* t = tab + c.cls[fl] * ml_class_stride(NL, NB, sizeof(T)) + i * c.RS;
+    const T* t = ml_class_tab<NL, NB, R, T>(c, tab, fl) + i * c.RS;
 #pragma unroll
     for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -198,7 +220,7 @@ __device__ __forceinline__ void ml_binv_row(const MLCtx<NL, NB, R>& c, int f, in
                                             R (&t)[ml_modes(BS)]) {
   constexpr int MP = ml_modes(BS), LB = ml_lanes(BS);
   if constexpr (BS == 1) {
-    t[0] = c.classes ? c.tab[c.cls[f - c.f0] * ml_class_stride(NL, NB, sizeof(R)) + c.BLK + NL * c.RS + 4] * v[0]
+    t[0] = c.classes ? ml_class_tab<NL, NB, R, R>(c, c.tab, f - c.f0)[c.BLK + NL * c.RS + 4] * v[0]
                      : __ldg(c.tab + size_t(c.n) * ((NB + 1) * NL * c.LP + 4) + f) * v[0];
   } else {
     R w[BS];
@@ -208,7 +230,7 @@ __device__ __forceinline__ void ml_binv_row(const MLCtx<NL, NB, R>& c, int f, in
     for (int q = 0; q < MP; ++q) {
       R a[BS];
       if (c.classes) {
-        const R* o = c.tab + c.cls[f - c.f0] * ml_class_stride(NL, NB, sizeof(R)) + c.BLK;
+        const R* o = ml_class_tab<NL, NB, R, R>(c, c.tab, f - c.f0) + c.BLK;
         if constexpr (BS == NL) ld_tab<BS>(o + (i + q) * c.RS, a);
         else ld_tab<BS>(o + NL * c.RS + (i + q) * 2, a);
       } else {
@@ -358,7 +380,7 @@ __device__ __forceinline__ void ml_phase_b(const MLCtx<NL, NB, R>& c, const MLLe
           const int i2 = i & 1;
           R a[2];
           if (c.classes) {
-            ld_tab<2>(c.tab + c.cls[f - c.f0] * ml_class_stride(NL, NB, sizeof(R)) + c.BLK + NL * c.RS + i2 * 2, a);
+            ld_tab<2>(ml_class_tab<NL, NB, R, R>(c, c.tab, f - c.f0) + c.BLK + NL * c.RS + i2 * 2, a);
           } else {
             const R* t = c.tab + size_t(c.n) * (NB + 1) * NL * c.LP;
             a[0] = __ldg(t + size_t(f) * 2 + i2);
@@ -673,16 +695,50 @@ __device__ void ml_context(const MLSys<R>& m, MLCtx<NL, NB, R>& c, MLLevelT<R>* 
   c.classes = m.ncls > 0;
   c.tab64 = m.tab64;
   c.tab = m.tab;
+  c.gtab64 = m.tab64;
+  c.gtab = m.tab;
   unsigned char* next = reinterpret_cast<unsigned char*>(t64);
+  // More classes than fit (faces of tetrahedra only): the block holds those of its own faces, in
+  // the order of their numbers, as far as the slots go. map: class -> slot, or ~class (none left;
+  // it reads the global table), in the reductions' scratch (ml_class_slots bounds ncls).
+  int32_t* map = reinterpret_cast<int32_t*>(scr);
+  const bool local = NB == 7 && m.nslot < m.ncls;
+  if (local) {
+    for (int i = threadIdx.x; i < m.ncls; i += blockDim.x) map[i] = 0;
+    __syncthreads();
+    for (int f = c.f0 + threadIdx.x; f < c.f1; f += blockDim.x) map[__ldg(&m.cls[f])] = 1;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      int used = 0;
+      for (int i0 = 0; i0 < m.ncls; i0 += 32) {
+        const int i = i0 + threadIdx.x;
+        const bool on = i < m.ncls && map[i];
+        const unsigned b = __ballot_sync(0xffffffffu, on);
+        const int slot = used + __popc(b & ((1u << threadIdx.x) - 1));
+        if (i < m.ncls) map[i] = on && slot < m.nslot ? slot : ~i;
+        used += __popc(b);
+      }
+    }
+    __syncthreads();
+  }
   if (c.classes) {
-    const int w64 = m.ncls * ml_class_stride(NL, NB, 8);
-    for (int i = threadIdx.x; i < w64; i += blockDim.x) t64[i] = __ldg(&m.tab64[i]);
-    c.tab64 = t64;
+    const int w64 = m.nslot * ml_class_stride(NL, NB, 8);
     next += size_t(w64) * 8;
+    auto fill = [&](auto* dst, const auto* src, int st) {
+      if (!local) {
+        for (int i = threadIdx.x; i < m.ncls * st; i += blockDim.x) dst[i] = __ldg(&src[i]);
+      } else {
+        for (int k = threadIdx.x >> 5; k < m.ncls; k += blockDim.x >> 5)
+          if (map[k] >= 0)
+            for (int i = threadIdx.x & 31; i < st; i += 32) dst[map[k] * st + i] = __ldg(&src[size_t(k) * st + i]);
+      }
+    };
+    fill(t64, m.tab64, ml_class_stride(NL, NB, 8));
+    c.tab64 = t64;
     if constexpr (std::is_same<R, float>::value) {
       float* t32 = reinterpret_cast<float*>(next);
-      const int w32 = m.ncls * ml_class_stride(NL, NB, 4);
-      for (int i = threadIdx.x; i < w32; i += blockDim.x) t32[i] = __ldg(&m.tab[i]);
+      const int w32 = m.nslot * ml_class_stride(NL, NB, 4);
+      fill(t32, m.tab, ml_class_stride(NL, NB, 4));
       c.tab = t32;
       next += size_t(w32) * 4;
     } else {
@@ -695,7 +751,10 @@ __device__ void ml_context(const MLSys<R>& m, MLCtx<NL, NB, R>& c, MLLevelT<R>* 
     int32_t* idx = reinterpret_cast<int32_t*>(next);
     const int nf = c.f1 - c.f0;
     for (int i = threadIdx.x; i < nf * (NB - 1); i += blockDim.x) idx[i] = __ldg(&c.nbr[i]);
-    for (int i = threadIdx.x; i < nf; i += blockDim.x) idx[nf * (NB - 1) + i] = __ldg(&c.cls[i]);
+    for (int i = threadIdx.x; i < nf; i += blockDim.x) {
+      const int k = __ldg(&c.cls[i]);
+      idx[nf * (NB - 1) + i] = local ? map[k] : k;
+    }
     c.nbr = idx;
     c.cls = idx + nf * (NB - 1);
   }
@@ -930,6 +989,7 @@ template <typename R>
 MLSys<R> ml_system(const DevMesh& v) {
   MLSys<R> s{};
   s.ncls = v.ml_ncls;
+  s.nslot = v.ml_ncls;
   s.nlev = v.ml_nlev;
   s.nc = v.ml_nc;
   s.ld = v.ml_ld;
@@ -973,6 +1033,7 @@ template <typename R>
 MLSys<R> ml_system(const DevMesh3& m, const DevMesh& v) {
   MLSys<R> s = ml_system<R>(v);
   s.n = m.n_face;
+  s.nslot = m.ml_nslot;
   s.nbr = m.face_nbr;
   s.cls = m.face_stencil;
   s.has_kernel = 1;   // closed mesh: the constant multiplier is the kernel of S
@@ -984,12 +1045,18 @@ MLSys<R> ml_system(const DevMesh3& m, const DevMesh& v) {
 }
 
 // Blocks of the solver's grid: one per SM, fewer on meshes that would leave a block less than
-// two warps of facet lanes. Also lets the kernel use its shared memory. 0: it does not fit.
+// two warps of facet lanes.
+int ml_want_blocks(int nl, int n, int sms) {
+  const int want = (n * ml_lanes(nl) + 63) / 64;
+  return want < 1 ? 1 : (want < sms ? want : sms);
+}
+
+// The grid's blocks. Also lets the kernel use its shared memory. 0: it does not fit.
 int ml_blocks(const void* fn, int threads, int nl, int nb, bool fp32, int ncls, int n, int* fit = nullptr) {
   int dev = 0, sms = 0, per_sm = 0, idx = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int want = (n * ml_lanes(nl) + 63) / 64, blocks = want < 1 ? 1 : (want < sms ? want : sms);
+  const int blocks = ml_want_blocks(nl, n, sms);
   const size_t smem = ml_smem(nl, nb, fp32, ncls, n, blocks, &idx);
   if (!fn || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMLSmemMax) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess || per_sm < 1) {
@@ -1003,8 +1070,10 @@ int ml_blocks(const void* fn, int threads, int nl, int nb, bool fp32, int ncls, 
 template <int NL, int NB, typename R, typename Mesh>
 cudaError_t ml_launch(const Mesh& mesh, const DevMesh& v, const SolveArgs& a, int nblocks, cudaStream_t s) {
   MLSys<R> sys = ml_system<R>(mesh, v);
-  const size_t smem = ml_smem(NL, NB, std::is_same<R, float>::value, sys.ncls, sys.n, nblocks, &sys.idx_smem);
+  const size_t smem = ml_smem(NL, NB, std::is_same<R, float>::value, sys.nslot, sys.n, nblocks, &sys.idx_smem);
   if (sys.nlev < 1 || sys.nlev > kMLMaxLevels || smem > size_t(kMLSmemMax)) return cudaErrorInvalidValue;
+  // a block's own classes are numbered in its neighbour lists' shared memory
+  if (sys.nslot < sys.ncls && (NB != 7 || !sys.idx_smem || sys.ncls > kMLMapMax)) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(sys.bar, 0, sizeof(GridBar), s);
   if (e != cudaSuccess) return e;
   Mesh mm = mesh;
@@ -1017,7 +1086,7 @@ cudaError_t ml_launch(const Mesh& mesh, const DevMesh& v, const SolveArgs& a, in
 template <int NL, typename R>
 cudaError_t ml_launch_apply(const DevMesh& v, const double* r, double* z, int nblocks, cudaStream_t s) {
   MLSys<R> sys = ml_system<R>(v, v);
-  const size_t smem = ml_smem(NL, 5, std::is_same<R, float>::value, sys.ncls, sys.n, nblocks, &sys.idx_smem);
+  const size_t smem = ml_smem(NL, 5, std::is_same<R, float>::value, sys.nslot, sys.n, nblocks, &sys.idx_smem);
   if (sys.nlev < 1 || sys.nlev > kMLMaxLevels || smem > size_t(kMLSmemMax)) return cudaErrorInvalidValue;
   const void* fn = (const void*)k_ml_apply<NL, 5, R>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMLSmemMax);
@@ -1033,6 +1102,37 @@ cudaError_t ml_launch_apply(const DevMesh& v, const double* r, double* z, int nb
 bool ml_class_tables_fit(int nl, int nb, bool fp32, int ncls) {
   int idx = 0;
   return ml_smem(nl, nb, fp32, ncls, 1, 1, &idx) + kMLIdxMax <= size_t(kMLSmemMax);
+}
+
+// Blocks' own class tables, where the tables of all classes don't fit. A periodic Kuhn cube has 120
+// classes (the wrapped vertex ids order 48 kinds of tetrahedra), 437 KB at k = 2, but a block of
+// 324 faces meets 12 to 60 of them, and some 45 fit. With a table per face a V-cycle and the product
+// with S streamed 340 MB from HBM each iteration (ncu): 140 us, with the slots 110 (16^3, k = 2;
+// 15.9 -> 13.3 ms a step).
+// Slots a block, or 0 where this does not pay: where more than a quarter of some block's faces would
+// have to read the global table, scattered over its lanes, the tables per face are read coalesced.
+int ml_class_slots(int nl, int nb, bool fp32, int ncls, int n, const int32_t* cls) {
+  int dev = 0, sms = 152, idx = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int blocks = ml_want_blocks(nl, n, sms), share = (n + blocks - 1) / blocks;
+  const size_t none = ml_smem(nl, nb, fp32, 0, n, blocks, &idx), one = ml_smem(nl, nb, fp32, 1, n, blocks, &idx) - none;
+  if (!idx || ncls > kMLMapMax || none + one > size_t(kMLSmemMax)) return 0;
+  const int fit = int((size_t(kMLSmemMax) - none) / one);
+  int most = 0;
+  std::vector<int32_t> own;
+  for (int f0 = 0; f0 < n; f0 += share) {
+    own.assign(cls + f0, cls + std::min(n, f0 + share));
+    std::sort(own.begin(), own.end());
+    int used = 0, over = 0;
+    for (size_t i = 0; i < own.size(); ++i) {
+      used += i == 0 || own[i] != own[i - 1];
+      over += used > fit;
+    }
+    if (over * 4 > int(own.size())) return 0;
+    most = std::max(most, std::min(used, fit));
+  }
+  return most;
 }
 
 int ml_grid_threads() {
@@ -1071,8 +1171,8 @@ cudaError_t launch_solve_ml(const DevMesh& m, const SolveArgs& a, int nblocks, c
 
 // the three-dimensional path runs its V-cycle in FP32
 int solver3_ml_blocks(const DevMesh3& m, const DevMesh& mv) {
-  if (m.k == 1) return ml_blocks((const void*)k_solve_ml<3, 7, float, DevMesh3>, ml_threads<3, float>(), 3, 7, true, mv.ml_ncls, m.n_face);
-  if (m.k == 2) return ml_blocks((const void*)k_solve_ml<6, 7, float, DevMesh3>, ml_threads<6, float>(), 6, 7, true, mv.ml_ncls, m.n_face);
+  if (m.k == 1) return ml_blocks((const void*)k_solve_ml<3, 7, float, DevMesh3>, ml_threads<3, float>(), 3, 7, true, m.ml_nslot, m.n_face);
+  if (m.k == 2) return ml_blocks((const void*)k_solve_ml<6, 7, float, DevMesh3>, ml_threads<6, float>(), 6, 7, true, m.ml_nslot, m.n_face);
   return 0;
 }
 

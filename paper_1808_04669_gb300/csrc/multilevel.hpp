@@ -109,7 +109,7 @@ void fuse_levels(MLHost& ml, int word, int dense_max, int grid_threads);
 // Per-class operator tables of the solver kernel (class_tables = true): for each stencil class its
 // nb blocks [nb][nl][rs], the block-Jacobi inverse of all modes [nl][rs], of the leading two modes
 // [2][2] and of mode 0 (then 3 words of padding), rs = ml_row_stride(nl), classes ml_class_stride
-// apart. Otherwise (more classes than fit in shared memory) one set a facet, transposed so that the
+// apart. Otherwise (more classes than a block can hold) one set a facet, transposed so that the
 // lanes of a warp read consecutive words: [nb][nl (column)][facet][lanes x modes], then the three
 // inverses [nl][facet][lanes x modes], [2][facet][2], [facet].
 std::vector<double> ml_operator_table(bool class_tables, int nl, int nb, int n_cls, int n, const int32_t* cls,

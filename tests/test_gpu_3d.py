@@ -245,3 +245,24 @@ def test_residual_tiles_match_the_oracle(g, N, k, nu, perturb):
     d = Discretization3(vid, X, k, nu)
     ref = d.to_lattice(d.riesz(d.residual(d.from_lattice(v))))
     assert np.linalg.norm(mesh.eval_residual() - ref) < 1e-12 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("N,k,shuffle", [(3, 1, False), (5, 2, False), (16, 1, False), (16, 2, False), (10, 2, True)])
+def test_multilevel_operator_tables_match_block_jacobi(g, N, k, shuffle):
+    # where the solver's blocks read the face operators: class tables of the block's own faces, all
+    # of them (N = 3 and 5, fewer faces a block than classes; k = 1) or some left in global memory
+    # (16^3, k = 2), and tables per face (elements shuffled: every block meets every class). The
+    # block-Jacobi solver reads none of them and meets the same rtol 1e-13, so that the projections
+    # differ by that times sqrt(cond(S)) (below 1e3 N), with a factor of ten to spare
+    vid, X = kuhn_cube_mesh(N)
+    if shuffle:
+        order = np.random.default_rng(N).permutation(len(vid))
+        vid, X = np.ascontiguousarray(vid[order]), np.ascontiguousarray(X[order])
+    v = field(X, k, N)
+    out = []
+    for pc in (g.PRECOND_AUTO, g.PRECOND_BLOCK_JACOBI):
+        m = g.DGMesh3(vid, X, k, 0.0, precond=pc)
+        m.set_velocity(v)
+        m.project_divfree()
+        out.append(m.get_velocity())
+    assert rel(out[0], out[1]) < 1e-13 * np.sqrt(1e3 * N) * 10
