@@ -722,14 +722,14 @@ def run_three_d(args, g, stream, flush):
 
 
 def stage3_flops_per_tet(k):
-    """Flops of the 3-D residual per tetrahedron (FMA = 2), counted from its loops: volume points
-    (3k+1)//2 cubed, each evaluating u and grad u (12 ns) and testing (9 ns) plus the flux (~40);
-    four faces of ((3k+2)//2)^2 points, each evaluating both traces and normal derivatives (18 ns)
-    and testing (9 ns) plus ~30."""
+    """Flops of the 3-D residual per tetrahedron (FMA = 2), counted from the tiled kernel's loops:
+    u and grad u at (3k+1)//2 cubed volume points (12 ns) and their flux (~60), traces and normal
+    derivatives at ((3k+2)//2)^2 points of four faces (12 ns) and their flux (~25); each of the 3 ns
+    test functions sums 3 terms a volume point and 2 a face point."""
     ns = (k + 1) * (k + 2) * (k + 3) // 6
     nq = ((3 * k + 1) // 2) ** 3
-    nqf = ((3 * k + 2) // 2) ** 2
-    fma = nq * (21 * ns + 40) + 4 * nqf * (27 * ns + 30)
+    nqf = 4 * ((3 * k + 2) // 2) ** 2
+    fma = nq * (12 * ns + 60) + nqf * (12 * ns + 25) + 3 * ns * (3 * nq + 2 * nqf)
     return 2 * fma
 
 
