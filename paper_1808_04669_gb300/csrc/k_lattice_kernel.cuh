@@ -923,7 +923,9 @@ __device__ __forceinline__ void add_square(dacc& a, dfl v) {
 
 // Iterative refinement. Returns 0 when the solve ended (st.conv, st.relres and it are set), -1 when
 // a barrier's wait ran out, 1 when lat_pcg has to take the solve from its start, 2 when it has to
-// go on from lam (the history has moved then).
+// go on from lam (the history has moved then). A start that is farther off than zero (multipliers of
+// another state, or not finite) is dropped: against it rounding, eps |S lam0|, would stay in lam and
+// the recursive residual would not show it.
 template <int K, bool MIXED>
 __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, const LatCtx<K, MIXED>& L,
                                           const typename LatT<MIXED>::V* S, Barrier& bar,
@@ -940,7 +942,8 @@ __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, 
   V* hist1 = static_cast<V*>(a.hist1);
   V* hist2 = static_cast<V*>(a.hist2);
   V* hnew = static_cast<V*>(a.hist_new);
-  const bool use2 = a.c2 != 0.0, lam0 = hist1 || a.warm_scale != 0.0;
+  const bool use2 = a.c2 != 0.0;
+  bool lam0 = hist1 || a.warm_scale != 0.0;   // false: start from zero
   // (S x)_i from the lanes' x of the five facets
   auto product = [&](const A (&x)[5], int cls, int i) {
     Acc acc = acc_zero(Acc{});
@@ -951,66 +954,72 @@ __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, 
       for (int j = 0; j < NL; ++j) mad(acc, lat_entry<NL>(row, b * NL * NL + j, A{}), shfl_lane(x[b], j, LP));
     return fin(acc);
   };
-  // g from both sides of every facet, the warm start lam0 = c1 hist1 + c2 hist2 (or warm_scale lam,
-  // or zero) and r = g - S lam0 in one pass: a facet forms its neighbours' lam0 from the history
-  // with the same operations as they do, so that lam0 is the same bits wherever it is formed
-  Acc s4[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) s4[i] = acc_zero(Acc{});
-  lat_facets<NL>(nF, [&](int f, int i, bool live) {
-    const size_t o = size_t(f) * VS + i;
-    const A g = lat_g(m, f, i, A{});
-    A r = g;
-    if (lam0) {
-      const int4 nb = __ldg(reinterpret_cast<const int4*>(m.facet_nbr) + f);
-      const int n5[5] = {f, nb.x, nb.y, nb.z, nb.w};
-      const int cls = __ldg(&m.facet_stencil[f]);
-      const V* src = hist1 ? hist1 : L.lam;
-      A x[5], x2[5];
-#pragma unroll
-      for (int b = 0; b < 5; ++b) x[b] = ldv(src + size_t(n5[b]) * VS + i);
-      if (hist1 && use2) {
-#pragma unroll
-        for (int b = 0; b < 5; ++b) x2[b] = ldv(hist2 + size_t(n5[b]) * VS + i);
-#pragma unroll
-        for (int b = 0; b < 5; ++b) x[b] = hc1 * x[b] + hc2 * x2[b];
-      } else {
-        const A c = hist1 ? hc1 : warm;
-#pragma unroll
-        for (int b = 0; b < 5; ++b) x[b] = c * x[b];
-      }
-      r = g - product(x, cls, i);
-      if (hist1 && live) stv(L.lam + o, x[0]);
-    }
-    if (!live) return;
-    stv(L.r + o, r);
-    add_square(s4[0], g);
-    add_square(s4[1], r);
-    if (i == 0) {
-      acc_add(s4[2], g);
-      acc_add(s4[3], r);
-    }
-  });
   // thread 0's own: the squared norms (scaled), without the constant-multiplier component
   double stop2 = 0.0, floor2 = 0.0, gg = 0.0, rr = 0.0;
   const double f2 = MIXED ? double(kLatScale) * double(kLatScale) : 1.0;
-  if (!lat_reduce<4>(m, bar, 4, s4, scr, [&](const double (&t)[4]) {
-        const double inv = 1.0 / double(nF);
-        gg = t[0] - t[2] * t[2] * f2 * inv;
-        rr = fmax(t[1] - t[3] * t[3] * f2 * inv, 0.0);
-        stop2 = a.rtol * a.rtol * gg;
-        floor2 = a.floor_rtol * a.floor_rtol * gg;
-        sc.mean = A(t[3] * inv);
-        sc.conv = 0;
-        sc.done = 0;
-        if (!(stop2 >= (MIXED ? kLatSumMin * 1e-22 : 1e-280) && gg <= (MIXED ? kLatSumMax : 1e280) && rr <= 1e280)) {
-          sc.done = 3;   // out of range, zero or not finite
-        } else if (rr <= stop2) {
-          sc.done = sc.conv = 1;
-          sc.relres = sqrt(rr / gg);
+  // g from both sides of every facet, the warm start lam0 = c1 hist1 + c2 hist2 (or warm_scale lam,
+  // or zero) and r = g - S lam0 in one pass: a facet forms its neighbours' lam0 from the history
+  // with the same operations as they do, so that lam0 is the same bits wherever it is formed
+  for (;; lam0 = false) {
+    Acc s4[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s4[i] = acc_zero(Acc{});
+    lat_facets<NL>(nF, [&](int f, int i, bool live) {
+      const size_t o = size_t(f) * VS + i;
+      const A g = lat_g(m, f, i, A{});
+      A r = g;
+      if (lam0) {
+        const int4 nb = __ldg(reinterpret_cast<const int4*>(m.facet_nbr) + f);
+        const int n5[5] = {f, nb.x, nb.y, nb.z, nb.w};
+        const int cls = __ldg(&m.facet_stencil[f]);
+        const V* src = hist1 ? hist1 : L.lam;
+        A x[5], x2[5];
+#pragma unroll
+        for (int b = 0; b < 5; ++b) x[b] = ldv(src + size_t(n5[b]) * VS + i);
+        if (hist1 && use2) {
+#pragma unroll
+          for (int b = 0; b < 5; ++b) x2[b] = ldv(hist2 + size_t(n5[b]) * VS + i);
+#pragma unroll
+          for (int b = 0; b < 5; ++b) x[b] = hc1 * x[b] + hc2 * x2[b];
+        } else {
+          const A c = hist1 ? hc1 : warm;
+#pragma unroll
+          for (int b = 0; b < 5; ++b) x[b] = c * x[b];
         }
-      }))
-    return -1;
+        r = g - product(x, cls, i);
+        if (hist1 && live) stv(L.lam + o, x[0]);
+      }
+      if (!live) return;
+      stv(L.r + o, r);
+      add_square(s4[0], g);
+      add_square(s4[1], r);
+      if (i == 0) {
+        acc_add(s4[2], g);
+        acc_add(s4[3], r);
+      }
+    });
+    // (a second pass sums in other slots: blocks may still read the first one's)
+    if (!lat_reduce<4>(m, bar, lam0 ? 4 : 0, s4, scr, [&](const double (&t)[4]) {
+          const double inv = 1.0 / double(nF);
+          gg = t[0] - t[2] * t[2] * f2 * inv;
+          rr = nonneg(t[1] - t[3] * t[3] * f2 * inv);
+          stop2 = a.rtol * a.rtol * gg;
+          floor2 = a.floor_rtol * a.floor_rtol * gg;
+          sc.mean = A(t[3] * inv);
+          sc.conv = 0;
+          sc.done = 0;
+          if (!(stop2 >= (MIXED ? kLatSumMin * 1e-22 : 1e-280) && gg <= (MIXED ? kLatSumMax : 1e280))) {
+            sc.done = 3;   // out of range, zero or not finite
+          } else if (lam0 && !(rr <= gg)) {
+            sc.done = 4;
+          } else if (rr <= stop2) {
+            sc.done = sc.conv = 1;
+            sc.relres = sqrt(rr / gg);
+          }
+        }))
+      return -1;
+    if (sc.done != 4) break;
+  }
   if (sc.done == 3) return 1;
   const bool at_once = sc.done != 0;
   while (!sc.done) {
@@ -1071,7 +1080,7 @@ __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, 
     const int n = it;
     if (!lat_reduce<2>(m, bar, n & 1 ? 0 : 2, s2, scr, [&](const double (&t)[2]) {
           const double inv = 1.0 / double(nF), prev = rr;
-          rr = fmax(t[0] - t[1] * t[1] * f2 * inv, 0.0);
+          rr = nonneg(t[0] - t[1] * t[1] * f2 * inv);
           sc.mean = A(t[1] * inv);
           sc.relres = sqrt(rr / gg);
           if (!isfinite(rr)) {
@@ -1098,7 +1107,7 @@ __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, 
         ldf<NL, VS>(hist1 + o, hv);
         stf<NL, VS>(hist2 + o, hv);
       }
-      if (!hist1) {
+      if (!(hist1 && lam0)) {
 #pragma unroll
         for (int j = 0; j < NL; ++j) lv[j] = A(0);
         if (lam0) {
@@ -1138,10 +1147,11 @@ __device__ __forceinline__ bool grid_reduce_pair(const DevMesh& m, Barrier& bar,
 }
 
 // The solve as PCG preconditioned by B, on the system scaled by the size of g: for systems where
-// refinement gains too little, or whose size is outside the range of its sums. Returns false when
-// a barrier's wait ran out.
+// refinement gains too little, or whose size is outside the range of its sums. Returns 0 when the
+// solve ended, -1 when a barrier's wait ran out, 1 when the start is farther off than zero (the
+// history has moved; call again without it).
 template <int K, bool MIXED>
-__device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const LatCtx<K, MIXED>& L,
+__device__ __noinline__ int lat_pcg(const DevMesh& m, const SolveArgs& a, const LatCtx<K, MIXED>& L,
                                      typename LatT<MIXED>::V* p, Barrier& bar, LatScal<typename LatT<MIXED>::A>& sc,
                                      typename LatT<MIXED>::Acc (*scr)[kLatThreads], int& it) {
   using T = LatT<MIXED>;
@@ -1196,7 +1206,7 @@ __device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const
   double gg[2];
   {
     // FP64 sums (the squares of any g fit), through the double slots of the scratch
-    if (!grid_reduce_pair(m, bar, 4, ga, acc_val(g0), gg)) return false;
+    if (!grid_reduce_pair(m, bar, 4, ga, acc_val(g0), gg)) return -1;
   }
   const double c0 = gg[1] / double(nF);
   const double gnorm0 = sqrt(fmax(gg[0] - gg[1] * gg[1] / double(nF), 0.0));
@@ -1241,7 +1251,7 @@ __device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const
         for (int j = 0; j < NL; ++j) y[j] = gv[j] - y[j];
         stf<NL, VS>(L.r + o, y);
       }
-      if (!grid_sync(bar, m.stats)) return false;
+      if (!grid_sync(bar, m.stats)) return -1;
     }
     // z = M r
     // The constant multiplier is in the kernel of S and of the preconditioner, so PCG cannot
@@ -1270,11 +1280,13 @@ __device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const
       });
     }
     double rr[2];
-    if (!lat_sums<2>(m, bar, 6, rra, scr, sc, rr)) return false;
+    if (!lat_sums<2>(m, bar, 6, rra, scr, sc, rr)) return -1;
     double cmode = rr[1] / double(nF);
-    rr[0] = fmax(rr[0] - rr[1] * rr[1] / double(nF), 0.0);
+    rr[0] = nonneg(rr[0] - rr[1] * rr[1] / double(nF));
+    // (gnorm is that of g's leading words: up to its rounding)
+    if ((hist1 || a.warm_scale != 0.0) && !(rr[0] <= gnorm * gnorm * 1.0001)) return 1;
     columns<K, MIXED>(L);
-    if (!grid_sync(bar, m.stats)) return false;
+    if (!grid_sync(bar, m.stats)) return -1;
     Acc rza[2] = {acc_zero(Acc{}), acc_zero(Acc{})};
     rows_inverse<K, MIXED>(L, [&](size_t o, const Z (&zv)[NL]) {
       A rv[NL];
@@ -1286,7 +1298,7 @@ __device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const
     {
       const Acc rz1[1] = {rza[0]};
       double rzt[1];
-      if (!lat_sums<1>(m, bar, 1, rz1, scr, sc, rzt)) return false;
+      if (!lat_sums<1>(m, bar, 1, rz1, scr, sc, rzt)) return -1;
       rz[0] = rzt[0];
     }
     double rho = rz[0], rrv = rr[0];
@@ -1338,7 +1350,7 @@ __device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const
         stf<NL, VS>(L.q + o, qv);
       }
       double pq[1];
-      if (!lat_sums<1>(m, bar, 0, pqa, scr, sc, pq)) return false;
+      if (!lat_sums<1>(m, bar, 0, pqa, scr, sc, pq)) return -1;
       if (threadIdx.x == 0) {
         sc.done = 0;
         if (!(pq[0] > 0.0)) {
@@ -1375,10 +1387,10 @@ __device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const
           stf<NL, VS>(L.lam + o, lv);
         });
       }
-      if (!lat_sums<2>(m, bar, 6, rra, scr, sc, rr)) return false;
+      if (!lat_sums<2>(m, bar, 6, rra, scr, sc, rr)) return -1;
       cmode = rr[1] / double(nF);
       const double rr_prev = rrv;
-      rrv = fmax(rr[0] - rr[1] * rr[1] / double(nF), 0.0);
+      rrv = nonneg(rr[0] - rr[1] * rr[1] / double(nF));
       if (threadIdx.x == 0) {
         sc.done = 0;
         sc.conv = 0;
@@ -1398,7 +1410,7 @@ __device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const
         break;
       }
       columns<K, MIXED>(L);
-      if (!grid_sync(bar, m.stats)) return false;
+      if (!grid_sync(bar, m.stats)) return -1;
       rza[0] = acc_zero(Acc{});
       rza[1] = acc_zero(Acc{});
       rows_inverse<K, MIXED>(L, [&](size_t o, const Z (&zv)[NL]) {
@@ -1412,7 +1424,7 @@ __device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const
           mad(rza[0], rv[j], zv[j]);
         }
       });
-      if (!lat_sums<2>(m, bar, 1, rza, scr, sc, rz)) return false;
+      if (!lat_sums<2>(m, bar, 1, rza, scr, sc, rz)) return -1;
       // flexible (Polak-Ribiere) beta: the FP32 preconditioner is symmetric only up to rounding
       beta = (rz[0] - rz[1]) / rho;
       rho = rz[0];
@@ -1420,7 +1432,7 @@ __device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const
   }
   if (a.hist_new) {
     V* hnew = static_cast<V*>(a.hist_new);
-    if (!grid_sync(bar, m.stats)) return false;
+    if (!grid_sync(bar, m.stats)) return -1;
     for (int f = gtid; f < nF; f += gsz) {
       A lv[NL];
       ldf<NL, VS>(L.lam + size_t(f) * VS, lv);
@@ -1432,7 +1444,7 @@ __device__ __noinline__ bool lat_pcg(const DevMesh& m, const SolveArgs& a, const
     sc.conv = conv ? 1 : 0;
     sc.relres = relres;
   }
-  return true;
+  return 0;
 }
 
 // One solve: refinement, and PCG where it does not do.
@@ -1504,7 +1516,14 @@ __global__ void __launch_bounds__(kLatThreads, 2) k_solve_lat(DevMesh m, SolveAr
       b.hist1 = nullptr;
       b.warm_scale = 1.0;
     }
-    if (!grid_sync(bar, m.stats) || !lat_pcg<K, MIXED>(m, b, L, p, bar, sc, scr, it)) return;
+    if (!grid_sync(bar, m.stats)) return;
+    for (;;) {
+      const int left = lat_pcg<K, MIXED>(m, b, L, p, bar, sc, scr, it);
+      if (left < 0) return;
+      if (left == 0) break;
+      b.hist1 = nullptr;
+      b.warm_scale = 0.0;
+    }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     DevStats* st = m.stats;

@@ -70,6 +70,10 @@ __device__ bool grid_sync(Barrier& b, DevStats* st) {
   return ok != 0;
 }
 
+// A squared norm that rounding made negative is zero; NaN stays (fmax would drop it, and a solve
+// that has broken down would count as converged).
+__device__ __forceinline__ double nonneg(double v) { return v < 0.0 ? 0.0 : v; }
+
 // Writes N block partials to red slots, synchronises the grid, and returns
 // the grid sums in every thread (same summation order in every block).
 template <int N>

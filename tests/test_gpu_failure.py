@@ -97,3 +97,28 @@ def test_energy_watchdog_quiet_under_cfl_and_fires_above_it(g, precision):
     mesh.set_velocity(v)
     mesh.project_divfree()
     mesh.rk3_step(40 * dt, 1)
+
+
+@pytest.mark.parametrize("precision,size0,dt0,size,dt", [(1, 1e8, 1e-2, 1.0, 1e-2), (1, 1e8, 1e-2, 1e-15, 1.0),
+                                                         (1, 1e12, 1e-2, 1e9, 1e-13), (0, 1e8, 1e-2, 1.0, 1e-2),
+                                                         (0, 1e70, 1e10, 1e-30, 1e20)])
+def test_lattice_solve_drops_a_start_far_from_the_solution(g, precision, size0, dt0, size, dt):
+    # a state that has nothing to do with the multipliers of the last steps, smaller by so much that
+    # the residual of the extrapolated start overflows its sums or leaves its rounding in the result:
+    # the steps agree with those of a fresh mesh. Both meet rtol 1e-13, so that they differ by that
+    # times sqrt(cond(S)) (below 1e3 N), with a factor of ten to spare
+    N, k = 16, 2
+    vid, X = synth.split_square_mesh(N, L=1.0)
+    mesh = g.DGMesh(vid, X, k, 0.0, precision=precision)
+    fresh = g.DGMesh(vid, X, k, 0.0, precision=precision)
+    mesh.set_velocity(size0 * random_lattice(2 * N * N, k, 5))
+    mesh.step(dt0, 1, g.EULER)
+    for m in (mesh, fresh):
+        m.set_velocity(size * random_lattice(2 * N * N, k, 6))
+    for _ in range(3):
+        out = []
+        for m in (mesh, fresh):
+            m.step(dt, 1, g.EULER)
+            out.append(m.get_velocity() / size)
+        assert np.isfinite(out[1]).all()
+        assert np.linalg.norm(out[0] - out[1]) < 1e-13 * np.sqrt(1e3 * N) * 10 * np.linalg.norm(out[1])
