@@ -428,21 +428,27 @@ bool invert_spd(Vec& A, int n) {
 
 // Pseudo-inverse of the coarsest operator A (symmetric positive semi-definite, nc rows), dense,
 // symmetrised. Up to 256 rows: from its eigen-decomposition, the eigenvalues below 1e-10 of the
-// largest dropped. Larger (the Jacobi eigensolver's cost grows as nc^3 per sweep): when the
-// near-null vector v is in the kernel (|A v| <= 1e-9 |A|_F |v|, a closed mesh), through the
-// definite matrix B = A + s u u^T (u = v / |v|, s the mean diagonal entry), whose inverse is
-// A^+ + u u^T / s, so that A^+ = B^-1 - u u^T / s; otherwise (A definite) A^-1. Both by
-// symmetric sweeps (invert_spd). Returns false if the matrix is not definite.
+// largest dropped. Larger (the Jacobi eigensolver's cost grows as nc^3 per sweep): for each part of
+// the mesh that shares no facet with the others (a connected component of A), when the near-null
+// vector v restricted to it is in the kernel (|A v| <= 1e-9 |A|_F |v|, a closed part), through the
+// definite matrix B = A + s u u^T (u = v / |v| on the part, s the mean diagonal entry), whose inverse
+// is A^+ + u u^T / s, so that A^+ = B^-1 - u u^T / s; otherwise (A definite there) A^-1. Both by
+// symmetric sweeps (invert_spd), or where rounding leaves them a pivot that is not positive, by
+// elimination with pivoting. Returns false if that fails, too.
 bool coarse_pinv(const CsrHost& A, const Vec& v, Vec& out) {
   const int nc = A.n_rows;
-  Vec D(size_t(nc) * nc, 0.0);
-  for (int r = 0; r < nc; ++r)
-    for (int p = A.rp[r]; p < A.rp[r + 1]; ++p) D[size_t(r) * nc + A.ci[p]] += A.v[p];
-  for (int r = 0; r < nc; ++r)
-    for (int c = r + 1; c < nc; ++c) {
-      const double h = 0.5 * (D[size_t(r) * nc + c] + D[size_t(c) * nc + r]);
-      D[size_t(r) * nc + c] = D[size_t(c) * nc + r] = h;
-    }
+  Vec D;
+  auto dense = [&] {
+    D.assign(size_t(nc) * nc, 0.0);
+    for (int r = 0; r < nc; ++r)
+      for (int p = A.rp[r]; p < A.rp[r + 1]; ++p) D[size_t(r) * nc + A.ci[p]] += A.v[p];
+    for (int r = 0; r < nc; ++r)
+      for (int c = r + 1; c < nc; ++c) {
+        const double h = 0.5 * (D[size_t(r) * nc + c] + D[size_t(c) * nc + r]);
+        D[size_t(r) * nc + c] = D[size_t(c) * nc + r] = h;
+      }
+  };
+  dense();
   out.assign(size_t(nc) * nc, 0.0);
   if (nc <= 256) {
     Vec ev, V;
@@ -457,25 +463,57 @@ bool coarse_pinv(const CsrHost& A, const Vec& v, Vec& out) {
     }
     return true;
   }
-  double fro = 0.0, vv = 0.0, avv = 0.0, tr = 0.0;
-  for (double x : D) fro += x * x;
+  // components of A's graph
+  std::vector<int32_t> comp(nc, -1), todo;
+  int ncomp = 0;
+  for (int r0 = 0; r0 < nc; ++r0) {
+    if (comp[r0] >= 0) continue;
+    comp[r0] = ncomp;
+    todo.assign(1, r0);
+    while (!todo.empty()) {
+      const int r = todo.back();
+      todo.pop_back();
+      for (int c = 0; c < nc; ++c)
+        if (D[size_t(r) * nc + c] != 0.0 && comp[c] < 0) {
+          comp[c] = ncomp;
+          todo.push_back(c);
+        }
+    }
+    ++ncomp;
+  }
+  Vec fro(ncomp, 0.0), vv(ncomp, 0.0), avv(ncomp, 0.0);
+  double tr = 0.0;
   for (int r = 0; r < nc; ++r) {
+    const int q = comp[r];
     double y = 0.0;
-    for (int c = 0; c < nc; ++c) y += D[size_t(r) * nc + c] * v[c];
-    avv += y * y;
-    vv += v[r] * v[r];
+    for (int c = 0; c < nc; ++c) {
+      fro[q] += D[size_t(r) * nc + c] * D[size_t(r) * nc + c];
+      y += D[size_t(r) * nc + c] * v[c];
+    }
+    avv[q] += y * y;
+    vv[q] += v[r] * v[r];
     tr += D[size_t(r) * nc + r];
   }
-  const bool kernel = vv > 0.0 && std::sqrt(avv) <= 1e-9 * std::sqrt(fro) * std::sqrt(vv);
   const double s = tr / nc;
-  if (kernel)
+  std::vector<char> kernel(ncomp);
+  for (int q = 0; q < ncomp; ++q)
+    kernel[q] = vv[q] > 0.0 && std::sqrt(avv[q]) <= 1e-9 * std::sqrt(fro[q]) * std::sqrt(vv[q]);
+  auto shift = [&] {   // += s u u^T of the closed parts
     for (int r = 0; r < nc; ++r)
-      for (int c = 0; c < nc; ++c) D[size_t(r) * nc + c] += s * v[r] * v[c] / vv;
-  if (!invert_spd(D, nc)) return false;
+      if (kernel[comp[r]])
+        for (int c = 0; c < nc; ++c)
+          if (comp[c] == comp[r]) D[size_t(r) * nc + c] += s * v[r] * v[c] / vv[comp[r]];
+  };
+  shift();
+  if (!invert_spd(D, nc)) {
+    dense();
+    shift();
+    if (!host_invert(D, nc)) return false;
+  }
   for (int r = 0; r < nc; ++r)
     for (int c = 0; c < nc; ++c) {
       double x = 0.5 * (D[size_t(r) * nc + c] + D[size_t(c) * nc + r]);
-      if (kernel) x -= v[r] * v[c] / (vv * s);
+      if (kernel[comp[r]] && comp[c] == comp[r]) x -= v[r] * v[c] / (vv[comp[r]] * s);
       out[size_t(r) * nc + c] = x;
     }
   return true;

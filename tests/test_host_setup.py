@@ -298,6 +298,26 @@ def test_multilevel_v_cycle_is_symmetric_positive_on_the_range(g, N, k):
     assert np.linalg.eigvalsh(0.5 * (G + G.T)).min() > 0
 
 
+@pytest.mark.parametrize("N1,N2,k", [(64, 48, 2), (64, 64, 3), (80, 60, 3), (72, 50, 1), (100, 90, 1), (128, 20, 2),
+                                     (96, 48, 1), (64, 40, 2), (20, 20, 1)])
+def test_multilevel_takes_a_mesh_of_two_parts(g, N1, N2, k):
+    # two walled boxes that share no facet: the coarsest operator has a kernel on each. PCG needs the
+    # iterations of one box (up to 45, as above; the starts differ), and solves on both
+    vid, X = zip(*(synth.split_square_mesh(N, L=1.0, origin=(2.0 * i, 0.0), periodic=False)
+                   for i, N in enumerate((N1, N2))))
+    nf = [g.host_facet_operator(v, x, k)[0].shape[0] for v, x in zip(vid, X)]
+    vid, X = np.concatenate([vid[0], vid[1] + vid[0].max() + 1]), np.concatenate(X)
+    nbr, st, blk, binv = g.host_facet_operator(vid, X, k)
+    assert nbr.shape[0] == sum(nf)
+    b = np.random.default_rng(N1).standard_normal((sum(nf), k + 1))
+    for f in (slice(0, nf[0]), slice(nf[0], None)):
+        b[f, 0] -= b[f, 0].mean()
+    res = g.host_multilevel(vid, X, k, g=b, rtol=1e-12)
+    assert 0 < res["iters"] <= 45, res["iters"]
+    r = b - _apply_S(nbr, st, blk, res["lam"]).reshape(b.shape)
+    assert np.linalg.norm(r) <= 1e-11 * np.linalg.norm(b)
+
+
 @pytest.mark.parametrize("N,k", [(2, 1), (2, 2), (3, 2)])
 def test_three_dimensional_setup_projects_like_the_oracle(g, N, k):
     # the library's 3-D host set-up (topology, canonical faces, class operators, face stencil and
