@@ -857,8 +857,9 @@ __device__ __forceinline__ bool lat_reduce(const DevMesh& m, Barrier& bar, int s
 // all after a block barrier.
 template <typename A>
 struct LatScal {
-  A alpha, alpha_lam, beta, mean, sigma;
+  A alpha, alpha_lam, beta, mean;
   double sum[2];
+  float scale;
   int done, conv;
   double relres;
 };
@@ -910,15 +911,18 @@ __device__ __forceinline__ dfl lat_g(const DevMesh& m, int f, int i, dfl) {
   return ((s.x & i & 1) ? -a : a) + ((s.y & i & 1) ? -b : b);
 }
 
-// The squares that give |r| and |g| are summed as FP32 pairs in the mixed form, of values scaled
-// by a power of two: 2^32 keeps values of 1e-28 to 1e9 within the FP32 exponents. Outside
-// [kLatSumMin, kLatSumMax] the sums say nothing, and lat_pcg (which scales by |g|) takes the solve.
+// The squares that give |g| and |r| are summed in double-float in the mixed form, of values scaled
+// by a power of two against the ends of the FP32 exponents: 2^32 in the first pass, which does not
+// know |g| yet, then the one that brings g to a root mean square in [1, 2). A sum above kLatSumMax,
+// or a mean square at the stopping threshold (rtol |g|)^2 below kLatMeanMin (of the scaled values:
+// there a square's trailing word would leave the exponents), is left to lat_pcg, which scales by |g|
+// from the start. FP64: unscaled.
 constexpr float kLatScale = 4294967296.f;
-constexpr double kLatSumMin = 1e-8, kLatSumMax = 1e36;
-__device__ __forceinline__ void add_square(double& a, double v) { a = fma(v, v, a); }
-__device__ __forceinline__ void add_square(dacc& a, dfl v) {
-  const float x = v.hi * kLatScale;
-  acc_add(a, dfl(x * x, 0.f));
+constexpr double kLatMeanMin = 1e-30, kLatSumMax = 1e36;
+__device__ __forceinline__ void add_square(double& a, double v, float) { a = fma(v, v, a); }
+__device__ __forceinline__ void add_square(dacc& a, dfl v, float scale) {
+  const dfl x(v.hi * scale, v.lo * scale);
+  mad(a, x, x);
 }
 
 // Iterative refinement. Returns 0 when the solve ended (st.conv, st.relres and it are set), -1 when
@@ -956,7 +960,7 @@ __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, 
   };
   // thread 0's own: the squared norms (scaled), without the constant-multiplier component
   double stop2 = 0.0, floor2 = 0.0, gg = 0.0, rr = 0.0;
-  const double f2 = MIXED ? double(kLatScale) * double(kLatScale) : 1.0;
+  double f2 = MIXED ? double(kLatScale) * double(kLatScale) : 1.0;   // the scale's square
   // g from both sides of every facet, the warm start lam0 = c1 hist1 + c2 hist2 (or warm_scale lam,
   // or zero) and r = g - S lam0 in one pass: a facet forms its neighbours' lam0 from the history
   // with the same operations as they do, so that lam0 is the same bits wherever it is formed
@@ -991,8 +995,8 @@ __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, 
       }
       if (!live) return;
       stv(L.r + o, r);
-      add_square(s4[0], g);
-      add_square(s4[1], r);
+      add_square(s4[0], g, kLatScale);
+      add_square(s4[1], r, kLatScale);
       if (i == 0) {
         acc_add(s4[2], g);
         acc_add(s4[3], r);
@@ -1008,13 +1012,23 @@ __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, 
           sc.mean = A(t[3] * inv);
           sc.conv = 0;
           sc.done = 0;
-          if (!(stop2 >= (MIXED ? kLatSumMin * 1e-22 : 1e-280) && gg <= (MIXED ? kLatSumMax : 1e280))) {
+          if (!(stop2 * (MIXED ? inv / NL : 1.0) >= (MIXED ? kLatMeanMin : 1e-280) &&
+                gg <= (MIXED ? kLatSumMax : 1e280))) {
             sc.done = 3;   // out of range, zero or not finite
           } else if (lam0 && !(rr <= gg)) {
             sc.done = 4;
           } else if (rr <= stop2) {
             sc.done = sc.conv = 1;
             sc.relres = sqrt(rr / gg);
+          } else if constexpr (MIXED) {
+            const int e = ilogb(gg * inv / NL) >> 1;   // the root mean square of kLatScale g is 2^e to 2^(e+1)
+            const double down = ldexp(1.0, -2 * e);
+            sc.scale = ldexpf(kLatScale, -e);
+            f2 *= down;
+            gg *= down;
+            rr *= down;
+            stop2 *= down;
+            floor2 *= down;
           }
         }))
       return -1;
@@ -1033,6 +1047,7 @@ __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, 
     if (!grid_sync(bar, m.stats)) return -1;
     // lam += z; the first pass moves the history down one slot, every pass stores the new entry
     const A mean = sc.mean;
+    const float scale = sc.scale;
     rows_inverse<K, MIXED>(L, [&](size_t o, const Z (&zv)[NL]) {
       A lv[NL];
       if (first && !lam0) {
@@ -1073,7 +1088,7 @@ __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, 
       if (i == 0) r = r - mean;
       if (!live) return;
       stv(L.r + o, r);
-      add_square(s2[0], r);
+      add_square(s2[0], r, scale);
       if (i == 0) acc_add(s2[1], r);
     });
     ++it;

@@ -657,3 +657,22 @@ def test_mixed_inviscid_residual_matches_the_oracle(g, N, k, perturb):
     v = random_lattice(mesh.n_tri, k, N)
     mesh.set_velocity(v)
     assert rel(mesh.eval_residual(), d.to_lattice(d.riesz(d.residual(d.from_lattice(v))))) < 1e-11
+
+
+@pytest.mark.parametrize("N,k", [(1, 1), (4, 2), (16, 3)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_lattice_solver_norms_keep_the_precision_of_the_form(g, N, k, precision):
+    # a state s times the last one, with a step size too small to matter: the start from the last
+    # multipliers leaves the residual (s - 1) / s |g|, up to their own error, 1e-5 (FP32 inverse, one
+    # iteration) / s = 1e-11. rtol lies above that, so that the solve ends there and reports the ratio
+    # of the two norms. Squares rounded to FP32 would show at 1e-9 to 1e-8; double-float leaves 1e-14
+    s = 1e6
+    vid, X = synth.split_square_mesh(N, L=1.0)
+    mesh = g.DGMesh(vid, X, k, 0.0, precision=precision, cg_rtol=0.9999995)
+    v = random_lattice(2 * N * N, k, N)
+    for size in (1.0, s):
+        mesh.set_velocity(size * v)
+        mesh.step(1e-30, 1, g.EULER)
+    st = mesh.solver_stats()
+    assert st["preconditioner"] == "lattice FFT" and st["last_iters"] == 0
+    assert abs(st["last_relres"] - (s - 1) / s) < 1e-10
