@@ -172,7 +172,10 @@ int dg_project_divfree(dg_mesh* mesh);
  * the last steps (linear on lattice meshes, quadratic otherwise, once the steps had the
  * same dt; an initial guess only: every solve meets cg_rtol).
  * Returns DG_ERR_NOT_CONVERGED if any solve hit cg_maxit, DG_ERR_NONFINITE if
- * a residual norm became NaN/Inf (the state is then undefined).
+ * a residual norm became NaN/Inf (the state is then undefined, and its multipliers start no
+ * later solve). Where the state itself already holds a NaN, the solve has no data: its
+ * multipliers are zero, the state keeps its NaN and no error is returned (the energy
+ * watchdog, dg_set_energy_watchdog, reports the growth that leads there).
  * Same as dg_step(mesh, DG_SCHEME_SSPRK3, dt, nsteps). */
 int dg_rk3_step(dg_mesh* mesh, double dt, int64_t nsteps);
 

@@ -235,6 +235,10 @@ void collect_profile(dg_mesh* M) {
   M->prof_prev = nullptr;
 }
 
+void forget_history(dg_mesh* M) {
+  for (int s = 0; s < dg_mesh::kMaxStages; ++s) M->hist_n[s] = 0;
+}
+
 // Synchronise the stream, gather profiling, translate device flags to a status.
 int finish(dg_mesh* M, bool check_solver) {
   CK(cudaStreamSynchronize(M->stream));
@@ -242,6 +246,10 @@ int finish(dg_mesh* M, bool check_solver) {
   if (!check_solver) return DG_OK;
   CK(cudaMemcpy(M->host_stats, M->dm.stats, sizeof(dgdf::DevStats), cudaMemcpyDeviceToHost));
   const int fl = M->host_stats->flags;
+  if (fl & (dgdf::kFlagBarrierTimeout | dgdf::kFlagNonFinite)) {   // no start for the next state's solves
+    M->has_lam = false;
+    forget_history(M);
+  }
   if (fl & dgdf::kFlagBarrierTimeout) return fail(DG_ERR_CUDA, "solver grid barrier timed out");
   if (fl & dgdf::kFlagNonFinite) return fail(DG_ERR_NONFINITE, "non-finite residual in the facet solve");
   if (fl & dgdf::kFlagNotConverged) return fail(DG_ERR_NOT_CONVERGED, "facet solve reached cg_maxit");
@@ -278,10 +286,6 @@ int ensure_udf(dg_mesh* M) {
   int rc = launch(M, KC_LATTICE, [&] { return dgdf::launch_to_dfl(M->dm.u, M->dm.u_df, n, M->stream); });
   if (rc == DG_OK) M->udf_valid = true;
   return rc;
-}
-
-void forget_history(dg_mesh* M) {
-  for (int s = 0; s < dg_mesh::kMaxStages; ++s) M->hist_n[s] = 0;
 }
 
 // Persistent solver blocks: those that fit on the device, divided by the ensemble's lanes while a batch

@@ -82,6 +82,10 @@ int finish3(dg_mesh3* M, bool check_solver) {
   if (!check_solver) return DG_OK;
   CK3(cudaMemcpy(M->host_stats, M->dm.stats, sizeof(dgdf::DevStats), cudaMemcpyDeviceToHost));
   const int fl = M->host_stats->flags;
+  if (fl & (dgdf::kFlagBarrierTimeout | dgdf::kFlagNonFinite)) {   // no start for the next state's solves
+    M->has_lam = false;
+    for (int s = 0; s < 3; ++s) M->hist_n[s] = 0;
+  }
   if (fl & dgdf::kFlagBarrierTimeout) return api_fail(DG_ERR_CUDA, "solver grid barrier timed out");
   if (fl & dgdf::kFlagNonFinite) return api_fail(DG_ERR_NONFINITE, "non-finite residual in the face solve");
   if (fl & dgdf::kFlagNotConverged) return api_fail(DG_ERR_NOT_CONVERGED, "face solve reached cg_maxit");

@@ -1224,7 +1224,7 @@ __device__ __noinline__ int lat_pcg(const DevMesh& m, const SolveArgs& a, const 
     if (!grid_reduce_pair(m, bar, 4, ga, acc_val(g0), gg)) return -1;
   }
   const double c0 = gg[1] / double(nF);
-  const double gnorm0 = sqrt(fmax(gg[0] - gg[1] * gg[1] / double(nF), 0.0));
+  const double gnorm0 = sqrt(nonneg(gg[0] - gg[1] * gg[1] / double(nF)));
   // PCG runs on the system scaled by sigma = 2^-e, e the exponent of the RMS entry of g
   // (exact in any precision): residuals and dot products stay near 1 whatever the size
   // of g, away from the FP32 exponent limits of the double-float form. r and p are
@@ -1239,7 +1239,7 @@ __device__ __noinline__ int lat_pcg(const DevMesh& m, const SolveArgs& a, const 
   const double floor2 = (a.floor_rtol * gnorm) * (a.floor_rtol * gnorm);
   bool conv = false;
   double relres = 0.0;
-  if (gnorm == 0.0) {
+  if (!(gnorm0 > 0.0)) {   // no data, or a NaN (a state that holds one): zero
     for (int f = gtid; f < nF; f += gsz) {
       const size_t o = size_t(f) * VS;
       A zero[NL];

@@ -799,12 +799,11 @@ __global__ void __launch_bounds__((ml_threads<NL, R>()), 1) k_solve_ml(Mesh mesh
   if (!ml_reduce<2>(m, bar, 4, gg, scr, [&](const double (&t)[2]) {
         // with outflow facets S is definite: no constant component to remove (inv_nf = 0)
         inv_nf = m.has_kernel ? 1.0 / double(m.n) : 0.0;
-        const double g2 = fmax(t[0] - t[1] * t[1] * inv_nf, 0.0);
-        gnorm = sqrt(g2);
+        gnorm = sqrt(nonneg(t[0] - t[1] * t[1] * inv_nf));
         stop2 = (a.rtol * gnorm) * (a.rtol * gnorm);
         floor2 = (a.floor_rtol * gnorm) * (a.floor_rtol * gnorm);
         sc.c0 = t[1] * inv_nf;
-        sc.zero = gnorm == 0.0;
+        sc.zero = !(gnorm > 0.0);   // no data, or a NaN (a state that holds one): zero
       }))
     return;
   if (sc.zero) {
@@ -852,7 +851,7 @@ __global__ void __launch_bounds__((ml_threads<NL, R>()), 1) k_solve_ml(Mesh mesh
       double red[3] = {0.0, 0.0, 0.0};
       if (!ml_vcycle<NL, NB, R>(m, c, lv, bar, red)) return;
       if (!ml_reduce<3>(m, bar, 1, red, scr, [&](const double (&t)[3]) {
-            rr = fmax(t[1] - t[2] * t[2] * inv_nf, 0.0);
+            rr = nonneg(t[1] - t[2] * t[2] * inv_nf);
             sc.beta = first ? 0.0 : t[0] / rho;
             rho = t[0];
             sc.mean = t[2] * inv_nf;   // mode-0 mean of r as the V-cycle saw it

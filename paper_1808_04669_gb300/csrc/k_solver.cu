@@ -54,7 +54,7 @@ __device__ int pcg(const DevMesh& m, R* x, R* rv, R* zv, R* pa, R* pb, R* qv, co
     red[2] += double(r[0]);
   }
   if (!grid_reduce<3>(m, 1, red, bar)) return 0;
-  double rho = red[0], rr = fmax(red[1] - red[2] * red[2] * inv_nf, 0.0);
+  double rho = red[0], rr = nonneg(red[1] - red[2] * red[2] * inv_nf);
   double beta = 0.0;
   R* pold = pa;
   R* pnew = pb;
@@ -122,7 +122,7 @@ __device__ int pcg(const DevMesh& m, R* x, R* rv, R* zv, R* pa, R* pb, R* qv, co
     if (!grid_reduce<3>(m, 1, red2, bar)) return it + 1;
     beta = red2[0] / rho;
     rho = red2[0];
-    rr = fmax(red2[1] - red2[2] * red2[2] * inv_nf, 0.0);
+    rr = nonneg(red2[1] - red2[2] * red2[2] * inv_nf);
     R* t = pold;
     pold = pnew;
     pnew = t;
@@ -160,12 +160,12 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve(DevMesh m, SolveArgs a
   const double c0 = gg[1] * inv_nf;
   if (c0 != 0.0)
     for (int f = gtid; f < nF; f += gsz) m.g[size_t(f) * NL] -= c0;
-  const double gnorm = sqrt(fmax(gg[0] - gg[1] * gg[1] * inv_nf, 0.0));
+  const double gnorm = sqrt(nonneg(gg[0] - gg[1] * gg[1] * inv_nf));
   const double stop = a.rtol * gnorm;
   int iters = 0, sweeps = 0;
   bool conv = false;
   double relres = 0.0;
-  if (gnorm == 0.0) {
+  if (!(gnorm > 0.0)) {   // no data, or a NaN (a state that holds one): zero
     for (int f = gtid; f < nF; f += gsz)
 #pragma unroll
       for (int j = 0; j < NL; ++j) m.lam[size_t(f) * NL + j] = 0.0;
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve(DevMesh m, SolveArgs a
         break;
       }
       if (!grid_reduce<2>(m, 6, rr, bar)) return;
-      rr[0] = fmax(rr[0] - rr[1] * rr[1] * inv_nf, 0.0);
+      rr[0] = nonneg(rr[0] - rr[1] * rr[1] * inv_nf);
       const double prev = relres;
       relres = sqrt(rr[0]) / gnorm;
       if (!isfinite(rr[0])) {
@@ -338,15 +338,16 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve_noalloc(DevMesh m, con
   if (!grid_reduce<2>(m, 4, gg, bar)) return;
   const double c0 = gg[1] / double(nF);
   for (int f = gtid; f < nF; f += gsz) m.g[size_t(f) * NL] -= c0;
-  const double gnorm = sqrt(fmax(gg[0] - gg[1] * gg[1] / double(nF), 0.0));
+  const double gnorm = sqrt(nonneg(gg[0] - gg[1] * gg[1] / double(nF)));
   bool conv = false;
   int iters = 0;
   double relres = 0.0;
-  if (gnorm == 0.0) {
+  if (!(gnorm > 0.0)) {   // zero; of a g that holds a NaN it is no solution
     for (int f = gtid; f < nF; f += gsz)
 #pragma unroll
       for (int j = 0; j < NL; ++j) m.lam[size_t(f) * NL + j] = 0.0;
-    conv = true;
+    conv = gnorm == 0.0;
+    if (!conv && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&m.stats->flags, kFlagNonFinite);
   } else {
     for (int f = gtid; f < nF; f += gsz) {
       double y[NL];

@@ -468,12 +468,12 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
   }
   if (!reduce3<2>(m, bar, 4, gg)) return;
   const double c0 = gg[1] * inv_nf;
-  const double gnorm = sqrt(fmax(gg[0] - gg[1] * gg[1] * inv_nf, 0.0));
+  const double gnorm = sqrt(nonneg(gg[0] - gg[1] * gg[1] * inv_nf));
   const double stop = a.rtol * gnorm;
   int it = 0;
   bool conv = false;
   double rr = 0.0;
-  if (gnorm == 0.0) {
+  if (!(gnorm > 0.0)) {   // no data, or a NaN (a state that holds one): zero
     for (int f = gtid; f < nF; f += gsz)
 #pragma unroll
       for (int j = 0; j < NL; ++j) m.lam[size_t(f) * NL + j] = 0.0;
@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
     }
     if (!reduce3<3>(m, bar, 1, red)) return;
     double rho = red[0];
-    rr = fmax(red[1] - red[2] * red[2] * inv_nf, 0.0);
+    rr = nonneg(red[1] - red[2] * red[2] * inv_nf);
     double beta = 0.0;
     double* pold = m.pa;
     double* pnew = m.pb;
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
       if (!reduce3<3>(m, bar, 1, red2)) return;
       beta = red2[0] / rho;
       rho = red2[0];
-      rr = fmax(red2[1] - red2[2] * red2[2] * inv_nf, 0.0);
+      rr = nonneg(red2[1] - red2[2] * red2[2] * inv_nf);
       double* tmp = pold;
       pold = pnew;
       pnew = tmp;

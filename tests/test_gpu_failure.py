@@ -122,3 +122,73 @@ def test_lattice_solve_drops_a_start_far_from_the_solution(g, precision, size0, 
             out.append(m.get_velocity() / size)
         assert np.isfinite(out[1]).all()
         assert np.linalg.norm(out[0] - out[1]) < 1e-13 * np.sqrt(1e3 * N) * 10 * np.linalg.norm(out[1])
+
+
+def check_good_state_after_overflow(mesh, fresh, v):
+    # steps far above the stability limit, until a solve reports that its residual overflowed: nothing
+    # of its multipliers stays, and a good state then gives the result of a fresh mesh
+    from paper_1808_04669_gb300 import DGError
+    mesh.set_velocity(v)
+    mesh.project_divfree()
+    code = 0
+    for _ in range(10):
+        try:
+            mesh.rk3_step(10.0, 1)
+        except DGError as e:
+            code = e.code
+            break
+    assert code == -6
+    for m in (mesh, fresh):
+        m.set_velocity(v)
+        m.rk3_step(1e-3, 2)
+    a, b = mesh.get_velocity(), fresh.get_velocity()
+    assert np.abs(a - b).max() <= 1e-13 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("precond", [1, 2])
+def test_good_state_after_an_overflow(g, precond):
+    N, k = 8, 2
+    vid, X = synth.split_square_mesh(N, L=1.0, periodic=False)
+    mesh, fresh = (g.DGMesh(vid, X, k, 0.0, precond=precond) for _ in range(2))
+    check_good_state_after_overflow(mesh, fresh, random_lattice(2 * N * N, k, 1))
+
+
+@pytest.mark.parametrize("precond", [0, 1])
+def test_good_state_after_an_overflow_in_three_dimensions(g, precond):
+    from synth.mesh3 import kuhn_cube_mesh
+    vid, X = kuhn_cube_mesh(4)
+    mesh, fresh = (g.DGMesh3(vid, X, 1, 0.0, precond=precond) for _ in range(2))
+    check_good_state_after_overflow(mesh, fresh, np.random.default_rng(1).standard_normal((mesh.n_tet, mesh.n_lat, 3)))
+
+
+def test_residual_that_is_not_a_number_is_no_solution(g):
+    # a step size 1e297 times the last one scales the start by as much: the residual's norm is inf - inf,
+    # which is not zero (mixed block Jacobi, whose refinement tests that norm alone)
+    from paper_1808_04669_gb300 import DGError
+    N, k = 8, 2
+    vid, X = synth.split_square_mesh(N, L=1.0)
+    v = random_lattice(2 * N * N, k, 1)
+    mesh, fresh = (g.DGMesh(vid, X, k, 0.0, precision=1, precond=1) for _ in range(2))
+    mesh.set_velocity(v)
+    mesh.step(1e-300, 1, g.EULER)
+    mesh.set_velocity(v)
+    with pytest.raises(DGError) as e:
+        mesh.step(1e-3, 1, g.EULER)
+    assert e.value.code == -6
+    for m in (mesh, fresh):
+        m.set_velocity(v)
+        m.step(1e-3, 1, g.EULER)
+    a, b = mesh.get_velocity(), fresh.get_velocity()
+    assert np.abs(a - b).max() <= 1e-13 * np.abs(b).max()
+
+
+def test_facet_solve_reports_a_right_hand_side_that_is_not_a_number(g):
+    import torch
+    from paper_1808_04669_gb300 import DGError
+    vid, X = synth.split_square_mesh(4)
+    t = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in g.host_facet_operator(vid, X, 1)]
+    rhs = torch.zeros(t[0].shape[0], 2, dtype=torch.float64, device="cuda")
+    rhs[3, 1] = float("nan")
+    with pytest.raises(DGError) as e:
+        g.facet_solve_noalloc(1, *t, rhs, torch.zeros_like(rhs))
+    assert e.value.code == -6
