@@ -5,6 +5,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <exception>
+#include <system_error>
 #include <thread>
 
 #include "../../include/dgdf.h"
@@ -20,15 +22,32 @@ double dot(const Vec& a, const Vec& b) {
   return s;
 }
 
-// fn(begin, end, worker) over [0, n) on up to `most` of the host's cores, `grain` rows each at least
+// fn(begin, end, worker) over [0, n) on up to `most` of the host's cores, `grain` rows each at least.
+// Parts for which the host has no thread left run on the caller's; an exception of a part is the
+// caller's, too.
 template <typename F>
 void parallel_rows(int n, F fn, int most = 16, int grain = 512) {
   const int nt = std::max(1, std::min({int(std::thread::hardware_concurrency()), most, n / grain}));
+  std::vector<std::exception_ptr> error(nt);
+  auto part = [&](int w) {
+    try {
+      fn(int(int64_t(n) * w / nt), int(int64_t(n) * (w + 1) / nt), w);
+    } catch (...) {
+      error[w] = std::current_exception();
+    }
+  };
   std::vector<std::thread> th;
-  for (int w = 1; w < nt; ++w)
-    th.emplace_back([&, w] { fn(int(int64_t(n) * w / nt), int(int64_t(n) * (w + 1) / nt), w); });
-  fn(0, n / nt, 0);
+  th.reserve(nt);
+  int started = 1;
+  try {
+    for (; started < nt; ++started) th.emplace_back(part, started);
+  } catch (const std::system_error&) {
+  }
+  part(0);
+  for (int w = started; w < nt; ++w) part(w);
   for (std::thread& t : th) t.join();
+  for (const std::exception_ptr& e : error)
+    if (e) std::rethrow_exception(e);
 }
 
 // ---- operators of one level on the host

@@ -318,6 +318,32 @@ def test_multilevel_takes_a_mesh_of_two_parts(g, N1, N2, k):
     assert np.linalg.norm(r) <= 1e-11 * np.linalg.norm(b)
 
 
+def test_multilevel_setup_without_threads(g):
+    # a host that gives no thread (here: thread stacks larger than the address space) builds the same
+    # hierarchy on the caller's
+    import os
+    import resource
+    import subprocess
+    import sys
+    code = ("import hashlib, numpy as np, synth, paper_1808_04669_gb300 as g\n"
+            "vid, X = synth.split_square_mesh(120, L=1.0, periodic=False)\n"
+            "n = g.host_facet_operator(vid, X, 2)[0].shape[0] * 3\n"
+            "r = np.random.default_rng(1).standard_normal((1, n))\n"
+            "print(hashlib.sha1(g.host_multilevel(vid, X, 2, r=r)['z'].tobytes()).hexdigest())\n")
+    env = dict(os.environ, OPENBLAS_NUM_THREADS="1", OMP_NUM_THREADS="1")
+    hard = resource.getrlimit(resource.RLIMIT_STACK)[1]
+    if hard != resource.RLIM_INFINITY:
+        pytest.skip("the stack limit cannot be raised")
+    out = []
+    for limit in (None, 1 << 47):
+        pre = limit and (lambda: resource.setrlimit(resource.RLIMIT_STACK, (limit, hard)))
+        p = subprocess.run([sys.executable, "-c", code], env=env, preexec_fn=pre, capture_output=True, text=True,
+                           cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))), timeout=300)
+        assert p.returncode == 0, p.stderr
+        out.append(p.stdout.split()[-1])
+    assert out[0] == out[1]
+
+
 @pytest.mark.parametrize("N,k", [(2, 1), (2, 2), (3, 2)])
 def test_three_dimensional_setup_projects_like_the_oracle(g, N, k):
     # the library's 3-D host set-up (topology, canonical faces, class operators, face stencil and
