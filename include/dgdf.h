@@ -358,6 +358,13 @@ int dg_test_multilevel_apply(dg_mesh* mesh, const double* r, double* z, int on_d
  * The state after such a solve is undefined; (0, -1) restores normal operation. */
 int dg_test_barrier_fault(dg_mesh* mesh, int64_t spin_limit, int skip_block);
 
+/* Test hook of the lattice facet solver (no counterpart in the paper). Its refinement
+ * goes on as PCG when an iteration leaves more than gain times the squared residual
+ * (0.01 by default, which no mesh measured reaches); 0 makes every solve that the first
+ * iteration does not end go on as PCG. Results meet cg_rtol either way.
+ * Errors: DG_ERR_INVALID_ARG. */
+int dg_test_refine_gain(dg_mesh* mesh, double gain);
+
 /* Per-kernel-class device timing. enable = 1 makes the library record CUDA events
  * on its stream around every kernel launch from then on and add the elapsed times
  * up at the end of each call; inside a time step, a launch that directly follows

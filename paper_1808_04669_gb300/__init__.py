@@ -223,6 +223,10 @@ class DGMesh:
         """Failure-detection test hook (dg_test_barrier_fault): bounded barrier waits of the solvers."""
         check(lib().dg_test_barrier_fault(self._h, int(spin_limit), int(skip_block)), "dg_test_barrier_fault")
 
+    def test_refine_gain(self, gain):
+        """Test hook of the lattice solver (dg_test_refine_gain): where refinement goes on as PCG."""
+        check(lib().dg_test_refine_gain(self._h, float(gain)), "dg_test_refine_gain")
+
     def profile(self, enable):
         n = 16
         ms = (ctypes.c_double * n)()

@@ -71,6 +71,7 @@ struct dg_mesh {
   int solver_blocks[2] = {1, 1};
   bool use_lattice = false;
   int lattice_blocks = 0, lattice_work = 0;
+  double refine_gain = 0.01;      // SolveArgs::gain
   bool tc_available = false;      // the tensor-core recovery is set up (mixed form, <= 2 classes)
   bool use_ml = false;            // multilevel-preconditioned PCG (k_multilevel.cu)
   int grid_div = 1;               // solver grid divided by this while a batch runs lanes
@@ -330,6 +331,7 @@ int solve(dg_mesh* M, double warm_scale, int stage = -1, double dt = 0.0, bool h
   a.max_sweeps = 40;
   a.inner_maxit = M->p.cg_maxit;
   a.floor_rtol = 1e-9;
+  a.gain = M->refine_gain;
   if (M->use_lattice) {
     const int nb = capped(M, M->lattice_blocks, M->lattice_work);
     return launch(M, a.mixed ? KC_SOLVE_LAT32 : KC_SOLVE_LAT64,
@@ -1777,6 +1779,14 @@ int dg_test_barrier_fault(dg_mesh* M, int64_t spin_limit, int skip_block) {
   CK(cudaMemcpyAsync(&M->dm.stats->spin_limit, &lim, sizeof(lim), cudaMemcpyHostToDevice, M->stream));
   CK(cudaMemcpyAsync(&M->dm.stats->skip_block, &skip, sizeof(skip), cudaMemcpyHostToDevice, M->stream));
   return finish(M, false);
+}
+
+int dg_test_refine_gain(dg_mesh* M, double gain) {
+  if (int rc = check_mesh(M)) return rc;
+  if (!(gain >= 0.0) || !std::isfinite(gain)) return fail(DG_ERR_INVALID_ARG, "gain must be finite and >= 0");
+  M->refine_gain = gain;
+  ++M->gen;
+  return DG_OK;
 }
 
 int dg_profile(dg_mesh* M, int enable, double* out_ms, int64_t* out_launches, int n) {

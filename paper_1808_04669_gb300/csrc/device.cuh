@@ -216,6 +216,7 @@ struct SolveArgs {
   void* hist2;
   void* hist3;
   double c1, c2, c3;
+  double gain;         // lattice solver: refinement that leaves more than gain |r|^2 goes on as PCG
   void* hist_new;      // lattice solver: where to store the new lam too (NULL: nowhere); may be hist1
 };
 

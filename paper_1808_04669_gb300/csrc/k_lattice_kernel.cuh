@@ -1106,7 +1106,7 @@ __device__ __forceinline__ int lat_refine(const DevMesh& m, const SolveArgs& a, 
             sc.done = sc.conv = 1;
           } else if (n >= a.maxit) {
             sc.done = 1;
-          } else if (!(rr <= 0.01 * prev)) {
+          } else if (!(rr <= a.gain * prev)) {
             sc.done = 3;
           }
         }))

@@ -676,3 +676,48 @@ def test_lattice_solver_norms_keep_the_precision_of_the_form(g, N, k, precision)
     st = mesh.solver_stats()
     assert st["preconditioner"] == "lattice FFT" and st["last_iters"] == 0
     assert abs(st["last_relres"] - (s - 1) / s) < 1e-10
+
+
+@pytest.mark.parametrize("N,k", [(2, 1), (13, 2), (66, 3)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_lattice_refinement_goes_on_as_pcg(g, N, k, precision):
+    # gain 0: a solve that its first iteration does not end hands over to PCG then, with the history already moved
+    # and lam as its start (rtol 1e-17 in FP64, where one iteration reaches 1e-15). Block Jacobi meets
+    # rtol 1e-13, so that the states differ by that times sqrt(cond(S)) (below 1e3 N), with a factor of
+    # ten to spare; the steps after the first start from the history and need no more iterations than
+    # the first one's cold solves
+    vid, X = synth.split_square_mesh(N, L=1.0)
+    v = random_lattice(2 * N * N, k, N)
+    mesh = g.DGMesh(vid, X, k, 0.0, precision=precision, cg_rtol=1e-13 if precision else 1e-17)
+    ref = g.DGMesh(vid, X, k, 0.0, precision=precision, precond=g.PRECOND_BLOCK_JACOBI)
+    mesh.test_refine_gain(0.0)
+    its = []
+    for step in range(5):
+        for m in (mesh, ref):
+            if step == 0:
+                m.set_velocity(v)
+                m.project_divfree()
+            m.rk3_step(1e-3 / N, 1)
+        its.append(mesh.solver_stats()["total_iters"])
+        assert rel(mesh.get_velocity(), ref.get_velocity()) < 1e-13 * np.sqrt(1e3 * N) * 10
+    its = np.diff([0.0] + its)
+    assert its[0] > 4 and its[1:].max() <= its[0], its
+
+
+@pytest.mark.parametrize("N,k", [(2, 3), (13, 2), (127, 1)])
+@pytest.mark.parametrize("size", [1e-15, 1e11])
+def test_lattice_pcg_takes_sizes_outside_the_range_of_refinement(g, N, k, size):
+    # g so small or large that the mixed form's sums of squares leave the FP32 exponents (scaled by
+    # 2^32, the squares are 2e-11 and 2e41 times those of size 1 / N): PCG from the start. Against
+    # block Jacobi and against refinement at size 1, tolerance as above
+    vid, X = synth.split_square_mesh(N, L=1.0)
+    v = random_lattice(2 * N * N, k, N)
+    out = []
+    for pc, sz in ((g.PRECOND_AUTO, size), (g.PRECOND_BLOCK_JACOBI, size), (g.PRECOND_AUTO, 1.0)):
+        mesh = g.DGMesh(vid, X, k, 0.0, precision=1, precond=pc)
+        mesh.set_velocity(sz * v)
+        mesh.project_divfree()
+        mesh.rk3_step(1e-3 / (N * sz), 3)
+        out.append(mesh.get_velocity())
+    assert rel(out[0], out[1]) < 1e-13 * np.sqrt(1e3 * N) * 10
+    assert rel(out[0] / size, out[2]) < 1e-13 * np.sqrt(1e3 * N) * 10
