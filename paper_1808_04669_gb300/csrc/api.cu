@@ -501,9 +501,9 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
       }
     }
     if ((rc = upload(M, &d.dn64, dn))) return cleanup(rc);
-    // the viscous terms that a triangle's own coefficients enter linearly, as matrices on them:
-    // vown = -int grad phi_j . grad phi_i + sum over the facets of vfac, and
-    // vfac[e] = int_e (phi_j d_n phi_i + d_n phi_j phi_i) / 2
+    // the viscous terms of a triangle's own gradient as matrices on its coefficients j, tested by
+    // phi_i: vown[j][i] = -int grad phi_j . grad phi_i + sum over the facets of vfac, and
+    // vfac[e][j][i] = int_e d_n phi_j phi_i / 2
     const int ns_ = hm.ns;
     std::vector<double> vown(size_t(d.n_class) * ns_ * ns_, 0.0), vfac(size_t(d.n_class) * 3 * ns_ * ns_, 0.0);
     for (int c = 0; c < d.n_class; ++c) {
@@ -522,7 +522,7 @@ int dg_mesh_create_ex(int64_t n_tri, const int64_t* tri_vertex_ids, const double
             double f = 0.0;
             for (int q = 0; q < nqf; ++q) {
               const double *ph = &ref.fphi[(size_t(e) * nqf + q) * ns_], *dq = &dn[((size_t(c) * 3 + e) * nqf + q) * ns_];
-              f += ref.fw[q] * co.flen[e] * s2 * 0.5 * (ph[j] * dq[i] + dq[j] * ph[i]);
+              f += ref.fw[q] * co.flen[e] * s2 * 0.5 * dq[j] * ph[i];
             }
             vfac[((size_t(c) * 3 + e) * ns_ + j) * ns_ + i] = f;
             v += f;

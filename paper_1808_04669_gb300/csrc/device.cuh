@@ -97,8 +97,9 @@ struct DevMesh {
   // both leading words, then both trailing words)
   const float4 *ptab, *P2, *G2;
   const double* dn64;   // the same normal derivatives in FP64, [n_class][3][nqf][ns] (NULL: more classes)
-  // the viscous terms linear in a triangle's own coefficients, per class: vown [ns][ns] with all three
-  // facets interior (also in ptab), vfac [3][ns][ns] what a facet adds (subtracted on boundary facets)
+  // the viscous terms of a triangle's own gradient on its coefficients, [coefficient][test function] per
+  // class: vown [ns][ns] with all three facets interior (also in ptab), vfac [3][ns][ns] what a facet
+  // adds (subtracted on boundary facets)
   const double *vown64, *vfac64;
   const float4* vfac2;  // vfac in double-float pairs [n_class][3][ns][ceil(ns/2)]
   int ptab_words;   // float4 words of ptab

@@ -26,9 +26,10 @@ constexpr int kTileThreads = 128;
 
 // How a kernel takes the viscous terms: none (nu = 0), with the normal derivatives of the basis at
 // the facet points from a per-class table (m.dn64, at most kDnClasses classes), or from reference
-// gradients. The stage kernel with tables takes the terms that a triangle's own coefficients enter
-// linearly (volume, own consistency and symmetry) as one matrix per class (m.vown64): its volume
-// points then need no gradients, its facet points no own normal derivative.
+// gradients. The stage kernel with tables takes the terms of a triangle's own gradient (volume, own
+// consistency) as one matrix per class (m.vown64): its volume points then need no gradients, its facet
+// points no own normal derivative. The symmetry term stays at the facet points, where both traces,
+// nearly equal in a smooth field, meet before a derivative multiplies them.
 enum Visc { VISC_NONE, VISC_TABLE, VISC_GENERAL };
 
 template <int K>
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
                 const double jc = ui[c] - uo[c], wn = w * nu;
                 if constexpr (V == VISC_TABLE) {
                   x += wn * (0.5 * dd[c] - g.sig * jc);
-                  B = -0.5 * wn * uo[c];
+                  B = 0.5 * wn * jc;
                 } else {
                   x += wn * (0.5 * (di[c] + dd[c]) - g.sig * jc);
                   B = 0.5 * wn * jc;
@@ -300,18 +301,18 @@ __global__ void __launch_bounds__(kTileThreads) k_stage64(DevMesh m, StageArgs a
         }
         if constexpr (V == VISC_TABLE) {
           const int cls = info[el] >> 3, walls = info[el] & 7;
-          const double *tab = dn + cls * NF * NS + j, *vo = dn + m.n_class * NF * NS + (cls * NS + j) * NS;
+          const double *tab = dn + cls * NF * NS + j, *vo = dn + m.n_class * NF * NS + cls * NS * NS + j;
           const double* u = U + el * L::LU + c * NS;
 #pragma unroll
           for (int p = 0; p < NF; ++p) y += A_[p * L::NA + 2 + c] * tab[p * NS];
           double z = 0.0;
 #pragma unroll
-          for (int k = 0; k < NS; ++k) z += vo[k] * u[k];
+          for (int k = 1; k < NS; ++k) z += vo[k * NS] * u[k];   // (mode 0 has no gradient)
           for (int e = 0; walls >> e; ++e)
             if (walls >> e & 1) {   // a boundary facet has no viscous terms
-              const double* vf = m.vfac64 + ((size_t(cls) * 3 + e) * NS + j) * NS;
+              const double* vf = m.vfac64 + (size_t(cls) * 3 + e) * NS * NS + j;
 #pragma unroll
-              for (int k = 0; k < NS; ++k) z -= __ldg(&vf[k]) * u[k];
+              for (int k = 1; k < NS; ++k) z -= __ldg(&vf[k * NS]) * u[k];
             }
           x += nu * z;
         }

@@ -277,10 +277,12 @@ __global__ void __launch_bounds__(kStageDfThreads, 2) k_stage_df(DevMesh m, Stag
 // once in the packed FP32x2 instructions (dacc2 / mad2), with the tables laid out as
 // pairs {hi_j, hi_j+1, lo_j, lo_j+1}. The terms and the per-point arithmetic are those of
 // k_stage_df; only the order of summation inside each dot product differs (even and odd
-// j apart). The viscous terms that a triangle's own coefficients enter linearly (volume, own
-// consistency and symmetry) are one matrix per class (PairTables::visc): the volume points
-// need no gradients, the facet points no own normal derivative, and the symmetry term keeps the
-// neighbour's trace alone. 4080 -> 3340 multiply-adds a triangle at k = 3: 256^2 287 -> 233 us.
+// j apart). The viscous terms of a triangle's own gradient (volume, own consistency) are one matrix
+// per class on its coefficients (PairTables::visc): the volume points need no gradients, the facet
+// points no own normal derivative. The symmetry term stays at the facet points, where both traces,
+// nearly equal in a smooth field, meet before a derivative multiplies them (in the matrix, too, with
+// the neighbour's trace alone at the points, it made the residual's error 1.12 times as large: fields
+// at 150^2; now 1.01). 4080 -> 3340 multiply-adds a triangle at k = 3: 256^2 287 -> 233 us.
 template <int K>
 struct PairTables {
   static constexpr int NS2 = (Dims<K>::NS + 1) / 2, NQ = Dims<K>::NQ, NQF = Dims<K>::NQF;
@@ -378,7 +380,7 @@ __device__ __forceinline__ void residual_pairs(const DevMesh& m, const PairTable
       const dfl w = to_dfl(T.fw[q]) * lens;
       if constexpr (VISC) {
         const dfl2 A = splat(w * (hnu * dn - vn * wup - nusig * jc));
-        const dfl2 B = splat(-(w * hnu * uo));
+        const dfl2 B = splat(w * hnu * jc);
 #pragma unroll
         for (int jp = 0; jp < NS2; ++jp) {
           mad2(acc[jp], A, pair(T.fphi[e][q][jp]));
@@ -391,24 +393,33 @@ __device__ __forceinline__ void residual_pairs(const DevMesh& m, const PairTable
       }
     }
   }
-  // the viscous terms of the own coefficients; a boundary facet has none
+  // the viscous terms of the own gradient (mode 0 has none), multiplied by nu once they are summed; a
+  // boundary facet has none
   if constexpr (VISC) {
+    dacc2 z[NS2];
 #pragma unroll
-    for (int i = 0; i < NS; ++i) {
-      const dfl2 x = splat(nu * lane(up[i / 2], i & 1));
+    for (int jp = 0; jp < NS2; ++jp) z[jp] = dacc2_zero();
 #pragma unroll
-      for (int jp = 0; jp < NS2; ++jp) mad2(acc[jp], x, pair(T.visc[cls][i][jp]));
+    for (int i = 1; i < NS; ++i) {
+      const dfl2 x = splat(lane(up[i / 2], i & 1));
+#pragma unroll
+      for (int jp = 0; jp < NS2; ++jp) mad2(z[jp], x, pair(T.visc[cls][i][jp]));
     }
 #pragma unroll 1
     for (int e = 0; e < 3; ++e) {
       if (__ldg(&m.tri_nbr[size_t(t) * 3 + e]) >= 0) continue;
       const float4* vf = m.vfac2 + (size_t(cls) * 3 + e) * NS * NS2;
 #pragma unroll
-      for (int i = 0; i < NS; ++i) {
-        const dfl2 x = splat(-(nu * lane(up[i / 2], i & 1)));
+      for (int i = 1; i < NS; ++i) {
+        const dfl2 x = splat(-lane(up[i / 2], i & 1));
 #pragma unroll
-        for (int jp = 0; jp < NS2; ++jp) mad2(acc[jp], x, pair(__ldg(&vf[i * NS2 + jp])));
+        for (int jp = 0; jp < NS2; ++jp) mad2(z[jp], x, pair(__ldg(&vf[i * NS2 + jp])));
       }
+    }
+#pragma unroll
+    for (int jp = 0; jp < NS2; ++jp) {
+      const dfl zx = val_x(z[jp]), zy = val_y(z[jp]);
+      mad2(acc[jp], splat(nu), dfl2{make_float2(zx.hi, zy.hi), make_float2(zx.lo, zy.lo)});
     }
   }
   if (m.facet_kind)

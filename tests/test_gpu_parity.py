@@ -721,3 +721,20 @@ def test_lattice_pcg_takes_sizes_outside_the_range_of_refinement(g, N, k, size):
         out.append(mesh.get_velocity())
     assert rel(out[0], out[1]) < 1e-13 * np.sqrt(1e3 * N) * 10
     assert rel(out[0] / size, out[2]) < 1e-13 * np.sqrt(1e3 * N) * 10
+
+
+@pytest.mark.parametrize("N,k", [(4, 1), (7, 2), (10, 3)])
+@pytest.mark.parametrize("walls", [False, True])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_uniform_state_has_no_viscous_terms(g, N, k, walls, precision):
+    # of a uniform state every jump and gradient is zero, in exact arithmetic and, with equal operations
+    # on both sides of a facet, in the kernels': the viscous terms vanish whatever nu. Left over by terms
+    # that only cancel in the sum they would be the form's rounding (1e-16, 1e-14) times nu / h^2
+    vid, X = synth.split_square_mesh(N, L=1.0, periodic=not walls)
+    mesh = g.DGMesh(vid, X, k, 0.0, precision=precision)
+    c = np.zeros((mesh.n_tri, 2, mesh.n_lat))
+    c[:, 0, 0], c[:, 1, 0] = 0.3, -0.7
+    mesh.set_coefficients(c.reshape(mesh.n_tri, -1))
+    inviscid = mesh.eval_residual()
+    mesh.set_viscosity(1e8)
+    assert np.abs(mesh.eval_residual() - inviscid).max() <= 1e-12 * max(1.0, np.abs(inviscid).max())
