@@ -41,7 +41,7 @@ L2_FLUSH_BYTES = 512 << 20
 # over the three stages of a step (the first stage reads one state, the others two), from the
 # ncu capture summarised in profiles/; used only while the stage-kernel sources still hash to
 # the captured `sha`, else the line reports null.
-NCU_TRAFFIC = {"stage_residual": {"sha": "606d4b9243dd1631", "n_tri": 131072, "bytes": 40762283,
+NCU_TRAFFIC = {"stage_residual": {"sha": "b82797c0b5404b51", "n_tri": 131072, "bytes": 40764757,
                                   "source": "profiles/k_stage_df2_shear_n256_k3.md"}}
 
 
@@ -211,7 +211,7 @@ def element_kernel_sha():
 def stage_flops_per_triangle(k, tabulated=True):
     """Flops of the viscous stage kernel per triangle (FMA = 2), counted from its loops: the volume
     rule has 3, 7, 16 points for k = 1, 2, 3 (fully symmetric, degree 3k - 1). With `tabulated`
-    (meshes of at most 4 geometry classes) the viscous terms of the triangle's own coefficients are
+    (meshes of at most 4 geometry classes) the viscous terms of the triangle's own gradient are
     one matrix per class, and the facet normal derivatives of the basis come from per-class tables:
     per volume point the trace and its test, per facet point both traces, the neighbour's normal
     derivative and two tests. Otherwise gradients (volume) and three sums per trace and per test."""

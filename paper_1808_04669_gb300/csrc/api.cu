@@ -290,8 +290,10 @@ int ensure_udf(dg_mesh* M) {
 }
 
 // Persistent solver blocks: those that fit on the device, divided by the ensemble's lanes while a batch
-// runs members on parallel graph branches (so that every solver grid that can run at the
-// same time fits on the device together, and no grid barrier waits for another grid's blocks).
+// runs members on parallel graph branches, so that the solver grids that can run at the same time take
+// at most every SM once over. A block of the multilevel solver takes a whole SM: it may wait for
+// half-SM blocks of other lanes' grids to end, which find their place beside it. Time lost, where both
+// kinds share a batch, but no wait without end.
 // work: blocks that the solve has work for.
 int capped(const dg_mesh* M, int nb, int work) {
   if (M->grid_div > 1) nb = std::max(1, nb / M->grid_div);

@@ -37,10 +37,11 @@ __global__ void __launch_bounds__(128) k_recover(DevMesh m, double* out) {
   }
 }
 
-// The same with a thread per coefficient, for meshes of fewer than kRecoverSmall triangles: below
-// that a thread per triangle leaves SM quarters without a warp (FP64 instructions take one 64 cycles),
-// above it the shared multipliers win. 8^2, BDM_2: 10.4 us a thread per triangle, 6.0 per coefficient;
-// 64^2, BDM_2: 11.1, 8.3; 128^2, BDM_3: 22.9, 28.7.
+// The same with a thread per coefficient, for meshes of fewer than kRecoverSmall triangles (a warp for
+// each of the four quarters of this chip's 152 SMs): below that a thread per triangle leaves quarters
+// without a warp (FP64 instructions take one 64 cycles), above it the shared multipliers win. 8^2,
+// BDM_2: 10.4 us a thread per triangle, 6.0 per coefficient; 64^2, BDM_2: 11.1, 8.3; 128^2, BDM_3:
+// 22.9, 28.7.
 constexpr int kRecoverSmall = 608 * 32;
 template <int K>
 __global__ void __launch_bounds__(128) k_recover_coef(DevMesh m, double* out) {

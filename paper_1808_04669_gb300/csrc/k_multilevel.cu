@@ -48,8 +48,10 @@ namespace {
 
 constexpr int kMLThreads = 1024;         // most threads of a block
 // Threads of a block: 1024 (64 registers) in FP32; 512 (128 registers) in FP64 and for the six modes
-// of 3-D faces, whose rows of operands spill at 64 (FP64, 48^2 BDM_2: 1.33 -> 1.26 ms a solve; FP32
-// at 128^2 BDM_3: 1.26 ms with 512, 1.21 with 1024).
+// of 3-D faces, whose rows of operands do not fit 64 (FP64, 48^2 BDM_2: 1.33 -> 1.26 ms a solve; FP32
+// at 128^2 BDM_3: 1.26 ms with 512, 1.21 with 1024). At 64 registers the four modes of BDM_3 spill 230
+// bytes, and the three of 3-D BDM_1, on seven blocks, 290: there the line could lie on either side (two
+// steps with 1024 and 512: 5.38 and 4.85 ms at 8^3, 12.3 and 11.4 at 16^3, 27.3 and 27.6 at 24^3).
 template <int NL, typename R>
 constexpr int ml_threads() {
   return NL == 6 || std::is_same<R, double>::value ? 512 : 1024;
