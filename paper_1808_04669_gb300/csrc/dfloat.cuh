@@ -24,15 +24,28 @@ struct dfl {
   __host__ __device__ __forceinline__ explicit operator double() const { return double(hi) + double(lo); }
 };
 
+// Each operation of the transformations is rounded by itself: a product that the compiler fuses with
+// the sum behind it is no longer the value whose error is taken, and the pair keeps FP32's bits only
+// (the general stage kernel at k = 3 lost its viscous terms' trailing words that way).
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ float rnd_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float rnd_sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float rnd_mul(float a, float b) { return __fmul_rn(a, b); }
+#else
+inline float rnd_add(float a, float b) { return a + b; }
+inline float rnd_sub(float a, float b) { return a - b; }
+inline float rnd_mul(float a, float b) { return a * b; }
+#endif
+
 __host__ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
+  s = rnd_add(a, b);
+  const float bb = rnd_sub(s, a);
+  e = rnd_add(rnd_sub(a, rnd_sub(s, bb)), rnd_sub(b, bb));
 }
 
 __host__ __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  e = b - (s - a);
+  s = rnd_add(a, b);
+  e = rnd_sub(b, rnd_sub(s, a));
 }
 
 __host__ __device__ __forceinline__ dfl operator+(dfl x, dfl y) {
@@ -48,7 +61,7 @@ __host__ __device__ __forceinline__ dfl operator-(dfl x) { return dfl(-x.hi, -x.
 __host__ __device__ __forceinline__ dfl operator-(dfl x, dfl y) { return x + (-y); }
 
 __host__ __device__ __forceinline__ dfl operator*(dfl x, dfl y) {
-  const float p = x.hi * y.hi;
+  const float p = rnd_mul(x.hi, y.hi);
   float e = fmaf(x.hi, y.hi, -p);
   e = fmaf(x.hi, y.lo, e);
   e = fmaf(x.lo, y.hi, e);
@@ -79,7 +92,7 @@ __host__ __device__ __forceinline__ dacc dacc_of(dfl x) { return dacc{x.hi, x.lo
 
 // a += x * y (the lo * lo product is below the double-float rounding and dropped)
 __host__ __device__ __forceinline__ void mad(dacc& a, dfl x, dfl y) {
-  const float p = x.hi * y.hi;
+  const float p = rnd_mul(x.hi, y.hi);
   float e = fmaf(x.hi, y.hi, -p);
   e = fmaf(x.hi, y.lo, e);
   e = fmaf(x.lo, y.hi, e);
@@ -91,7 +104,7 @@ __host__ __device__ __forceinline__ void mad(dacc& a, dfl x, dfl y) {
 
 // a += x * z for a double-float x and an FP32 z
 __host__ __device__ __forceinline__ void mad(dacc& a, dfl x, float z) {
-  const float p = x.hi * z;
+  const float p = rnd_mul(x.hi, z);
   float e = fmaf(x.hi, z, -p);
   e = fmaf(x.lo, z, e);
   float s, t;

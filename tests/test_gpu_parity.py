@@ -738,3 +738,20 @@ def test_uniform_state_has_no_viscous_terms(g, N, k, walls, precision):
     inviscid = mesh.eval_residual()
     mesh.set_viscosity(1e8)
     assert np.abs(mesh.eval_residual() - inviscid).max() <= 1e-12 * max(1.0, np.abs(inviscid).max())
+
+
+@pytest.mark.parametrize("N,k,perturb", [(1, 3, 0.0), (4, 1, 0.1), (5, 3, 0.1), (8, 2, 0.1), (10, 3, 0.1), (9, 3, 0.0)])
+@pytest.mark.parametrize("walls", [False, True])
+def test_mixed_viscous_residual_matches_the_oracle(g, N, k, walls, perturb):
+    # both stage kernels of the mixed form with their viscous sums (the general one on perturbed meshes),
+    # on random fields (no cancellation), with viscous terms as large as the convective ones: double-float
+    # sums keep some 44 bits, 1e-11 leaves them a few thousand roundings, an FP32 word shows at 1e-8
+    nu = 1e-2
+    vid, X = synth.split_square_mesh(N, L=1.0, periodic=not walls)
+    if perturb:
+        X = X + (perturb / N * np.random.default_rng(N).uniform(-1, 1, size=(vid.max() + 1, 2)))[vid]
+    mesh = g.DGMesh(vid, X, k, nu, precision=1)
+    d = Discretization(vid, X, k, nu)
+    v = random_lattice(mesh.n_tri, k, N)
+    mesh.set_velocity(v)
+    assert rel(mesh.eval_residual(), d.to_lattice(d.riesz(d.residual(d.from_lattice(v))))) < 1e-11
