@@ -49,8 +49,8 @@ namespace {
 constexpr int kMLThreads = 1024;         // most threads of a block
 // Threads of a block: 1024 (64 registers) in FP32; 512 (128 registers) in FP64 and for the six modes
 // of 3-D faces, whose rows of operands do not fit 64 (FP64, 48^2 BDM_2: 1.33 -> 1.26 ms a solve; FP32
-// at 128^2 BDM_3: 1.26 ms with 512, 1.21 with 1024). At 64 registers the four modes of BDM_3 spill 230
-// bytes, and the three of 3-D BDM_1, on seven blocks, 290: there the line could lie on either side (two
+// at 128^2 BDM_3: 1.26 ms with 512, 1.21 with 1024). At 64 registers the four modes of BDM_3 spill 250
+// bytes, and the three of 3-D BDM_1, on seven blocks, 310: there the line could lie on either side (two
 // steps with 1024 and 512: 5.38 and 4.85 ms at 8^3, 12.3 and 11.4 at 16^3, 27.3 and 27.6 at 24^3).
 template <int NL, typename R>
 constexpr int ml_threads() {
@@ -821,8 +821,8 @@ __global__ void __launch_bounds__((ml_threads<NL, R>()), 1) k_solve_ml(Mesh mesh
     // rounding that leaves a constant component in r would soon dominate z. So r is kept in the
     // range of S: the mode-0 mean that it had at the last V-cycle is subtracted in the next
     // update (S p has none but its rounding, some 1e-16 of r).
-    // r = (g - c0 1) - S lam, and its mode-0 sum
-    double r0s[1] = {0.0};
+    // r = (g - c0 1) - S lam, its mode-0 sum and square
+    double r0s[2] = {0.0, 0.0};
     const double c0 = sc.c0;
     ml_facets<NL>(c, [&](int f, int i, bool live) {
       double y[MP];
@@ -834,9 +834,24 @@ __global__ void __launch_bounds__((ml_threads<NL, R>()), 1) k_solve_ml(Mesh mesh
         const double r = (i + q == 0 ? m.g[o] - c0 : m.g[o]) - y[q];
         m.r[o] = r;
         if (i + q == 0) r0s[0] += r;
+        r0s[1] += r * r;
       }
     });
-    if (!ml_reduce<1>(m, bar, 0, r0s, scr, [&](const double (&t)[1]) { sc.mean = t[0] * inv_nf; })) return;
+    if (!ml_reduce<2>(m, bar, 0, r0s, scr, [&](const double (&t)[2]) {
+          sc.done = drop_start(a, nonneg(t[1] - t[0] * t[0] * inv_nf), gnorm);
+          sc.mean = sc.done ? 0.0 : t[0] * inv_nf;
+        }))
+      return;
+    if (sc.done)
+      ml_facets<NL>(c, [&](int f, int i, bool live) {
+        if (live)
+#pragma unroll
+          for (int q = 0; q < MP; ++q) {
+            const size_t o = size_t(f) * NL + i + q;
+            m.lam[o] = 0.0;
+            m.r[o] = i + q == 0 ? m.g[o] - c0 : m.g[o];
+          }
+      });
     // remove the constant component; first Chebyshev step of the V-cycle on r
     const double mean0 = sc.mean;
     ml_facets<NL>(c, [&](int f, int i, bool live) {

@@ -187,11 +187,23 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve(DevMesh m, SolveArgs a
           if (j == 0) rr[1] += r;
         }
       }
+      if (!grid_reduce<2>(m, 6, rr, bar)) return;
+      rr[0] = nonneg(rr[0] - rr[1] * rr[1] * inv_nf);
+      if (sweep == 0 && drop_start(a, rr[0], gnorm)) {
+        for (int f = gtid; f < nF; f += gsz)
+#pragma unroll
+          for (int j = 0; j < NL; ++j) {
+            const size_t o = size_t(f) * NL + j;
+            m.lam[o] = 0.0;
+            if (MIXED) m.rf[o] = float(m.g[o]);
+            else m.r[o] = m.g[o];
+          }
+        rr[0] = gnorm * gnorm;
+      }
       if (!MIXED) {
         // FP64 CG directly on S d = r with lam as the iterate (no refinement needed)
         bool c = false;
         double rr_end = 0.0;
-        if (!grid_sync(bar, m.stats)) return;
         iters = pcg<NL, double>(m, m.lam, m.r, m.z, m.pa, m.pb, m.q, m.st_blk, m.st_binv, stop, a.maxit, false, bar,
                                 &c, &rr_end);
         conv = c;
@@ -199,8 +211,6 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve(DevMesh m, SolveArgs a
         sweeps = 1;
         break;
       }
-      if (!grid_reduce<2>(m, 6, rr, bar)) return;
-      rr[0] = nonneg(rr[0] - rr[1] * rr[1] * inv_nf);
       const double prev = relres;
       relres = sqrt(rr[0]) / gnorm;
       if (!isfinite(rr[0])) {

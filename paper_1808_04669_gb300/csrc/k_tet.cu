@@ -497,6 +497,26 @@ __global__ void __launch_bounds__(kSolverThreads) k_solve3(DevMesh3 m, SolveArgs
       red[2] += r[0];
     }
     if (!reduce3<3>(m, bar, 1, red)) return;
+    if (drop_start(a, nonneg(red[1] - red[2] * red[2] * inv_nf), gnorm)) {
+      red[0] = red[1] = red[2] = 0.0;
+      for (int f = gtid; f < nF; f += gsz) {
+        double r[NL], z[NL];
+#pragma unroll
+        for (int j = 0; j < NL; ++j) r[j] = m.g[size_t(f) * NL + j] - (j == 0 ? c0 : 0.0);
+        binv3<NL>(m, f, r, z);
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+          m.lam[size_t(f) * NL + j] = 0.0;
+          m.r[size_t(f) * NL + j] = r[j];
+          m.z[size_t(f) * NL + j] = z[j];
+          red[0] += r[j] * z[j];
+          red[1] += r[j] * r[j];
+        }
+        red[2] += r[0];
+      }
+      // (other slots: blocks may still read the first sums)
+      if (!reduce3<3>(m, bar, 4, red)) return;
+    }
     double rho = red[0];
     rr = nonneg(red[1] - red[2] * red[2] * inv_nf);
     double beta = 0.0;

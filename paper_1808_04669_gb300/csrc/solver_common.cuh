@@ -74,6 +74,13 @@ __device__ bool grid_sync(Barrier& b, DevStats* st) {
 // that has broken down would count as converged).
 __device__ __forceinline__ double nonneg(double v) { return v < 0.0 ? 0.0 : v; }
 
+// Whether the start that left the squared residual rr is dropped for a zero one: it is farther off
+// (multipliers of another state, or not finite), and lam would keep the rounding of its larger
+// numbers, which the recursive residual does not show. (Of a zero start rr is gnorm^2 up to rounding.)
+__device__ __forceinline__ bool drop_start(const SolveArgs& a, double rr, double gnorm) {
+  return (a.hist1 || a.warm_scale != 0.0) && !(rr <= 1.0001 * gnorm * gnorm);
+}
+
 // Writes N block partials to red slots, synchronises the grid, and returns
 // the grid sums in every thread (same summation order in every block).
 template <int N>
