@@ -41,7 +41,7 @@ L2_FLUSH_BYTES = 512 << 20
 # over the three stages of a step (the first stage reads one state, the others two), from the
 # ncu capture summarised in profiles/; used only while the stage-kernel sources still hash to
 # the captured `sha`, else the line reports null.
-NCU_TRAFFIC = {"stage_residual": {"sha": "b82797c0b5404b51", "n_tri": 131072, "bytes": 40764757,
+NCU_TRAFFIC = {"stage_residual": {"sha": "4087f6ca148c8c3f", "n_tri": 131072, "bytes": 40748629,
                                   "source": "profiles/k_stage_df2_shear_n256_k3.md"}}
 
 
